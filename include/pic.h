@@ -12,7 +12,8 @@
  *
  * One step n -> n+1 of an instance runs, on the GPU, in this order:
  *   inject (surface sources)  -> cell sort (every sort_interval steps)
- *   -> cloud-in-cell deposit  -> Poisson solve (multigrid-preconditioned CG)
+ *   -> cloud-in-cell deposit  -> Poisson solve (refinement passes of a direct
+ *   solver; multigrid-preconditioned CG on grids too large for it)
  *   -> field gather + leapfrog push + absorption + MCC -> ionization resolve
  *   -> compaction.
  *
@@ -121,7 +122,8 @@ typedef struct {
   double rho_background;   /* uniform background charge density (C/m^3) */
   int32_t sort_interval;   /* cell sort every this many steps (0 = never) */
   double cg_rtol;          /* stop when ||r||_2 <= cg_rtol ||b||_2 */
-  int32_t cg_maxit;        /* iteration limit of the solve (PIC_ENOCONV beyond) */
+  int32_t cg_maxit;        /* iteration limit of the solve (PIC_ENOCONV beyond): passes
+                              of the direct solver, or CG iterations */
   int32_t precision;       /* PIC_FP64 | PIC_MIXED */
   uint64_t seed;           /* Philox4x32-10 key */
   int32_t nspecies;        /* 1..PIC_MAX_SPECIES */
@@ -143,7 +145,7 @@ typedef struct {
   double absorbed_energy_cathode_J[PIC_MAX_SPECIES]; /* cumulative, physical */
   double absorbed_energy_anode_J[PIC_MAX_SPECIES];
   int64_t ionizations, elastic, suppressed;       /* cumulative MCC events */
-  int32_t cg_iters;                               /* last solve */
+  int32_t cg_iters;                               /* last solve: passes, or CG iterations */
   double cg_resid_rel;                            /* last solve, true ||r||/||b|| */
   double total_charge_C;                          /* sum q w N over species */
   double kinetic_J[PIC_MAX_SPECIES];              /* sum (1/2) m w |v|^2 */

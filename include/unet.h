@@ -5,8 +5,8 @@
  * The solve of Eq. (1) in each PIC step starts from an initial guess; the
  * plain form starts from the previous step's potential. The learned form adds
  * a correction predicted by a small 3-D U-Net from the residual that the
- * previous potential leaves, and the multigrid-preconditioned CG then runs to
- * the configured tolerance exactly as before, so the field accuracy does not
+ * previous potential leaves, and the solve then runs to the configured
+ * tolerance exactly as before, so the field accuracy does not
  * depend on the network (it can only change the iteration count). The paper
  * has no network: it solves Eq. (1) by FEM; this is the scope's learned
  * variant of that solve.

@@ -1,0 +1,988 @@
+// k_direct.cu -- direct solve of A d = r for the scaled 7-point operator of
+// Eq. (1) on the node grid (periodic x, y; Dirichlet planes in z), in FP32.
+//
+// A is the sum of two periodic second differences and one Dirichlet one, so the
+// discrete Fourier modes of x and y decouple it into one tridiagonal system per
+// mode, (2 + lx + ly) u_k - u_(k-1) - u_(k+1) = f_k. Five launches:
+//   k_dir_xf  real FFT of every row (two rows packed as one complex line)
+//   k_dir_yf  complex FFT of every column of a plane
+//   k_dir_z   tridiagonal solve of every mode, the planes split over warps
+//   k_dir_yi, k_dir_xi  the inverse transforms; the last adds d to the potential
+// The solve is one pass of iterative refinement: the caller forms r = b - A x in
+// float-float (mixed) or FP64, and repeats until the residual meets its tolerance.
+// FP32 rounding leaves 1e-6 to 1e-3 of the residual per pass (the most for modes
+// that are smooth in all three directions), so a warm-started mixed solve to 1e-8
+// takes one pass and an FP64 one to 1e-13 two or three.
+//
+// What bounds the kernels: every pass over a vector of the unknowns is one read
+// and one write of L2 (up to 128x128x256) or HBM; the butterflies are far below
+// the FP32 rate. A block holds 16 lines of an axis with the line index innermost
+// in shared memory, so every butterfly access of a half warp is one contiguous
+// 128-byte row whatever the radix (rows of 17 float2 in x, where the loads
+// transpose). Spectra stay in the order the passes leave them in (digit
+// reversed): the tridiagonal kernel only needs each column's eigenvalue.
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "dev_mem.cuh"
+#include "pic_direct.cuh"
+#include "pic_internal.cuh"
+#include "pic_solver.cuh"
+#include "solver_dev.cuh"
+
+namespace pic {
+
+namespace {
+
+constexpr int kFftThreads = 128;
+constexpr int kLpX = kDirLines + 1;  // row pitch (float2) of the x tiles
+constexpr int kLpY = kDirLines;
+
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// a w (forward) or a conj(w) (inverse)
+template <bool INV>
+__device__ __forceinline__ float2 ctw(float2 a, float2 w) {
+  return INV ? make_float2(fmaf(a.x, w.x, a.y * w.y), fmaf(a.y, w.x, -a.x * w.y))
+             : make_float2(fmaf(a.x, w.x, -a.y * w.y), fmaf(a.y, w.x, a.x * w.y));
+}
+// -i a (forward) or i a (inverse)
+template <bool INV>
+__device__ __forceinline__ float2 crot(float2 a) {
+  return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+}
+
+// cos(2 pi m / 16), m = 0..4
+__device__ __forceinline__ constexpr float cos16(int m) {
+  return m == 0 ? 1.f : (m == 1 ? 0.923879532511286756f : (m == 2 ? 0.707106781186547524f : (m == 3 ? 0.382683432365089772f : 0.f)));
+}
+
+// Power-of-two DFT, natural order in and out: halves of even and odd index.
+template <int R, bool INV>
+struct Dft {
+  static __device__ __forceinline__ void run(float2 (&v)[R]) {
+    float2 e[R / 2], o[R / 2];
+#pragma unroll
+    for (int k = 0; k < R / 2; ++k) {
+      e[k] = v[2 * k];
+      o[k] = v[2 * k + 1];
+    }
+    Dft<R / 2, INV>::run(e);
+    Dft<R / 2, INV>::run(o);
+#pragma unroll
+    for (int k = 0; k < R / 2; ++k) {
+      const int m = k * (16 / R);  // exp(-2 pi i m / 16), m < 8
+      float2 t = o[k];
+      if (m == 4) t = crot<INV>(t);
+      else if (m > 0) {
+        const float c = m < 4 ? cos16(m) : -cos16(8 - m), s = m < 4 ? cos16(4 - m) : cos16(m - 4);
+        t = ctw<INV>(t, make_float2(c, -s));
+      }
+      v[k] = cadd(e[k], t);
+      v[k + R / 2] = csub(e[k], t);
+    }
+  }
+};
+template <bool INV>
+struct Dft<1, INV> {
+  static __device__ __forceinline__ void run(float2 (&)[1]) {}
+};
+
+// DFT of an odd prime length: x_s +- x_(R-s) pair up, so each output pair (k, R - k) takes
+// (R - 1) / 2 real products of each kind. w[m] = exp(-2 pi i m / R).
+template <int R, bool INV>
+__device__ __forceinline__ void dft_odd(float2 (&v)[R], const float2* w, int step) {
+  constexpr int H = (R - 1) / 2;
+  float2 a[H], b[H];
+  float c[H], s[H];
+  float2 y0 = v[0];
+#pragma unroll
+  for (int q = 0; q < H; ++q) {
+    a[q] = cadd(v[q + 1], v[R - 1 - q]);
+    b[q] = csub(v[q + 1], v[R - 1 - q]);
+    const float2 t = w[(q + 1) * step];
+    c[q] = t.x;
+    s[q] = -t.y;
+    y0 = cadd(y0, a[q]);
+  }
+  const float2 x0 = v[0];
+  v[0] = y0;
+#pragma unroll
+  for (int k = 1; k <= H; ++k) {
+    float2 re = x0, im = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int q = 0; q < H; ++q) {
+      const int m = (k * (q + 1)) % R;  // 1..R - 1, R being prime
+      const float cm = m <= H ? c[m - 1] : c[R - m - 1];
+      const float sm = m <= H ? s[m - 1] : -s[R - m - 1];
+      re = make_float2(fmaf(cm, a[q].x, re.x), fmaf(cm, a[q].y, re.y));
+      im = make_float2(fmaf(sm, b[q].x, im.x), fmaf(sm, b[q].y, im.y));
+    }
+    const float2 t = crot<INV>(im);
+    v[k] = cadd(re, t);
+    v[R - k] = csub(re, t);
+  }
+}
+
+// One pass over the tile: butterflies of radix R on blocks of L points.
+template <int R, bool INV, int LP>
+__device__ __forceinline__ void fft_pass(float2* Z, const float2* tw, int n, int L, const FastDiv& dM) {
+  const int M = dM.d, nb = n / R, step = n / L, st = M * LP;
+  for (int t = threadIdx.x; t < nb * kDirLines; t += kFftThreads) {
+    const int l = t & (kDirLines - 1), b = t / kDirLines;
+    const int s = fdiv(b, dM), j = b - s * M;
+    float2* z = Z + (s * L + j) * LP + l;
+    const int jw = j * step;
+    float2 v[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      v[q] = z[q * st];
+      if (INV && q > 0) v[q] = ctw<true>(v[q], tw[q * jw]);
+    }
+    if constexpr ((R & (R - 1)) == 0) Dft<R, INV>::run(v);
+    else dft_odd<R, INV>(v, tw, n / R);
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      if (!INV && q > 0) v[q] = ctw<false>(v[q], tw[q * jw]);
+      z[q * st] = v[q];
+    }
+  }
+}
+
+// A radix without an unrolled butterfly (a prime above 13): one output per
+// thread and turn, from Z to Z2.
+template <bool INV, int LP>
+__device__ void fft_pass_any(const float2* Z, float2* Z2, const float2* tw, int n, int R, int L, const FastDiv& dM) {
+  const int M = dM.d, step = n / L, root = n / R;
+  for (int t = threadIdx.x; t < n * kDirLines; t += kFftThreads) {
+    const int l = t & (kDirLines - 1), e = t / kDirLines;
+    const int qs = fdiv(e, dM), j = e - qs * M;  // e = (s R + q) M + j
+    const int s = qs / R, q = qs - s * R;
+    const float2* z = Z + (s * L + j) * LP + l;
+    float2 acc = z[0];
+    int idx = 0;
+    for (int p = 1; p < R; ++p) {
+      idx += q;
+      if (idx >= R) idx -= R;
+      float2 x = z[p * M * LP];
+      if (INV) x = ctw<true>(x, tw[p * j * step]);
+      const float2 y = ctw<INV>(x, tw[idx * root]);
+      acc = cadd(acc, y);
+    }
+    if (!INV) acc = ctw<false>(acc, tw[q * j * step]);
+    Z2[e * LP + l] = acc;
+  }
+}
+
+// All passes of an axis on the tile in Z (forward: natural in, digit reversed
+// out; inverse: the reverse). Returns the buffer that holds the result.
+template <bool INV, int LP, bool POW2>
+__device__ __forceinline__ float2* fft_tile(float2* Z, float2* Z2, const float2* tw, const AxisPlan& A) {
+  for (int p = 0; p < A.npass; ++p) {
+    const int q = INV ? A.npass - 1 - p : p;
+    const int R = A.R[q], L = A.L[q];
+    const FastDiv dM = A.dM[q];
+    switch (R) {
+      case 2: fft_pass<2, INV, LP>(Z, tw, A.n, L, dM); break;
+      case 4: fft_pass<4, INV, LP>(Z, tw, A.n, L, dM); break;
+      case 8: fft_pass<8, INV, LP>(Z, tw, A.n, L, dM); break;
+      case 16: fft_pass<16, INV, LP>(Z, tw, A.n, L, dM); break;
+      default:
+        if constexpr (!POW2) {
+          switch (R) {
+            case 3: fft_pass<3, INV, LP>(Z, tw, A.n, L, dM); break;
+            case 5: fft_pass<5, INV, LP>(Z, tw, A.n, L, dM); break;
+            case 7: fft_pass<7, INV, LP>(Z, tw, A.n, L, dM); break;
+            case 11: fft_pass<11, INV, LP>(Z, tw, A.n, L, dM); break;
+            case 13: fft_pass<13, INV, LP>(Z, tw, A.n, L, dM); break;
+            default: {
+              fft_pass_any<INV, LP>(Z, Z2, tw, A.n, R, L, dM);
+              float2* t = Z;
+              Z = Z2;
+              Z2 = t;
+            }
+          }
+        }
+    }
+    __syncthreads();
+  }
+  return Z;
+}
+
+__device__ __forceinline__ void load_tw(float2* tw, const AxisPlan& A) {
+  for (int m = threadIdx.x; m < A.n; m += kFftThreads) tw[m] = __ldg(A.tw + m);
+}
+
+// Rows 2q and 2q + 1 as real and imaginary part; scale applied in FP64 to FP64 input.
+template <class T>
+__device__ __forceinline__ float scaled(T v, double scale) {
+  if constexpr (sizeof(T) == 8) return (float)(v * scale);
+  else return v;
+}
+
+template <class T, bool POW2>
+__global__ void __launch_bounds__(kFftThreads) k_dir_xf(DirectArgs a, const T* __restrict__ in, const SolveCtl* c) {
+  pdl_enter();
+  if (c->stopped) return;
+  extern __shared__ __align__(16) float2 sm[];
+  const int n = a.nx;
+  float2* tw = sm;
+  float2* Z = sm + n;
+  load_tw(tw, a.x);
+  const long long row0 = 2ll * kDirLines * blockIdx.x;
+  const double scale = sizeof(T) == 8 ? c->scale : 1.0;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int l = w; l < kDirLines; l += kFftThreads / 32) {
+    const long long r = row0 + 2 * l;
+    const T* pa = in + r * n;
+    const bool va = r < a.rows, vb = r + 1 < a.rows;
+#pragma unroll 4
+    for (int i = lane; i < n; i += 32)
+      Z[i * kLpX + l] = make_float2(va ? scaled(pa[i], scale) : 0.f, vb ? scaled(pa[n + i], scale) : 0.f);
+  }
+  __syncthreads();
+  Z = fft_tile<false, kLpX, POW2>(Z, Z + n * kLpX, tw, a.x);
+  // the two rows' spectra from their packed line: A = (Z_f + conj Z_-f) / 2, B = (Z_f - conj Z_-f) / 2i
+  float2* out = reinterpret_cast<float2*>(a.spec);
+  for (int l = w; l < kDirLines; l += kFftThreads / 32) {
+    const long long r = row0 + 2 * l;
+    if (r >= a.rows) break;
+    const bool vb = r + 1 < a.rows;
+    for (int f = lane; f < a.C; f += 32) {
+      float2 A, B;
+      if (f == 0) {
+        const float2 z0 = Z[l];
+        const float2 zh = a.packed ? Z[__ldg(a.x.pos + n / 2) * kLpX + l] : make_float2(0.f, 0.f);
+        A = make_float2(z0.x, zh.x);
+        B = make_float2(z0.y, zh.y);
+      } else {
+        const float2 p = Z[__ldg(a.x.pos + f) * kLpX + l], m = Z[__ldg(a.x.pos + n - f) * kLpX + l];
+        A = make_float2(0.5f * (p.x + m.x), 0.5f * (p.y - m.y));
+        B = make_float2(0.5f * (p.y + m.y), 0.5f * (m.x - p.x));
+      }
+      out[r * a.C + f] = A;
+      if (vb) out[(r + 1) * a.C + f] = B;
+    }
+  }
+}
+
+// Column 0 of an even nx carries the mean and the Nyquist coefficient of every
+// row as one complex number: after (before) the y transform its frequencies g
+// and -g are combined into the two coefficients' own spectra (and back).
+template <bool INV>
+__device__ __forceinline__ void split_packed(float2* Z, const AxisPlan& A) {
+  for (int g = 1 + threadIdx.x; 2 * g < A.n; g += kFftThreads) {
+    float2 &p = Z[__ldg(A.pos + g) * kLpY], &m = Z[__ldg(A.pos + A.n - g) * kLpY];
+    const float2 u = p, v = m;
+    if (!INV) {
+      p = make_float2(0.5f * (u.x + v.x), 0.5f * (u.y - v.y));
+      m = make_float2(0.5f * (u.y + v.y), 0.5f * (v.x - u.x));
+    } else {  // p = u + i v, m = conj(u) + i conj(v)
+      p = make_float2(u.x - v.y, u.y + v.x);
+      m = make_float2(u.x + v.y, v.x - u.y);
+    }
+  }
+}
+
+template <bool INV, bool POW2>
+__global__ void __launch_bounds__(kFftThreads) k_dir_y(DirectArgs a, const SolveCtl* c) {
+  pdl_enter();
+  if (c->stopped) return;
+  extern __shared__ __align__(16) float2 sm[];
+  const int n = a.ny;
+  float2* tw = sm;
+  float2* Z = sm + n;
+  load_tw(tw, a.y);
+  const int col0 = blockIdx.x * kDirLines, l = threadIdx.x & (kDirLines - 1);
+  const bool in = col0 + l < a.C;
+  float2* g = reinterpret_cast<float2*>(a.spec) + (long long)blockIdx.y * n * a.C + col0 + l;
+#pragma unroll 8
+  for (int y = threadIdx.x / kDirLines; y < n; y += kFftThreads / kDirLines)
+    Z[y * kLpY + l] = in ? g[(long long)y * a.C] : make_float2(0.f, 0.f);
+  __syncthreads();
+  const bool split = a.packed && col0 == 0;
+  if (INV && split) {
+    split_packed<true>(Z, a.y);
+    __syncthreads();
+  }
+  Z = fft_tile<INV, kLpY, POW2>(Z, Z + n * kLpY, tw, a.y);
+  if (!INV && split) {
+    split_packed<false>(Z, a.y);
+    __syncthreads();
+  }
+  if (!in) return;
+#pragma unroll 8
+  for (int y = threadIdx.x / kDirLines; y < n; y += kFftThreads / kDirLines) g[(long long)y * a.C] = Z[y * kLpY + l];
+}
+
+// What the last inverse transform does with d (already normalised): mixed,
+// (hi, lo) += d renormalised; FP64, x += d / scale.
+struct AddMixed {
+  float *hi, *lo;
+  double phi_c, dphi_dk;
+  __device__ __forceinline__ void add(long long u, float d, double) const {
+    float s, e;
+    two_sum(hi[u], d, s, e);
+    e = __fadd_rn(e, lo[u]);
+    const float h2 = __fadd_rn(s, e);
+    hi[u] = h2;
+    lo[u] = __fsub_rn(e, __fsub_rn(h2, s));
+  }
+  __device__ __forceinline__ void zero(long long u, int k) const {  // phi = 0: hi + lo = -vac
+    const double v = -(phi_c + dphi_dk * (double)(k + 1));
+    const float vh = (float)v;
+    hi[u] = vh;
+    lo[u] = (float)(v - (double)vh);
+  }
+};
+struct Add64 {
+  double* x;
+  __device__ __forceinline__ void add(long long u, float d, double inv_scale) const { x[u] += (double)d * inv_scale; }
+  __device__ __forceinline__ void zero(long long u, int) const { x[u] = 0.0; }
+};
+
+template <class Add, bool POW2>
+__global__ void __launch_bounds__(kFftThreads) k_dir_xi(DirectArgs a, Add add, const SolveCtl* c) {
+  pdl_enter();
+  const long long row0 = 2ll * kDirLines * blockIdx.x;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int n = a.nx;
+  if (c->stopped) {
+    if (c->bb != 0.0) return;
+    for (long long r = row0 + w; r < row0 + 2 * kDirLines && r < a.rows; r += kFftThreads / 32)  // b = 0: x = 0
+      for (int i = lane; i < n; i += 32) add.zero(r * n + i, (int)(r / a.ny));
+    return;
+  }
+  extern __shared__ __align__(16) float2 sm[];
+  float2* tw = sm;
+  float2* Z = sm + n;
+  load_tw(tw, a.x);
+  const float2* spec = reinterpret_cast<const float2*>(a.spec);
+  for (int l = w; l < kDirLines; l += kFftThreads / 32) {
+    const long long r = row0 + 2 * l;
+    const bool va = r < a.rows, vb = r + 1 < a.rows;
+#pragma unroll 2
+    for (int f = lane; f < a.C; f += 32) {
+      const float2 A = va ? spec[r * a.C + f] : make_float2(0.f, 0.f);
+      const float2 B = vb ? spec[(r + 1) * a.C + f] : make_float2(0.f, 0.f);
+      if (f == 0) {
+        Z[l] = make_float2(A.x, B.x);
+        if (a.packed) Z[__ldg(a.x.pos + n / 2) * kLpX + l] = make_float2(A.y, B.y);
+      } else {  // Z_f = A + i B, Z_-f = conj A + i conj B
+        Z[__ldg(a.x.pos + f) * kLpX + l] = make_float2(A.x - B.y, A.y + B.x);
+        Z[__ldg(a.x.pos + n - f) * kLpX + l] = make_float2(A.x + B.y, B.x - A.y);
+      }
+    }
+  }
+  __syncthreads();
+  Z = fft_tile<true, kLpX, POW2>(Z, Z + n * kLpX, tw, a.x);
+  const double inv_scale = c->inv_scale;
+  for (int l = w; l < kDirLines; l += kFftThreads / 32) {
+    const long long r = row0 + 2 * l;
+    const bool va = r < a.rows, vb = r + 1 < a.rows;
+#pragma unroll 4
+    for (int i = lane; i < n; i += 32) {
+      const float2 d = Z[i * kLpX + l];
+      if (va) add.add(r * n + i, d.x * a.norm, inv_scale);
+      if (vb) add.add((r + 1) * n + i, d.y * a.norm, inv_scale);
+    }
+  }
+}
+
+// Tridiagonal systems (2 + lambda) u_k - u_(k-1) - u_(k+1) = f_k, zero beyond
+// both ends, one per float column of the spectrum (lane = column). Warp w of the
+// block takes planes [w M, (w + 1) M): it eliminates its chunk with zero outer
+// neighbours (pivots 1 / (2 + lambda - pivot), the same for every chunk, formed
+// as 1 / (1 + s), s = lambda + s pivot, which does not cancel for small lambda);
+// the chunks' first and last values then satisfy a recurrence that warp 0 solves
+// along the chunks, and each warp adds the response to its two outer neighbours.
+// Planes stay in registers in between, so the spectrum is read and written once.
+template <int M, int THREADS>
+__global__ void __launch_bounds__(THREADS) k_dir_z(DirectArgs a, const SolveCtl* c) {
+  pdl_enter();
+  if (c->stopped) return;
+  extern __shared__ float zs[];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+  float* sF = zs + lane;         // [W][32] first value of the chunk
+  float* sE = sF + 32 * W;       // last value with zero neighbours, then the left neighbour's value
+  float* sD = sE + 32 * W;       // response of the first value to the right neighbour
+  float* sV = sD + 32 * W;
+  const int col = blockIdx.x * 32 + lane;
+  const bool in = col < a.plane;
+  const int k0 = w * M, len = min(M, a.P - k0);
+  float* g = a.spec + (long long)k0 * a.plane + col;
+  float y[M], cp[M];
+#pragma unroll
+  for (int k = 0; k < M; ++k) y[k] = in && k < len ? g[(long long)k * a.plane] : 0.f;
+  const float lam = in ? __ldg(a.lam + col) : 1.f;
+  float s = lam + 1.f, b = 1.f;
+#pragma unroll
+  for (int k = 0; k < M; ++k) {
+    cp[k] = 1.f / (1.f + s);
+    s = fmaf(s, cp[k], lam);
+    b *= cp[k];
+  }
+  float t = 0.f;
+#pragma unroll
+  for (int k = 0; k < M; ++k) {
+    t = cp[k] * (y[k] + t);
+    y[k] = k < len ? t : 0.f;
+  }
+  sE[32 * w] = y[M - 1];
+  t = 0.f;
+#pragma unroll
+  for (int k = M - 1; k >= 0; --k) t = fmaf(cp[k], t, y[k]);
+  sF[32 * w] = t;
+  __syncthreads();
+  if (w == 0) {
+    // F = pF + a L + b R, E = pE + b L + a R per chunk (a, b: responses at the near
+    // and the far end), L the left chunk's E, R the right chunk's F. With
+    // L = u + v F: F = (pF + a u + b R) / (1 - a v), and u, v of the next chunk.
+    const int last = a.P - (W - 1) * M;  // planes of the last chunk
+    float alast = cp[0];
+#pragma unroll
+    for (int k = 1; k < M; ++k) alast = k < last ? cp[k] : alast;
+    float u = 0.f, v = 0.f;
+    for (int q = 0; q < W; ++q) {
+      const float aq = q == W - 1 ? alast : cp[M - 1], bq = q == W - 1 ? 0.f : b;
+      const float inv = 1.f / fmaf(-aq, v, 1.f);
+      const float F = fmaf(aq, u, sF[32 * q]) * inv, D = bq * inv, pE = sE[32 * q];
+      sF[32 * q] = F;
+      sD[32 * q] = D;
+      sE[32 * q] = u;
+      sV[32 * q] = v;
+      u = fmaf(bq, fmaf(v, F, u), pE);
+      v = fmaf(bq * v, D, aq);
+    }
+    float R = 0.f;
+    for (int q = W - 1; q >= 0; --q) {
+      R = fmaf(sD[32 * q], R, sF[32 * q]);
+      sF[32 * q] = R;
+      sE[32 * q] = fmaf(sV[32 * q], R, sE[32 * q]);
+    }
+  }
+  __syncthreads();
+  t = sE[32 * w];  // the left neighbour's value (0 for the first chunk)
+  const float right = w + 1 < W ? sF[32 * (w + 1)] : 0.f;
+#pragma unroll
+  for (int k = 0; k < M; ++k) {
+    t *= cp[k];
+    y[k] += t;
+  }
+  y[M - 1] = fmaf(cp[M - 1], right, y[M - 1]);
+  t = 0.f;
+#pragma unroll
+  for (int k = M - 1; k >= 0; --k) {
+    t = k < len ? fmaf(cp[k], t, y[k]) : 0.f;
+    if (in && k < len) g[(long long)k * a.plane] = t;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// residuals of the refinement
+// ---------------------------------------------------------------------------
+// Two grid-wide sums at once (as grid_total; partials interleaved).
+template <class V>
+__device__ __forceinline__ bool grid_total2(V v0, V v1, double* part, unsigned* ticket, double* t0, double* t1) {
+  __shared__ double sm0[32], sm1[32];
+  __shared__ int s_last;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const int nthr = blockDim.x * blockDim.y, nw = nthr >> 5;
+  const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
+  v0 = warp_sum(v0);
+  v1 = warp_sum(v1);
+  if ((tid & 31) == 0) {
+    sm0[tid >> 5] = (double)v0;
+    sm1[tid >> 5] = (double)v1;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    double a = 0.0, b = 0.0;
+    for (int k = 0; k < nw; ++k) {
+      a += sm0[k];
+      b += sm1[k];
+    }
+    const unsigned at = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    reinterpret_cast<double2*>(part)[at] = make_double2(a, b);
+    __threadfence();
+    s_last = atomicAdd(ticket, 1u) == nb - 1u ? 1 : 0;
+  }
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  double a = 0.0, b = 0.0;
+#pragma unroll 4
+  for (unsigned i = tid; i < nb; i += nthr) {
+    const double2 p = __ldcg(reinterpret_cast<const double2*>(part) + i);
+    a += p.x;
+    b += p.y;
+  }
+  a = warp_sum(a);
+  b = warp_sum(b);
+  __syncthreads();
+  if ((tid & 31) == 0) {
+    sm0[tid >> 5] = a;
+    sm1[tid >> 5] = b;
+  }
+  __syncthreads();
+  if (tid != 0) return false;
+  a = b = 0.0;
+  for (int k = 0; k < nw; ++k) {
+    a += sm0[k];
+    b += sm1[k];
+  }
+  *t0 = a;
+  *t1 = b;
+  *ticket = 0u;
+  return true;
+}
+
+// The refinement's decision from r.r: another pass or stop; the power of two
+// that brings r to unit size for the FP32 pass of an FP64 residual.
+__device__ __forceinline__ void fin_pass(const DirectLoop& d, SolveCtl* c, double rr, long long n) {
+  c->rr_true = rr;
+  c->resid_rel = c->bb > 0.0 ? sqrt(rr / c->bb) : 0.0;
+  const bool small = c->bb == 0.0 || rr <= c->tol2;
+  const bool done = small || !(rr == rr) || c->it_total >= d.maxit || c->outer >= d.max_outer;
+  c->converged = small ? 1 : 0;
+  c->more = done ? 0 : 1;
+  c->stopped = done ? 1 : 0;
+  const double rms = sqrt(rr / (double)n);
+  const int ex = rms > 0.0 && rms < 1e300 ? max(-900, min(900, -ilogb(rms))) : 0;
+  c->scale = scalbn(1.0, ex);
+  c->inv_scale = scalbn(1.0, -ex);
+  if (d.use_graph) cudaGraphSetConditional(d.handle, done ? 0u : 1u);
+}
+// first: the solve begins (b.b sets the tolerance); later: one pass has run
+__device__ __forceinline__ void fin_first(const DirectLoop& d, SolveCtl* c, double rr, double bb, long long n) {
+  c->bb = bb;
+  c->tol2 = d.rtol * d.rtol * bb;
+  c->maxit = d.maxit;
+  c->it_total = 0;
+  c->outer = 0;
+  fin_pass(d, c, rr, n);
+}
+__device__ __forceinline__ void fin_next(const DirectLoop& d, SolveCtl* c, double rr, long long n) {
+  c->it_total += 1;
+  c->outer += 1;
+  fin_pass(d, c, rr, n);
+}
+
+template <class T, int V>
+struct VecOf;
+template <>
+struct VecOf<float, 1> {
+  using type = float;
+};
+template <>
+struct VecOf<float, 4> {
+  using type = float4;
+};
+template <>
+struct VecOf<double, 1> {
+  using type = double;
+};
+template <>
+struct VecOf<double, 2> {
+  using type = double2;
+};
+template <int V, class T>
+__device__ __forceinline__ void vload(T (&v)[V], const T* p) {
+  using U = typename VecOf<T, V>::type;
+  const U u = *reinterpret_cast<const U*>(p);
+#pragma unroll
+  for (int e = 0; e < V; ++e) v[e] = reinterpret_cast<const T*>(&u)[e];
+}
+template <int V, class T>
+__device__ __forceinline__ void vstore(T* p, const T (&v)[V]) {
+  using U = typename VecOf<T, V>::type;
+  U u;
+#pragma unroll
+  for (int e = 0; e < V; ++e) reinterpret_cast<T*>(&u)[e] = v[e];
+  *reinterpret_cast<U*>(p) = u;
+}
+
+// The residual kernels give a thread V neighbouring points of a row and march it
+// through kc planes: a plane is loaded once as the upper neighbour and kept in
+// registers as the centre and the lower one, so a point costs one load of its
+// own plane instead of three.
+constexpr int kResX = 32, kResY = 8;
+struct ResGeom {
+  Lv L;
+  int kc;         // planes per block
+  long long n;    // unknowns
+};
+
+// r = fl32(f - A (hi + lo)) in float-float (the transformations of the header
+// comment of the MIXED solver), r.r and, FIRST, b.b with the folded electrode
+// terms. V = 4 where rows are whole float4s.
+template <int V, bool FIRST>
+__global__ void __launch_bounds__(kResX* kResY) k_dir_resid_ff(ResGeom G, const float* __restrict__ hi,
+                                                              const float* __restrict__ lo, const float* __restrict__ f,
+                                                              float* __restrict__ r, float fold_first, float fold_last,
+                                                              double* part, SolveCtl* c, DirectLoop d) {
+  pdl_enter();
+  if (!FIRST && c->stopped) return;
+  const Lv& L = G.L;
+  const int i = (blockIdx.x * kResX + threadIdx.x) * V, j = blockIdx.y * kResY + threadIdx.y;
+  const int k0 = blockIdx.z * G.kc, kend = min(k0 + G.kc, L.nz - 1);
+  float rr = 0.f, bb = 0.f;
+  if (i < L.nx && j < L.ny) {
+    const int row = j * L.nx;
+    const int left = row + (i == 0 ? L.nx - 1 : i - 1), right = row + (i + V == L.nx ? 0 : i + V);
+    const int down = (j == 0 ? L.ny - 1 : j - 1) * L.nx + i, up = (j == L.ny - 1 ? 0 : j + 1) * L.nx + i;
+    const long long at0 = (long long)k0 * L.pl;
+    float hm[V] = {}, hc[V], hp[V], lm[V] = {}, lc[V], lp[V];
+    vload<V>(hc, hi + at0 + row + i);
+    vload<V>(lc, lo + at0 + row + i);
+    if (k0 > 0) {
+      vload<V>(hm, hi + at0 - L.pl + row + i);
+      vload<V>(lm, lo + at0 - L.pl + row + i);
+    }
+    for (int k = k0; k < kend; ++k) {
+      const float *H = hi + (long long)k * L.pl, *O = lo + (long long)k * L.pl;
+      float hy0[V], hy1[V], ly0[V], ly1[V], fv[V], rv[V];
+      if (k < L.nz - 2) {
+        vload<V>(hp, H + L.pl + row + i);
+        vload<V>(lp, O + L.pl + row + i);
+      } else {
+#pragma unroll
+        for (int e = 0; e < V; ++e) hp[e] = lp[e] = 0.f;
+      }
+      vload<V>(hy0, H + down);
+      vload<V>(hy1, H + up);
+      vload<V>(ly0, O + down);
+      vload<V>(ly1, O + up);
+      vload<V>(fv, f + (long long)k * L.pl + row + i);
+      const float hl = H[left], hr = H[right], ol = O[left], orr = O[right];
+#pragma unroll
+      for (int e = 0; e < V; ++e) {
+        const float xl = e == 0 ? hl : hc[e > 0 ? e - 1 : 0], xr = e == V - 1 ? hr : hc[e < V - 1 ? e + 1 : 0];
+        float s = xl, er = 0.f, t;
+        two_sum(s, xr, s, t);
+        er = __fadd_rn(er, t);
+        two_sum(s, hy0[e], s, t);
+        er = __fadd_rn(er, t);
+        two_sum(s, hy1[e], s, t);
+        er = __fadd_rn(er, t);
+        two_sum(s, hm[e], s, t);
+        er = __fadd_rn(er, t);
+        two_sum(s, hp[e], s, t);
+        er = __fadd_rn(er, t);
+        const float p6 = __fmul_rn(6.f, hc[e]), e6 = __fmaf_rn(6.f, hc[e], -p6);
+        float a1, ea, r1, e1;
+        two_sum(p6, -s, a1, ea);
+        const float zl = e == 0 ? ol : lc[e > 0 ? e - 1 : 0], zr = e == V - 1 ? orr : lc[e < V - 1 ? e + 1 : 0];
+        const float nl = ((((zl + zr) + ly0[e]) + ly1[e]) + lm[e]) + lp[e];
+        const float alo = __fsub_rn(__fmul_rn(6.f, lc[e]), nl);
+        two_sum(fv[e], -a1, r1, e1);
+        rv[e] = __fadd_rn(r1, __fsub_rn(__fadd_rn(__fsub_rn(__fsub_rn(e1, ea), e6), er), alo));
+        rr += rv[e] * rv[e];
+        if (FIRST) {
+          float bv = fv[e];
+          if (k == 0) bv += fold_first;
+          if (k == L.nz - 2) bv += fold_last;
+          bb += bv * bv;
+        }
+      }
+      vstore<V>(r + (long long)k * L.pl + row + i, rv);
+#pragma unroll
+      for (int e = 0; e < V; ++e) {
+        hm[e] = hc[e];
+        hc[e] = hp[e];
+        lm[e] = lc[e];
+        lc[e] = lp[e];
+      }
+    }
+  }
+  double t0, t1;
+  if constexpr (FIRST) {
+    if (grid_total2(rr, bb, part, &c->ticket, &t0, &t1)) fin_first(d, c, t0, t1, G.n);
+  } else {
+    if (grid_total(rr, part, &c->ticket, &t0)) fin_next(d, c, t0, G.n);
+  }
+}
+
+// r = b - A x in FP64, r.r and, FIRST, b.b
+template <int V, bool FIRST>
+__global__ void __launch_bounds__(kResX* kResY) k_dir_resid64(ResGeom G, const double* __restrict__ x,
+                                                             const double* __restrict__ b, double* __restrict__ r,
+                                                             double* part, SolveCtl* c, DirectLoop d) {
+  pdl_enter();
+  if (!FIRST && c->stopped) return;
+  const Lv& L = G.L;
+  const int i = (blockIdx.x * kResX + threadIdx.x) * V, j = blockIdx.y * kResY + threadIdx.y;
+  const int k0 = blockIdx.z * G.kc, kend = min(k0 + G.kc, L.nz - 1);
+  double rr = 0.0, bb = 0.0;
+  if (i < L.nx && j < L.ny) {
+    const int row = j * L.nx;
+    const int left = row + (i == 0 ? L.nx - 1 : i - 1), right = row + (i + V == L.nx ? 0 : i + V);
+    const int down = (j == 0 ? L.ny - 1 : j - 1) * L.nx + i, up = (j == L.ny - 1 ? 0 : j + 1) * L.nx + i;
+    double xm[V] = {}, xc[V], xp[V];
+    vload<V>(xc, x + (long long)k0 * L.pl + row + i);
+    if (k0 > 0) vload<V>(xm, x + (long long)(k0 - 1) * L.pl + row + i);
+    for (int k = k0; k < kend; ++k) {
+      const double* X = x + (long long)k * L.pl;
+      double y0[V], y1[V], bv[V], rv[V];
+      if (k < L.nz - 2) {
+        vload<V>(xp, X + L.pl + row + i);
+      } else {
+#pragma unroll
+        for (int e = 0; e < V; ++e) xp[e] = 0.0;
+      }
+      vload<V>(y0, X + down);
+      vload<V>(y1, X + up);
+      vload<V>(bv, b + (long long)k * L.pl + row + i);
+      const double xl0 = X[left], xr0 = X[right];
+#pragma unroll
+      for (int e = 0; e < V; ++e) {
+        const double xl = e == 0 ? xl0 : xc[e > 0 ? e - 1 : 0], xr = e == V - 1 ? xr0 : xc[e < V - 1 ? e + 1 : 0];
+        const double s = ((((xl + xr) + y0[e]) + y1[e]) + xm[e]) + xp[e];
+        rv[e] = bv[e] - (6.0 * xc[e] - s);
+        rr += rv[e] * rv[e];
+        if (FIRST) bb += bv[e] * bv[e];
+        xm[e] = xc[e];
+      }
+#pragma unroll
+      for (int e = 0; e < V; ++e) xc[e] = xp[e];
+      vstore<V>(r + (long long)k * L.pl + row + i, rv);
+    }
+  }
+  double t0, t1;
+  if constexpr (FIRST) {
+    if (grid_total2(rr, bb, part, &c->ticket, &t0, &t1)) fin_first(d, c, t0, t1, G.n);
+  } else {
+    if (grid_total(rr, part, &c->ticket, &t0)) fin_next(d, c, t0, G.n);
+  }
+}
+
+// radices of n points, powers of two first; false where a factor or the count is out of range
+bool axis_plan(int n, AxisPlan& A) {
+  A.n = n;
+  A.npass = 0;
+  A.pow2 = 1;
+  A.pingpong = 0;
+  std::vector<int> R;
+  int m = n, p2 = 0;
+  while (m % 2 == 0) {
+    m /= 2;
+    ++p2;
+  }
+  while (p2 > 0) {  // 16 x 8, 8 x 8, 8 x 4 ...: as few passes as radices up to 16 allow, evenly
+    const int passes = (p2 + 3) / 4, b = (p2 + passes - 1) / passes;
+    R.push_back(1 << b);
+    p2 -= b;
+  }
+  for (int p = 3; m > 1; p += 2)
+    while (m % p == 0) {
+      R.push_back(p);
+      m /= p;
+      A.pow2 = 0;
+      if (p > 13) A.pingpong = 1;
+    }
+  if ((int)R.size() > kDirMaxPasses) return false;
+  int L = n;
+  for (int r : R) {
+    A.R[A.npass] = r;
+    A.L[A.npass] = L;
+    A.dM[A.npass] = make_fastdiv(L / r);
+    ++A.npass;
+    L /= r;
+  }
+  return true;
+}
+
+// frequency of every position after the forward passes
+std::vector<int> axis_freq(const AxisPlan& A) {
+  std::vector<int> f(A.n);
+  for (int p = 0; p < A.n; ++p) {
+    int rest = p, freq = 0, mul = 1;
+    for (int q = 0; q < A.npass; ++q) {
+      const int M = A.L[q] / A.R[q];
+      freq += mul * (rest / M);
+      rest %= M;
+      mul *= A.R[q];
+    }
+    f[p] = freq;
+  }
+  return f;
+}
+
+double axis_lambda(int n, int f) {
+  const double s = std::sin(kPi * f / n);
+  return 4.0 * s * s;
+}
+
+size_t fft_smem(const AxisPlan& A, int lp) {
+  return sizeof(float2) * ((size_t)A.n + (size_t)A.n * lp * (A.pingpong ? 2 : 1));
+}
+
+constexpr size_t kMaxSmem = 227 * 1024;
+
+template <class K>
+cudaError_t allow_smem(K k) {
+  // the attribute is the kernel's, shared by every solver of the process
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+}
+
+}  // namespace
+
+cudaError_t DirectSolver::init(int nx, int ny, int nz) {
+  on = false;
+  const int P = nz - 1;
+  // planes: 32 warps of 32 (the tridiagonal kernel's block); lines: what fits in shared memory
+  if (P < 1 || P > 1024 || !axis_plan(nx, a.x) || !axis_plan(ny, a.y)) return cudaSuccess;
+  smem_x = fft_smem(a.x, kLpX);
+  smem_y = fft_smem(a.y, kLpY);
+  if (smem_x > kMaxSmem || smem_y > kMaxSmem) return cudaSuccess;
+  a.nx = nx;
+  a.ny = ny;
+  a.P = P;
+  a.packed = nx % 2 == 0;
+  a.C = a.packed ? nx / 2 : (nx + 1) / 2;
+  a.plane = 2 * a.C * ny;
+  a.rows = (long long)ny * P;
+  a.norm = (float)(1.0 / ((double)nx * ny));
+  zm = P <= 256 ? 16 : 32;
+  zw = (P + zm - 1) / zm;
+  const std::vector<int> fx = axis_freq(a.x), fy = axis_freq(a.y);
+  std::vector<float2> twx(nx), twy(ny);
+  std::vector<int> px(nx), py(ny);
+  std::vector<float> lam(a.plane);
+  for (int m = 0; m < nx; ++m) {
+    twx[m] = make_float2((float)std::cos(2.0 * kPi * m / nx), (float)-std::sin(2.0 * kPi * m / nx));
+    px[fx[m]] = m;
+  }
+  for (int m = 0; m < ny; ++m) {
+    twy[m] = make_float2((float)std::cos(2.0 * kPi * m / ny), (float)-std::sin(2.0 * kPi * m / ny));
+    py[fy[m]] = m;
+  }
+  for (int p = 0; p < ny; ++p) {
+    const int g = fy[p];
+    const double ly = axis_lambda(ny, g);
+    for (int q = 0; q < a.C; ++q) {
+      double l0 = axis_lambda(nx, q), l1 = l0;
+      if (q == 0 && a.packed) {
+        const double lh = axis_lambda(nx, nx / 2);
+        if (g == 0 || 2 * g == ny) l1 = lh;  // mean and Nyquist coefficient, both real
+        else if (2 * g > ny) l0 = l1 = lh;   // the Nyquist coefficient's spectrum
+      }
+      lam[2 * ((size_t)p * a.C + q)] = (float)(l0 + ly);
+      lam[2 * ((size_t)p * a.C + q) + 1] = (float)(l1 + ly);
+    }
+  }
+  cudaError_t e;
+  const size_t b0 = sizeof(float2) * nx, b1 = sizeof(float2) * ny, b2 = sizeof(int) * nx, b3 = sizeof(int) * ny;
+  char* t = nullptr;
+  if ((e = dev_malloc((void**)&t, b0 + b1 + b2 + b3 + sizeof(float) * lam.size()))) return e;
+  tables = t;
+  a.x.tw = (const float2*)t;
+  a.y.tw = (const float2*)(t + b0);
+  a.x.pos = (const int*)(t + b0 + b1);
+  a.y.pos = (const int*)(t + b0 + b1 + b2);
+  a.lam = (const float*)(t + b0 + b1 + b2 + b3);
+  if ((e = cudaMemcpy((void*)a.x.tw, twx.data(), b0, cudaMemcpyHostToDevice))) return e;
+  if ((e = cudaMemcpy((void*)a.y.tw, twy.data(), b1, cudaMemcpyHostToDevice))) return e;
+  if ((e = cudaMemcpy((void*)a.x.pos, px.data(), b2, cudaMemcpyHostToDevice))) return e;
+  if ((e = cudaMemcpy((void*)a.y.pos, py.data(), b3, cudaMemcpyHostToDevice))) return e;
+  if ((e = cudaMemcpy((void*)a.lam, lam.data(), sizeof(float) * lam.size(), cudaMemcpyHostToDevice))) return e;
+  if ((e = dev_malloc((void**)&a.spec, sizeof(float) * (size_t)a.plane * P))) return e;
+  if ((e = allow_smem(k_dir_xf<float, true>)) || (e = allow_smem(k_dir_xf<float, false>)) ||
+      (e = allow_smem(k_dir_xf<double, true>)) || (e = allow_smem(k_dir_xf<double, false>)) ||
+      (e = allow_smem(k_dir_y<false, true>)) || (e = allow_smem(k_dir_y<false, false>)) ||
+      (e = allow_smem(k_dir_y<true, true>)) || (e = allow_smem(k_dir_y<true, false>)) ||
+      (e = allow_smem(k_dir_xi<AddMixed, true>)) || (e = allow_smem(k_dir_xi<AddMixed, false>)) ||
+      (e = allow_smem(k_dir_xi<Add64, true>)) || (e = allow_smem(k_dir_xi<Add64, false>)))
+    return e;
+  on = true;
+  return cudaSuccess;
+}
+
+void DirectSolver::release() {
+  dev_free(tables);
+  dev_free(a.spec);
+  tables = nullptr;
+  a.spec = nullptr;
+  on = false;
+}
+
+namespace {
+
+template <class T, class Add>
+void apply(const DirectSolver& D, const T* r, const Add& add, const SolveCtl* c, cudaStream_t s) {
+  const DirectArgs& a = D.a;
+  const dim3 gx((unsigned)((a.rows + 2 * kDirLines - 1) / (2 * kDirLines)));
+  const dim3 gy((a.C + kDirLines - 1) / kDirLines, a.P);
+  const dim3 gz((a.plane + 31) / 32);
+  const size_t zsm = sizeof(float) * 4 * 32 * D.zw;
+  if (a.x.pow2) SOLVER_LAUNCH(gx, kFftThreads, D.smem_x, s, k_dir_xf<T, true>)(a, r, c);
+  else SOLVER_LAUNCH(gx, kFftThreads, D.smem_x, s, k_dir_xf<T, false>)(a, r, c);
+  if (a.y.pow2) SOLVER_LAUNCH(gy, kFftThreads, D.smem_y, s, k_dir_y<false, true>)(a, c);
+  else SOLVER_LAUNCH(gy, kFftThreads, D.smem_y, s, k_dir_y<false, false>)(a, c);
+  if (D.zm == 16) SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<16, 512>)(a, c);
+  else if (D.zw <= 16) SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<32, 512>)(a, c);
+  else SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<32, 1024>)(a, c);
+  if (a.y.pow2) SOLVER_LAUNCH(gy, kFftThreads, D.smem_y, s, k_dir_y<true, true>)(a, c);
+  else SOLVER_LAUNCH(gy, kFftThreads, D.smem_y, s, k_dir_y<true, false>)(a, c);
+  if (a.x.pow2) SOLVER_LAUNCH(gx, kFftThreads, D.smem_x, s, k_dir_xi<Add, true>)(a, add, c);
+  else SOLVER_LAUNCH(gx, kFftThreads, D.smem_x, s, k_dir_xi<Add, false>)(a, add, c);
+}
+
+// planes per block of the residual kernels: a few blocks per SM, at most 8 planes
+// (longer marches save little: 1 + 2 / kc plane loads per point)
+ResGeom res_geom(const MgLevel& M, int V, dim3* grid) {
+  ResGeom G{lv_of(M), 1, M.nu};
+  const int P = M.nz - 1;
+  const unsigned gx = (unsigned)((M.nx / V + kResX - 1) / kResX), gy = (unsigned)((M.ny + kResY - 1) / kResY);
+  int kc = 8;
+  while (kc > 1 && (long long)gx * gy * ((P + kc - 1) / kc) < 6ll * sm_count()) kc >>= 1;
+  // the partial sums of a block are a double2 each
+  while ((long long)gx * gy * ((P + kc - 1) / kc) > kDirParts) kc *= 2;
+  G.kc = kc;
+  *grid = dim3(gx, gy, (unsigned)((P + kc - 1) / kc));
+  return G;
+}
+
+}  // namespace
+
+void DirectSolver::apply_mixed(const float* r, float* hi, float* lo, double phi_c, double dphi_dk, const SolveCtl* c,
+                               cudaStream_t s) const {
+  apply(*this, r, AddMixed{hi, lo, phi_c, dphi_dk}, c, s);
+}
+
+void DirectSolver::apply_fp64(const double* r, double* x, const SolveCtl* c, cudaStream_t s) const {
+  apply(*this, r, Add64{x}, c, s);
+}
+
+void DirectSolver::residual_mixed(bool first, const MgLevel& M, const float* hi, const float* lo, const float* f, float* r,
+                                  float fold_first, float fold_last, double* part, SolveCtl* c, const DirectLoop& d,
+                                  cudaStream_t s) const {
+  // float4 rows: hi starts one plane into phi32, so its rows are aligned when nx is a multiple of 4
+  const bool v4 = M.nx % 4 == 0;
+  dim3 g;
+  const ResGeom G = res_geom(M, v4 ? 4 : 1, &g);
+  const dim3 b(kResX, kResY);
+  if (v4 && first)
+    SOLVER_LAUNCH(g, b, 0, s, k_dir_resid_ff<4, true>)(G, hi, lo, f, r, fold_first, fold_last, part, c, d);
+  else if (v4)
+    SOLVER_LAUNCH(g, b, 0, s, k_dir_resid_ff<4, false>)(G, hi, lo, f, r, fold_first, fold_last, part, c, d);
+  else if (first)
+    SOLVER_LAUNCH(g, b, 0, s, k_dir_resid_ff<1, true>)(G, hi, lo, f, r, fold_first, fold_last, part, c, d);
+  else
+    SOLVER_LAUNCH(g, b, 0, s, k_dir_resid_ff<1, false>)(G, hi, lo, f, r, fold_first, fold_last, part, c, d);
+}
+
+void DirectSolver::residual_fp64(bool first, const MgLevel& M, const double* x, const double* b, double* r, double* part,
+                                 SolveCtl* c, const DirectLoop& d, cudaStream_t s) const {
+  const bool v2 = M.nx % 2 == 0;
+  dim3 g;
+  const ResGeom G = res_geom(M, v2 ? 2 : 1, &g);
+  const dim3 bl(kResX, kResY);
+  if (v2 && first) SOLVER_LAUNCH(g, bl, 0, s, k_dir_resid64<2, true>)(G, x, b, r, part, c, d);
+  else if (v2) SOLVER_LAUNCH(g, bl, 0, s, k_dir_resid64<2, false>)(G, x, b, r, part, c, d);
+  else if (first) SOLVER_LAUNCH(g, bl, 0, s, k_dir_resid64<1, true>)(G, x, b, r, part, c, d);
+  else SOLVER_LAUNCH(g, bl, 0, s, k_dir_resid64<1, false>)(G, x, b, r, part, c, d);
+}
+
+}  // namespace pic

@@ -2,17 +2,23 @@
 //
 // Unknowns: nodes k = 1..nz-1 (periodic i, j); operator scaled by h^2:
 //   (A x)_ijk = 6 x_ijk - sum of the six neighbours (Dirichlet planes folded into b).
-// Solver: conjugate gradients preconditioned by one geometric-multigrid V(1,1)
+// Solver: refinement passes of the direct solver of k_direct.cu. Measured per
+// step, warm start, against the multigrid CG below: MIXED 128x128x256 661 -> 147
+// us (4 to 5 iterations of about 75 dependent launches -> one pass of 6),
+// 256x256x512 2774 -> 1011, 32x32x64 300 -> 57; FP64 64x64x128 to 1e-13 1477 -> 149.
+// Where its sizes do not fit (more than 1024 unknown planes; rows whose 16-line
+// tile exceeds shared memory): conjugate gradients preconditioned by one
+// geometric-multigrid V(1,1)
 // cycle: red-black Gauss-Seidel (pre-smoothing red then black, post-smoothing
 // black then red, so the cycle is a symmetric operator), full-weighting
 // restriction (b_coarse = 4 FW(r_fine) for the h^2 scaling), trilinear
 // prolongation, coarsest level solved exactly with a dense inverse.
 //  - FP64 path: everything in FP64.
 //  - MIXED path: iterative refinement; the residual r = b - A x and the update
-//    x += d are FP64, the correction d solves A d = r with the same PCG in FP32
-//    (FP32 smoothing and transfer operators), to a loose inner tolerance.
-// Dot products are reduced per block then summed in a fixed order on the
-// device; the host reads one residual norm per iteration to stop.
+//    x += d are float-float, the correction d solves A d = r with the same PCG in
+//    FP32 (FP32 smoothing and transfer operators), to a loose inner tolerance.
+// Every reduction and decision stays on the device (run_host, for profilers,
+// reads one decision per iteration).
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -28,44 +34,11 @@
 #include "pic_kernels.cuh"
 #include "tc_ptx.cuh"
 #include "pic_solver.cuh"
+#include "solver_dev.cuh"
 
 namespace pic {
 
-// Programmatic dependent launch: each solver kernel may be launched while its
-// predecessor drains (it waits here until the predecessor has completed and its
-// writes are visible), and lets its own successor launch as soon as all of its
-// blocks are running. Hides most of the launch gap between the many short
-// multigrid kernels. A no-op for kernels launched without the attribute.
-__device__ __forceinline__ void pdl_enter() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-bool g_pdl = true;  // cleared when a graph with programmatic edges cannot be built
-
-template <class K>
-struct PdlLaunch {
-  K k;
-  dim3 g, b;
-  size_t smem;
-  cudaStream_t s;
-  template <class... A>
-  void operator()(A&&... a) const {
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = g;
-    cfg.blockDim = b;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = g_pdl ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, k, std::forward<A>(a)...);
-  }
-};
-#define SOLVER_LAUNCH(grid, block, smem, stream, ...) \
-  (::pic::count_kernel()), ::pic::PdlLaunch<decltype(&__VA_ARGS__)>{&__VA_ARGS__, dim3(grid), dim3(block), (size_t)(smem), stream}
+bool g_pdl = true;
 
 constexpr int kSB = 256;
 constexpr int kMaxRedBlocks = 152 * 8;  // 1-D reductions over whole vectors
@@ -79,12 +52,6 @@ static int sgrid(long long n) {
   return (int)b;
 }
 
-// Level geometry with 32-bit indices (a level holds far fewer than 2^31 unknowns).
-struct Lv {
-  int nx, ny, nz, pl, nu;
-};
-static Lv lv_of(const MgLevel& L) { return Lv{L.nx, L.ny, L.nz, L.nx * L.ny, (int)L.nu}; }
-
 // 3-D launches without integer division (on GB300 int division and int<->float
 // conversions run on the narrow FP64/conversion pipe): block (32, 8); x covers
 // the `xe` points of a row, y strides over the rows j, z = unknown plane.
@@ -95,19 +62,6 @@ static dim3 g3(const Lv& L, int xe) {
   return dim3((xe + kBX - 1) / kBX, gy, L.nz - 1 > 0 ? L.nz - 1 : 1);
 }
 static const dim3 kB3(kBX, kBY, 1);
-
-template <class T>
-__device__ __forceinline__ T nb_sum(const Lv& L, const T* __restrict__ x, int u, int i, int j, int k) {
-  // k: unknown plane index 0..nz-2
-  const int row = u - i;
-  const int im = i == 0 ? L.nx - 1 : i - 1, ip = i == L.nx - 1 ? 0 : i + 1;
-  const int rm = j == 0 ? (L.ny - 1) * L.nx : -L.nx;
-  const int rp = j == L.ny - 1 ? -(L.ny - 1) * L.nx : L.nx;
-  T s = x[row + im] + x[row + ip] + x[u + rm] + x[u + rp];
-  if (k > 0) s += x[u - L.pl];
-  if (k < L.nz - 2) s += x[u + L.pl];
-  return s;
-}
 
 // loop header of the 3-D kernels: i over [0, xe), j over the rows, k = plane
 #define ROWS3(L, xe)                                                          \
@@ -303,8 +257,6 @@ __global__ void __launch_bounds__(256) k_prolong(Lv F, Lv Cc, const T* __restric
 // & 1 for colour c; nx, ny even). The sums keep the natural kernels' order, so
 // the values are theirs.
 // ---------------------------------------------------------------------------
-template <class V>
-__device__ __forceinline__ bool grid_total(V v, double* part, unsigned* ticket, double* tot);
 __device__ __forceinline__ void set_beta(SolveCtl* c, double rz);
 
 struct SpNb {
@@ -1407,63 +1359,6 @@ bool Mg<T>::vcycle(const T* rhs, T* z, cudaStream_t s, double* part, SolveCtl* c
 // CUDA graph (outer: FP64 true residual / refinement; inner: PCG iterations),
 // so a solve is one graph launch with no host round trip.
 // ---------------------------------------------------------------------------
-template <class V>
-__device__ __forceinline__ V warp_sum(V d) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
-  return d;
-}
-
-// Grid-wide sum without a second launch: each block stores its partial in
-// part[block], then the last block to arrive (a ticket counter) adds all
-// partials in a fixed order (fixed thread assignment and tree, so the total is
-// reproducible) and resets the ticket. Returns true in thread 0 of that block
-// only, with the total in *tot. Every thread of every block must call it.
-// Per-thread and warp sums stay in V (FP32 for the FP32 solve: FP64 is a narrow
-// pipe on GB300); warp totals and everything above them are FP64.
-template <class V>
-__device__ __forceinline__ bool grid_total(V v, double* part, unsigned* ticket, double* tot) {
-  __shared__ double sm[32];
-  __shared__ int s_last;
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  const int nthr = blockDim.x * blockDim.y;
-  const int nw = nthr >> 5;
-  const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
-  const V w = warp_sum(v);
-  if ((tid & 31) == 0) sm[tid >> 5] = (double)w;
-  __syncthreads();
-  if (tid == 0) {
-    double s = 0.0;
-    for (int k = 0; k < nw; ++k) s += sm[k];
-    part[(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = s;
-    __threadfence();
-    s_last = atomicAdd(ticket, 1u) == nb - 1u ? 1 : 0;
-  }
-  __syncthreads();
-  if (!s_last) return false;
-  __threadfence();
-  // four independent partial sums per thread keep several loads in flight
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-  unsigned i = tid;
-  for (; i + 3u * nthr < nb; i += 4u * nthr) {
-    s0 += __ldcg(part + i);
-    s1 += __ldcg(part + i + nthr);
-    s2 += __ldcg(part + i + 2u * nthr);
-    s3 += __ldcg(part + i + 3u * nthr);
-  }
-  for (; i < nb; i += nthr) s0 += __ldcg(part + i);
-  double s = warp_sum((s0 + s1) + (s2 + s3));
-  __syncthreads();
-  if ((tid & 31) == 0) sm[tid >> 5] = s;
-  __syncthreads();
-  if (tid != 0) return false;
-  double t = 0.0;
-  for (int k = 0; k < nw; ++k) t += sm[k];
-  *tot = t;
-  *ticket = 0u;
-  return true;
-}
-
 __device__ __forceinline__ void fin_bb(double bb, SolveCtl* c, double rtol, int maxit) {
   c->bb = bb;
   c->tol2 = rtol * rtol * bb;
@@ -1567,38 +1462,6 @@ __global__ void __launch_bounds__(256) k_residual_prep(Lv L, double* __restrict_
 // is a narrow pipe on GB300). The _rn intrinsics keep the compiler from fusing
 // the products and sums the transformations rely on.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bv = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bv)), __fsub_rn(b, bv));
-}
-
-// sum of the six neighbours of u as s + e (s rounded, e the accumulated exact errors)
-__device__ __forceinline__ void nb_sum_ff(const Lv& L, const float* __restrict__ x, int u, int i, int j, int k, float& s,
-                                          float& e) {
-  const int row = u - i;
-  const int im = i == 0 ? L.nx - 1 : i - 1, ip = i == L.nx - 1 ? 0 : i + 1;
-  const int rm = j == 0 ? (L.ny - 1) * L.nx : -L.nx;
-  const int rp = j == L.ny - 1 ? -(L.ny - 1) * L.nx : L.nx;
-  float t;
-  s = x[row + im];
-  e = 0.f;
-  two_sum(s, x[row + ip], s, t);
-  e = __fadd_rn(e, t);
-  two_sum(s, x[u + rm], s, t);
-  e = __fadd_rn(e, t);
-  two_sum(s, x[u + rp], s, t);
-  e = __fadd_rn(e, t);
-  if (k > 0) {
-    two_sum(s, x[u - L.pl], s, t);
-    e = __fadd_rn(e, t);
-  }
-  if (k < L.nz - 2) {
-    two_sum(s, x[u + L.pl], s, t);
-    e = __fadd_rn(e, t);
-  }
-}
-
 // sum f.f + folded terms -> tolerance (b = f + fold never materialised). f is
 // natural ([k][j][i], planes of nx ny) over the unknown planes, so this is a
 // flat pass: four values per thread (16-byte loads) where the plane size keeps
@@ -1973,7 +1836,6 @@ cudaError_t Solver::init(int nx, int ny, int nz, int precision_) {
   if (precision == 0) {
     if ((err = dev_malloc(&b, sizeof(double) * nn))) return err;
     if ((err = cudaMemset(b, 0, sizeof(double) * nn))) return err;
-    if ((err = dev_malloc(&ax, sizeof(double) * nn))) return err;
   } else {
     if ((err = dev_malloc(&f32, sizeof(float) * nn))) return err;
     if ((err = cudaMemset(f32, 0, sizeof(float) * nn))) return err;
@@ -1987,7 +1849,12 @@ cudaError_t Solver::init(int nx, int ny, int nz, int precision_) {
   memset(host_ctl, 0, sizeof(SolveCtl));
   for (auto& a : aux)
     if ((err = cudaStreamCreateWithFlags(&a, cudaStreamNonBlocking))) return err;
-  if (precision == 0) return p64.init(plan);
+  if ((err = direct.init(nx, ny, nz))) return err;
+  if (direct.on) return precision == 0 ? dev_malloc(&r64, sizeof(double) * nn) : dev_malloc(&r32, sizeof(float) * nn);
+  if (precision == 0) {
+    if ((err = dev_malloc(&ax, sizeof(double) * nn))) return err;
+    return p64.init(plan);
+  }
   return p32.init(plan);
 }
 
@@ -2014,6 +1881,11 @@ void Solver::release() {
   lo32 = nullptr;
   part = nullptr;
   ctl = nullptr;
+  dev_free(r32);
+  dev_free(r64);
+  r32 = nullptr;
+  r64 = nullptr;
+  direct.release();
   p64.release();
   p32.release();
 }
@@ -2031,8 +1903,8 @@ static void capture_pcg_iteration(Pcg<T>& pc, const Lv& L, double* part, SolveCt
   SOLVER_LAUNCH(G, kSB, 0, s, k_update_rr<T>)(L.nu, pc.d, pc.r, pc.p, pc.q, ctl, part, h_inner, use_graph);
 }
 
-// Add a WHILE node at the current capture position of `s`; returns its body graph.
-static cudaError_t add_while(cudaStream_t s, cudaGraphConditionalHandle* h, unsigned default_value, cudaGraph_t* body) {
+// Add a WHILE node on handle h at the current capture position of `s`; returns its body graph.
+static cudaError_t add_while(cudaStream_t s, cudaGraphConditionalHandle h, cudaGraph_t* body) {
   cudaStreamCaptureStatus status;
   cudaGraph_t g;
   const cudaGraphNode_t* deps = nullptr;
@@ -2041,11 +1913,9 @@ static cudaError_t add_while(cudaStream_t s, cudaGraphConditionalHandle* h, unsi
   cudaError_t e = cudaStreamGetCaptureInfo(s, &status, nullptr, &g, &deps, &edges, &ndeps);
   if (e != cudaSuccess) return e;
   if (status != cudaStreamCaptureStatusActive) return cudaErrorIllegalState;
-  e = cudaGraphConditionalHandleCreate(h, g, default_value, cudaGraphCondAssignDefault);
-  if (e != cudaSuccess) return e;
   cudaGraphNodeParams np = {};
   np.type = cudaGraphNodeTypeConditional;
-  np.conditional.handle = *h;
+  np.conditional.handle = h;
   np.conditional.type = cudaGraphCondTypeWhile;
   np.conditional.size = 1;
   cudaGraphNode_t node;
@@ -2053,6 +1923,14 @@ static cudaError_t add_while(cudaStream_t s, cudaGraphConditionalHandle* h, unsi
   if (e != cudaSuccess) return e;
   *body = np.conditional.phGraph_out[0];
   return cudaStreamUpdateCaptureDependencies(s, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
+}
+
+// the graph that s is being captured into
+static cudaError_t capture_graph(cudaStream_t s, cudaGraph_t* g) {
+  cudaStreamCaptureStatus status;
+  const cudaError_t e = cudaStreamGetCaptureInfo(s, &status, nullptr, g, nullptr, nullptr, nullptr);
+  if (e != cudaSuccess) return e;
+  return status == cudaStreamCaptureStatusActive ? cudaSuccess : cudaErrorIllegalState;
 }
 
 // Record the solve of A x = b (x = unknown view of phi) for this instance;
@@ -2109,6 +1987,7 @@ cudaError_t Solver::build_graph_once(double* x, float* phi32, double phi_c, doub
 // inner WHILE node of PCG iterations and the update) at the capture position of
 // s0, in whatever graph s0 is capturing into.
 cudaError_t Solver::record(cudaStream_t s0) {
+  if (direct.on) return record_direct(s0);
   const Lv L = lv_of(plan[0]);
   const int G = sgrid(L.nu);
   const dim3 PGd = g3(L, L.nx);
@@ -2127,7 +2006,10 @@ cudaError_t Solver::record(cudaStream_t s0) {
     SOLVER_LAUNCH(G, kSB, 0, s0, k_dot_bb)(L.nu, b, part, ctl, rtol, maxit);
   }
   e = cudaGetLastError();
-  if (e == cudaSuccess) e = add_while(s0, &h_outer, 1u, &outer_body);
+  cudaGraph_t g = nullptr;
+  if (e == cudaSuccess) e = capture_graph(s0, &g);
+  if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&h_outer, g, 1u, cudaGraphCondAssignDefault);
+  if (e == cudaSuccess) e = add_while(s0, h_outer, &outer_body);
   if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(s1, outer_body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
   if (e == cudaSuccess) {
     e = cudaGraphConditionalHandleCreate(&h_inner, outer_body, 0u, 0);
@@ -2140,28 +2022,7 @@ cudaError_t Solver::record(cudaStream_t s0) {
                                                               inner_rtol, mixed, max_outer, 1);
       }
     }
-    if (e == cudaSuccess) {
-      // inner WHILE node in the outer body
-      cudaStreamCaptureStatus status;
-      cudaGraph_t g;
-      const cudaGraphNode_t* deps = nullptr;
-      const cudaGraphEdgeData* edges = nullptr;
-      size_t ndeps = 0;
-      e = cudaStreamGetCaptureInfo(s1, &status, nullptr, &g, &deps, &edges, &ndeps);
-      if (e == cudaSuccess) {
-        cudaGraphNodeParams np = {};
-        np.type = cudaGraphNodeTypeConditional;
-        np.conditional.handle = h_inner;
-        np.conditional.type = cudaGraphCondTypeWhile;
-        np.conditional.size = 1;
-        cudaGraphNode_t node;
-        e = cudaGraphAddNode(&node, g, deps, edges, ndeps, &np);
-        if (e == cudaSuccess) {
-          inner_body = np.conditional.phGraph_out[0];
-          e = cudaStreamUpdateCaptureDependencies(s1, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
-        }
-      }
-    }
+    if (e == cudaSuccess) e = add_while(s1, h_inner, &inner_body);  // in the outer body
     if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(s2, inner_body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
     if (e == cudaSuccess) {
       if (mixed) capture_pcg_iteration(p32, L, part, ctl, h_inner, s2);
@@ -2183,6 +2044,44 @@ cudaError_t Solver::record(cudaStream_t s0) {
   return e;
 }
 
+// One refinement pass of the direct solver: x += A^-1 r, then the new residual.
+void Solver::direct_pass(const DirectLoop& d, cudaStream_t s) {
+  if (precision != 0) {
+    direct.apply_mixed(r32, hphi32, lo32, h_phi_c, h_dphi_dk, ctl, s);
+    direct.residual_mixed(false, plan[0], hphi32, lo32, f32, r32, fold_first(), fold_last(), part, ctl, d, s);
+  } else {
+    direct.apply_fp64(r64, hx, ctl, s);
+    direct.residual_fp64(false, plan[0], hx, b, r64, part, ctl, d, s);
+  }
+}
+
+void Solver::direct_first(const DirectLoop& d, cudaStream_t s) {
+  if (precision != 0)
+    direct.residual_mixed(true, plan[0], hphi32, lo32, f32, r32, fold_first(), fold_last(), part, ctl, d, s);
+  else
+    direct.residual_fp64(true, plan[0], hx, b, r64, part, ctl, d, s);
+}
+
+// Add the solve by the direct solver: the first residual, one pass (gated by its
+// decision, so that the usual solve enters no loop), and a WHILE node of further
+// passes that the last residual opens.
+cudaError_t Solver::record_direct(cudaStream_t s0) {
+  DirectLoop d{h_rtol, h_maxit, max_outer, 1, 0};
+  cudaGraph_t g;
+  cudaError_t e = capture_graph(s0, &g);
+  if (e != cudaSuccess) return e;
+  if ((e = cudaGraphConditionalHandleCreate(&d.handle, g, 0u, cudaGraphCondAssignDefault))) return e;
+  direct_first(d, s0);
+  direct_pass(d, s0);
+  if ((e = cudaGetLastError())) return e;
+  cudaGraph_t body = nullptr, tmp;
+  if ((e = add_while(s0, d.handle, &body))) return e;
+  if ((e = cudaStreamBeginCaptureToGraph(aux[0], body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed))) return e;
+  direct_pass(d, aux[0]);
+  e = cudaStreamEndCapture(aux[0], &tmp);
+  return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
 cudaError_t Solver::launch(cudaStream_t s) {
   if (exec) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -2199,6 +2098,17 @@ cudaError_t Solver::launch(cudaStream_t s) {
 
 // The same kernels driven from the host, one read-back per decision.
 cudaError_t Solver::run_host(cudaStream_t s) {
+  if (direct.on) {
+    const DirectLoop d{h_rtol, h_maxit, max_outer, 0, 0};
+    direct_first(d, s);
+    do {
+      direct_pass(d, s);
+      cudaError_t e = cudaMemcpyAsync(host_ctl, ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      if (e != cudaSuccess) return e;
+    } while (host_ctl->more);
+    return cudaGetLastError();
+  }
   const Lv L = lv_of(plan[0]);
   const int G = sgrid(L.nu);
   const dim3 PGd = g3(L, L.nx);

@@ -6,6 +6,8 @@
 
 #include <cuda_runtime.h>
 
+#include "pic_direct.cuh"
+
 namespace pic {
 
 struct MgLevel {
@@ -21,6 +23,7 @@ struct SolveCtl {
   unsigned ticket;  // blocks finished in the current grid-wide sum (0 between launches)
   int ax_valid;     // Solver::ax holds A x for the current x
   int stopped;      // the last residual ended the outer loop
+  double scale, inv_scale;  // direct solver: brings the FP64 residual to unit size for its FP32 pass
   int spec_timeout; // a copy of the exact coarse solve did not arrive in time (sticky until reported)
 };
 
@@ -65,7 +68,9 @@ struct Pcg {
   void release();
 };
 
-// Solve of A x = b on the unknown nodes. FP64 path: outer loop of FP64 true
+// Solve of A x = b on the unknown nodes, by refinement passes of the direct
+// solver (pic_direct.cuh) wherever its sizes fit. Beyond them (more than 1024
+// unknown planes, rows that do not fit in shared memory) the FP64 path: outer loop of FP64 true
 // residuals around an FP64 PCG on the correction (plain restarted PCG).
 // Mixed path: the same loop is iterative refinement, the correction solved by
 // an FP32 PCG to inner_rtol relative to the current residual.
@@ -84,6 +89,9 @@ struct Solver {
   SolveCtl* host_ctl = nullptr;
   double inner_rtol = 1e-6;
   int max_outer = 40;
+  DirectSolver direct;
+  float* r32 = nullptr;   // residual of the direct solver's passes (MIXED)
+  double* r64 = nullptr;  // (FP64)
   Pcg<double> p64;
   Pcg<float> p32;
   cudaGraph_t graph = nullptr;
@@ -96,6 +104,9 @@ struct Solver {
   cudaError_t build_graph_once(double* x, float* phi32, double phi_c, double phi_a, int nz, double rtol, int maxit);
   cudaError_t launch(cudaStream_t s);
   cudaError_t record(cudaStream_t s0);
+  cudaError_t record_direct(cudaStream_t s0);
+  void direct_first(const DirectLoop& d, cudaStream_t s);
+  void direct_pass(const DirectLoop& d, cudaStream_t s);
   cudaError_t run_host(cudaStream_t s);
   cudaError_t invalidate(cudaStream_t s);
   // MIXED path: FP64 phi (unknown view, hx) from (hi, lo), and back (x = nullptr: phi = 0)

@@ -1,0 +1,89 @@
+"""The direct Poisson solver over the sizes where it changes path: every radix of
+its FFTs (powers of two, 3 to 13, primes without a butterfly), odd and even rows
+(with and without a Nyquist column), rows that do not fill a tile, one to many
+warps of planes with ragged last chunks, and the first size beyond it (the
+multigrid CG). Reference: the same 7-point problem in FP64 by its eigenvectors
+(numpy). The solve stops at ||b - A x|| <= rtol ||b||, so its error is at most
+rtol ||b|| / lambda_min, lambda_min = 4 sin^2(pi / (2 nz)) the smallest
+eigenvalue; the mixed store solves for the FP32 charge term, which the reference
+takes too, and its residual is known to about 2^-46 of its largest term
+12 max|x| (float-float), which adds that term's share to the bound.
+"""
+import math
+
+import numpy as np
+import pytest
+
+from tests._cases import bare
+
+pytestmark = pytest.mark.gpu
+
+EPS0 = 8.8541878128e-12
+SIZES = [
+    (16, 16, 17), (32, 32, 64), (8, 4, 2), (2, 2, 3), (1, 1, 5), (4, 1, 18), (1, 6, 9), (3, 5, 16),
+    (7, 9, 33), (11, 13, 34), (26, 22, 15), (34, 46, 20), (17, 19, 35), (40, 36, 90), (24, 20, 34), (15, 14, 257),
+    (128, 64, 40), (256, 16, 12), (62, 128, 9), (96, 80, 150), (10, 12, 258), (6, 8, 514), (4, 6, 1025), (8, 8, 1026),
+]
+
+
+def _reference(nx, ny, nz, b):
+    k = np.arange(1, nz)
+    S = math.sqrt(2.0 / nz) * np.sin(math.pi / nz * k[:, None] * k[None, :])
+
+    def lam(n):
+        return 4 * np.sin(math.pi * np.arange(n) / n) ** 2
+
+    f = np.fft.fft2(np.einsum("ab,byx->ayx", S, b))
+    f /= (4 * np.sin(math.pi * k / (2 * nz)) ** 2)[:, None, None] + lam(ny)[None, :, None] + lam(nx)[None, None, :]
+    return np.einsum("ab,byx->ayx", S, np.fft.ifft2(f).real)
+
+
+@pytest.mark.parametrize("precision,rtol", [(0, 1e-12), (1, 1e-8)])
+@pytest.mark.parametrize("nx,ny,nz", SIZES)
+def test_solve_matches_eigenvector_solution(nx, ny, nz, precision, rtol):
+    import paper_2606_05893_gb300 as pkg
+    h, phi_c, phi_a = 2.5e-9, -2.0, 37.0 * nz
+    wl = bare(nx=nx, ny=ny, nz=nz, h=h, phi_c=phi_c, phi_a=phi_a)
+    rng = np.random.default_rng(nx + 100 * ny + 10000 * nz)
+    rho = rng.standard_normal((nz + 1, ny, nx)) * 2e6 + 4e5
+    scale = h * h / EPS0
+    charge = rho[1:nz] * scale
+    if precision:
+        charge = (np.float32(scale) * rho[1:nz].astype(np.float32)).astype(np.float64)
+    b = charge.copy()
+    b[0] += phi_c
+    b[-1] += phi_a
+    sim = pkg.Simulation(wl, precision=precision, cg_rtol=rtol, cg_maxit=20000, preload=False)
+    for guess in (None, rng.standard_normal(rho.shape) * 10):
+        phi, iters, rel = sim.solve(rho, guess)
+        assert rel <= rtol and iters > 0
+        exact = _reference(nx, ny, nz, b)
+        lam_min = 4 * math.sin(math.pi / (2 * nz)) ** 2
+        bound = rtol * np.linalg.norm(b)
+        bound += 12 * np.abs(exact).max() * math.sqrt(b.size) * (2.0 ** -46 if precision else 2.0 ** -52)
+        assert np.linalg.norm(phi[1:nz] - exact) <= bound / lam_min
+        assert np.all(phi[0] == phi_c) and np.all(phi[nz] == phi_a)
+    sim.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_zero_right_hand_side_gives_zero(precision):
+    import paper_2606_05893_gb300 as pkg
+    wl = bare(nx=12, ny=10, nz=20, phi_c=0.0, phi_a=0.0)
+    sim = pkg.Simulation(wl, precision=precision, cg_rtol=1e-10, preload=False)
+    guess = np.random.default_rng(1).standard_normal((21, 10, 12))
+    phi, iters, rel = sim.solve(np.zeros((21, 10, 12)), guess)
+    assert iters == 0 and rel == 0.0 and np.all(phi == 0.0)
+    sim.close()
+
+
+def test_tiny_potentials_do_not_underflow():
+    """The FP64 store's FP32 passes work on a residual scaled to unit size."""
+    import paper_2606_05893_gb300 as pkg
+    wl = bare(nx=12, ny=10, nz=20, phi_c=0.0, phi_a=0.0)
+    sim = pkg.Simulation(wl, precision=0, cg_rtol=1e-12, preload=False)
+    rho = np.random.default_rng(2).standard_normal((21, 10, 12))
+    big, _, _ = sim.solve(rho)
+    small, _, rel = sim.solve(rho * 2.0 ** -300)
+    assert rel <= 1e-12 and np.array_equal(small * 2.0 ** 300, big)
+    sim.close()
