@@ -445,8 +445,9 @@ uint64_t pic_kernel_count(void);
  * own pool at start-up, or that must keep a fixed footprint between coupling
  * steps). It solves the node-grid Poisson problem that pic_solve solves --
  * 7-point operator, periodic x/y, Dirichlet planes phi(k=0) = phi_cathode_V and
- * phi(k=nz) = phi_anode_V -- by unpreconditioned conjugate gradients,
- * with every work vector in one fixed array inside the library (file-scope
+ * phi(k=nz) = phi_anode_V -- by refinement passes of the direct solver of the
+ * steps (on grids that it does not take, such as more than 1024 unknown planes, by
+ * unpreconditioned conjugate gradients), with every work vector in one fixed array inside the library (file-scope
  * __device__ storage of PIC_STATIC_MAX_UNKNOWNS-sized vectors, about 8 MiB,
  * held by every GPU that loads the library until the process exits). It calls
  * no cudaMalloc, cudaFree or other allocating routine.
@@ -454,23 +455,24 @@ uint64_t pic_kernel_count(void);
  *  phi_dev: device array of the same size; its interior (k = 1..nz-1) is the
  *           initial guess on entry; on return it holds the solution and the
  *           electrode planes hold their potentials. Caller-owned.
- *  Iterates until the recursive residual reaches rtol ||b|| or maxit
- *  iterations have run, then recomputes the true residual b - A phi; the status
- *  follows that true residual, which at very tight rtol can sit just above the
- *  recursive one. The true relative residual is reported in *resid_rel and the
- *  iteration count in *iters (either may be NULL). rho = 0 with both electrodes
+ *  Iterates until the residual (of the passes the true one b - A phi, of CG the
+ *  recursive one) reaches rtol ||b|| or maxit iterations have run (passes: at
+ *  most 40); the status follows the true residual, which CG recomputes at the end
+ *  and which at very tight rtol can sit just above its recursive one. The true
+ *  relative residual is reported in *resid_rel and the passes or CG iterations
+ *  in *iters (either may be NULL). rho = 0 with both electrodes
  *  at 0 V gives the zero solution after 0 iterations.
  * Returns PIC_EINVAL for bad arguments or nx*ny*(nz-1) > PIC_STATIC_MAX_UNKNOWNS,
  * PIC_ENOCONV if the true residual is above rtol, PIC_ECUDA if a launch or copy
  * fails; pic_last_error(NULL) then says which. The first call on a device looks up the address of
  * the fixed array on that device (cudaGetSymbolAddress, with that device
- * current). No call can be captured into a CUDA graph: every iteration
- * synchronises the stream (below). All calls share
+ * current). No call can be captured into a CUDA graph: it synchronises the
+ * stream (below). All calls share
  * the array and it keeps the last call's contents (each call writes every
  * vector before reading it); calls that overlap on the GPU -- on different
  * streams or from different host threads on the same device -- race on it.
- * Work runs on cuda_stream; the call reads the residual back and synchronises
- * that stream once per iteration. */
+ * Work runs on cuda_stream; the call reads the outcome back and synchronises
+ * that stream after the second and every later pass, or once per CG iteration. */
 #define PIC_STATIC_MAX_UNKNOWNS (1 << 18)
 pic_status pic_poisson_solve_static(int32_t nx, int32_t ny, int32_t nz, double h, double phi_cathode_V,
                                     double phi_anode_V, const double* rho_dev, double* phi_dev, double rtol,

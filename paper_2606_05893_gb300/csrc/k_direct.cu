@@ -23,6 +23,7 @@
 // reversed): the tridiagonal kernel only needs each column's eigenvalue.
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <vector>
 
 #include "dev_mem.cuh"
@@ -408,31 +409,40 @@ __global__ void __launch_bounds__(THREADS) k_dir_z(DirectArgs a, const SolveCtl*
   float* sE = sF + 32 * W;       // last value with zero neighbours, then the left neighbour's value
   float* sD = sE + 32 * W;       // response of the first value to the right neighbour
   float* sV = sD + 32 * W;
+  float* sC = sV + 32 * W;       // [M][32] the pivots, where registers do not hold them
   const int col = blockIdx.x * 32 + lane;
   const bool in = col < a.plane;
   const int k0 = w * M, len = min(M, a.P - k0);
   float* g = a.spec + (long long)k0 * a.plane + col;
-  float y[M], cp[M];
+  constexpr bool kShared = THREADS > 512;  // 64 registers a thread hold the planes alone
+  float y[M], cr[M] = {};
+  auto cp = [&](int k) -> float {
+    if constexpr (kShared) return *(volatile float*)(sC + 32 * k);  // reloaded at each use
+    else return cr[k];
+  };
 #pragma unroll
   for (int k = 0; k < M; ++k) y[k] = in && k < len ? g[(long long)k * a.plane] : 0.f;
   const float lam = in ? __ldg(a.lam + col) : 1.f;
   float s = lam + 1.f, b = 1.f;
 #pragma unroll
   for (int k = 0; k < M; ++k) {
-    cp[k] = 1.f / (1.f + s);
-    s = fmaf(s, cp[k], lam);
-    b *= cp[k];
+    const float v = 1.f / (1.f + s);
+    if (kShared) sC[32 * k] = v;  // every warp writes the same value
+    else cr[k] = v;
+    s = fmaf(s, v, lam);
+    b *= v;
   }
+  if (kShared) __syncwarp();
   float t = 0.f;
 #pragma unroll
   for (int k = 0; k < M; ++k) {
-    t = cp[k] * (y[k] + t);
+    t = cp(k) * (y[k] + t);
     y[k] = k < len ? t : 0.f;
   }
   sE[32 * w] = y[M - 1];
   t = 0.f;
 #pragma unroll
-  for (int k = M - 1; k >= 0; --k) t = fmaf(cp[k], t, y[k]);
+  for (int k = M - 1; k >= 0; --k) t = fmaf(cp(k), t, y[k]);
   sF[32 * w] = t;
   __syncthreads();
   if (w == 0) {
@@ -440,12 +450,12 @@ __global__ void __launch_bounds__(THREADS) k_dir_z(DirectArgs a, const SolveCtl*
     // and the far end), L the left chunk's E, R the right chunk's F. With
     // L = u + v F: F = (pF + a u + b R) / (1 - a v), and u, v of the next chunk.
     const int last = a.P - (W - 1) * M;  // planes of the last chunk
-    float alast = cp[0];
+    float alast = cp(0);
 #pragma unroll
-    for (int k = 1; k < M; ++k) alast = k < last ? cp[k] : alast;
+    for (int k = 1; k < M; ++k) alast = k < last ? cp(k) : alast;
     float u = 0.f, v = 0.f;
     for (int q = 0; q < W; ++q) {
-      const float aq = q == W - 1 ? alast : cp[M - 1], bq = q == W - 1 ? 0.f : b;
+      const float aq = q == W - 1 ? alast : cp(M - 1), bq = q == W - 1 ? 0.f : b;
       const float inv = 1.f / fmaf(-aq, v, 1.f);
       const float F = fmaf(aq, u, sF[32 * q]) * inv, D = bq * inv, pE = sE[32 * q];
       sF[32 * q] = F;
@@ -467,14 +477,14 @@ __global__ void __launch_bounds__(THREADS) k_dir_z(DirectArgs a, const SolveCtl*
   const float right = w + 1 < W ? sF[32 * (w + 1)] : 0.f;
 #pragma unroll
   for (int k = 0; k < M; ++k) {
-    t *= cp[k];
+    t *= cp(k);
     y[k] += t;
   }
-  y[M - 1] = fmaf(cp[M - 1], right, y[M - 1]);
+  y[M - 1] = fmaf(cp(M - 1), right, y[M - 1]);
   t = 0.f;
 #pragma unroll
   for (int k = M - 1; k >= 0; --k) {
-    t = k < len ? fmaf(cp[k], t, y[k]) : 0.f;
+    t = k < len ? fmaf(cp(k), t, y[k]) : 0.f;
     if (in && k < len) g[(long long)k * a.plane] = t;
   }
 }
@@ -793,25 +803,48 @@ bool axis_plan(int n, AxisPlan& A) {
   return true;
 }
 
-// frequency of every position after the forward passes
-std::vector<int> axis_freq(const AxisPlan& A) {
-  std::vector<int> f(A.n);
-  for (int p = 0; p < A.n; ++p) {
-    int rest = p, freq = 0, mul = 1;
-    for (int q = 0; q < A.npass; ++q) {
-      const int M = A.L[q] / A.R[q];
-      freq += mul * (rest / M);
-      rest %= M;
-      mul *= A.R[q];
-    }
-    f[p] = freq;
+// frequency that the forward passes leave at position p
+__device__ __forceinline__ int axis_freq(const AxisPlan& A, int p) {
+  int freq = 0, mul = 1;
+  for (int q = 0; q < A.npass; ++q) {
+    const int M = A.dM[q].d, d = fdiv(p, A.dM[q]);
+    freq += mul * d;
+    p -= d * M;
+    mul *= A.R[q];
   }
-  return f;
+  return freq;
+}
+__device__ __forceinline__ double axis_lambda(int n, int f) {  // 2 - 2 cos(2 pi f / n), without cancellation
+  const double s = sinpi((double)f / n);
+  return 4.0 * s * s;
 }
 
-double axis_lambda(int n, int f) {
-  const double s = std::sin(kPi * f / n);
-  return 4.0 * s * s;
+// twiddles, positions and eigenvalues of a plan, formed in FP64 and rounded once
+__global__ void k_dir_tables(DirectArgs a) {
+  const int t = (int)gtid(), n = (int)gstride();
+#pragma unroll
+  for (int axis = 0; axis < 2; ++axis) {
+    const AxisPlan& A = axis == 0 ? a.x : a.y;
+    for (int m = t; m < A.n; m += n) {
+      double s, c;
+      sincospi(2.0 * m / A.n, &s, &c);
+      const_cast<float2*>(A.tw)[m] = make_float2((float)c, (float)-s);
+      const_cast<int*>(A.pos)[axis_freq(A, m)] = m;
+    }
+  }
+  for (int u = t; u < a.plane / 2; u += n) {
+    const int p = u / a.C, q = u - p * a.C;
+    const int g = axis_freq(a.y, p);
+    const double ly = axis_lambda(a.ny, g);
+    double l0 = axis_lambda(a.nx, q), l1 = l0;
+    if (q == 0 && a.packed) {
+      if (g == 0 || 2 * g == a.ny) l1 = 4.0;  // mean and Nyquist coefficient, both real
+      else if (2 * g > a.ny) l0 = l1 = 4.0;   // the Nyquist coefficient's spectrum
+    }
+    float* lam = const_cast<float*>(a.lam);
+    lam[2 * u] = (float)(l0 + ly);
+    lam[2 * u + 1] = (float)(l1 + ly);
+  }
 }
 
 size_t fft_smem(const AxisPlan& A, int lp) {
@@ -828,14 +861,13 @@ cudaError_t allow_smem(K k) {
 
 }  // namespace
 
-cudaError_t DirectSolver::init(int nx, int ny, int nz) {
-  on = false;
+bool DirectSolver::plan(int nx, int ny, int nz) {
   const int P = nz - 1;
   // planes: 32 warps of 32 (the tridiagonal kernel's block); lines: what fits in shared memory
-  if (P < 1 || P > 1024 || !axis_plan(nx, a.x) || !axis_plan(ny, a.y)) return cudaSuccess;
+  if (P < 1 || P > 1024 || !axis_plan(nx, a.x) || !axis_plan(ny, a.y)) return false;
   smem_x = fft_smem(a.x, kLpX);
   smem_y = fft_smem(a.y, kLpY);
-  if (smem_x > kMaxSmem || smem_y > kMaxSmem) return cudaSuccess;
+  if (smem_x > kMaxSmem || smem_y > kMaxSmem) return false;
   a.nx = nx;
   a.ny = ny;
   a.P = P;
@@ -846,48 +878,23 @@ cudaError_t DirectSolver::init(int nx, int ny, int nz) {
   a.norm = (float)(1.0 / ((double)nx * ny));
   zm = P <= 256 ? 16 : 32;
   zw = (P + zm - 1) / zm;
-  const std::vector<int> fx = axis_freq(a.x), fy = axis_freq(a.y);
-  std::vector<float2> twx(nx), twy(ny);
-  std::vector<int> px(nx), py(ny);
-  std::vector<float> lam(a.plane);
-  for (int m = 0; m < nx; ++m) {
-    twx[m] = make_float2((float)std::cos(2.0 * kPi * m / nx), (float)-std::sin(2.0 * kPi * m / nx));
-    px[fx[m]] = m;
-  }
-  for (int m = 0; m < ny; ++m) {
-    twy[m] = make_float2((float)std::cos(2.0 * kPi * m / ny), (float)-std::sin(2.0 * kPi * m / ny));
-    py[fy[m]] = m;
-  }
-  for (int p = 0; p < ny; ++p) {
-    const int g = fy[p];
-    const double ly = axis_lambda(ny, g);
-    for (int q = 0; q < a.C; ++q) {
-      double l0 = axis_lambda(nx, q), l1 = l0;
-      if (q == 0 && a.packed) {
-        const double lh = axis_lambda(nx, nx / 2);
-        if (g == 0 || 2 * g == ny) l1 = lh;  // mean and Nyquist coefficient, both real
-        else if (2 * g > ny) l0 = l1 = lh;   // the Nyquist coefficient's spectrum
-      }
-      lam[2 * ((size_t)p * a.C + q)] = (float)(l0 + ly);
-      lam[2 * ((size_t)p * a.C + q) + 1] = (float)(l1 + ly);
-    }
-  }
-  cudaError_t e;
-  const size_t b0 = sizeof(float2) * nx, b1 = sizeof(float2) * ny, b2 = sizeof(int) * nx, b3 = sizeof(int) * ny;
-  char* t = nullptr;
-  if ((e = dev_malloc((void**)&t, b0 + b1 + b2 + b3 + sizeof(float) * lam.size()))) return e;
-  tables = t;
+  return true;
+}
+
+size_t DirectSolver::table_bytes() const {
+  return (sizeof(float2) + sizeof(int)) * (size_t)(a.nx + a.ny) + sizeof(float) * (size_t)a.plane;
+}
+size_t DirectSolver::spec_bytes() const { return sizeof(float) * (size_t)a.plane * a.P; }
+
+cudaError_t DirectSolver::place(void* tables_mem, void* spec_mem, cudaStream_t s) {
+  char* t = (char*)tables_mem;
   a.x.tw = (const float2*)t;
-  a.y.tw = (const float2*)(t + b0);
-  a.x.pos = (const int*)(t + b0 + b1);
-  a.y.pos = (const int*)(t + b0 + b1 + b2);
-  a.lam = (const float*)(t + b0 + b1 + b2 + b3);
-  if ((e = cudaMemcpy((void*)a.x.tw, twx.data(), b0, cudaMemcpyHostToDevice))) return e;
-  if ((e = cudaMemcpy((void*)a.y.tw, twy.data(), b1, cudaMemcpyHostToDevice))) return e;
-  if ((e = cudaMemcpy((void*)a.x.pos, px.data(), b2, cudaMemcpyHostToDevice))) return e;
-  if ((e = cudaMemcpy((void*)a.y.pos, py.data(), b3, cudaMemcpyHostToDevice))) return e;
-  if ((e = cudaMemcpy((void*)a.lam, lam.data(), sizeof(float) * lam.size(), cudaMemcpyHostToDevice))) return e;
-  if ((e = dev_malloc((void**)&a.spec, sizeof(float) * (size_t)a.plane * P))) return e;
+  a.y.tw = a.x.tw + a.nx;
+  a.x.pos = (const int*)(a.y.tw + a.ny);
+  a.y.pos = a.x.pos + a.nx;
+  a.lam = (const float*)(a.y.pos + a.ny);
+  a.spec = (float*)spec_mem;
+  cudaError_t e;
   if ((e = allow_smem(k_dir_xf<float, true>)) || (e = allow_smem(k_dir_xf<float, false>)) ||
       (e = allow_smem(k_dir_xf<double, true>)) || (e = allow_smem(k_dir_xf<double, false>)) ||
       (e = allow_smem(k_dir_y<false, true>)) || (e = allow_smem(k_dir_y<false, false>)) ||
@@ -895,6 +902,19 @@ cudaError_t DirectSolver::init(int nx, int ny, int nz) {
       (e = allow_smem(k_dir_xi<AddMixed, true>)) || (e = allow_smem(k_dir_xi<AddMixed, false>)) ||
       (e = allow_smem(k_dir_xi<Add64, true>)) || (e = allow_smem(k_dir_xi<Add64, false>)))
     return e;
+  const int n = std::max(std::max(a.nx, a.ny), a.plane / 2);
+  PIC_LAUNCH(std::min((n + 127) / 128, 1024), 128, 0, s, k_dir_tables)(a);
+  return cudaGetLastError();
+}
+
+cudaError_t DirectSolver::init(int nx, int ny, int nz) {
+  on = false;
+  if (!plan(nx, ny, nz)) return cudaSuccess;
+  cudaError_t e;
+  if ((e = dev_malloc(&tables, table_bytes()))) return e;
+  if ((e = dev_malloc((void**)&a.spec, spec_bytes()))) return e;
+  if ((e = place(tables, a.spec, cudaStreamLegacy))) return e;
+  if ((e = cudaStreamSynchronize(cudaStreamLegacy))) return e;
   on = true;
   return cudaSuccess;
 }
@@ -915,7 +935,7 @@ void apply(const DirectSolver& D, const T* r, const Add& add, const SolveCtl* c,
   const dim3 gx((unsigned)((a.rows + 2 * kDirLines - 1) / (2 * kDirLines)));
   const dim3 gy((a.C + kDirLines - 1) / kDirLines, a.P);
   const dim3 gz((a.plane + 31) / 32);
-  const size_t zsm = sizeof(float) * 4 * 32 * D.zw;
+  const size_t zsm = sizeof(float) * 32 * (4 * D.zw + (D.zw > 16 ? D.zm : 0));
   if (a.x.pow2) SOLVER_LAUNCH(gx, kFftThreads, D.smem_x, s, k_dir_xf<T, true>)(a, r, c);
   else SOLVER_LAUNCH(gx, kFftThreads, D.smem_x, s, k_dir_xf<T, false>)(a, r, c);
   if (a.y.pow2) SOLVER_LAUNCH(gy, kFftThreads, D.smem_y, s, k_dir_y<false, true>)(a, c);
@@ -975,7 +995,8 @@ void DirectSolver::residual_mixed(bool first, const MgLevel& M, const float* hi,
 
 void DirectSolver::residual_fp64(bool first, const MgLevel& M, const double* x, const double* b, double* r, double* part,
                                  SolveCtl* c, const DirectLoop& d, cudaStream_t s) const {
-  const bool v2 = M.nx % 2 == 0;
+  // double2 rows: the caller's own array may start anywhere on a double
+  const bool v2 = M.nx % 2 == 0 && ((uintptr_t)x | (uintptr_t)b | (uintptr_t)r) % 16 == 0;
   dim3 g;
   const ResGeom G = res_geom(M, v2 ? 2 : 1, &g);
   const dim3 bl(kResX, kResY);

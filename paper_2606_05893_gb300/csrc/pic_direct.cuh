@@ -57,6 +57,12 @@ struct DirectSolver {
   int zm = 0, zw = 0;  // planes per warp and warps of the tridiagonal kernel
   // nz - 1 unknown planes; on stays false where the sizes do not fit
   cudaError_t init(int nx, int ny, int nz);
+  // the same in parts, on memory of the caller's: the plan (false: the sizes do
+  // not fit), what it needs, and its placement (the tables are written on s)
+  bool plan(int nx, int ny, int nz);
+  size_t table_bytes() const;
+  size_t spec_bytes() const;
+  cudaError_t place(void* tables_mem, void* spec_mem, cudaStream_t s);
   void release();
   // x += A^-1 r: r FP32 (mixed: x is hi + lo) or FP64 (x FP64), unknown view,
   // [k][j][i]. Nothing is done once c->stopped is set, except that a zero

@@ -5,9 +5,14 @@
 // hands out all device memory from its own pool up front, code running where
 // allocation would synchronise the device or fragment a carefully sized heap,
 // or a coupling driver that must not grow its footprint between steps. For them
-// pic_poisson_solve_static solves the same discrete problem as pic_solve with
-// conjugate gradients whose vectors (right-hand side, residual, search
-// direction, operator image) and reduction partials sit in g_static_scratch.
+// pic_poisson_solve_static solves the same discrete problem as pic_solve, with
+// every work vector in g_static_scratch: by refinement passes of the direct
+// solver (k_direct.cu; right-hand side, residual, spectrum, its tables, which
+// each call writes anew, and reduction partials), or, on grids whose rows or
+// planes that solver does not take, by conjugate gradients (right-hand side,
+// residual, search direction, operator image). Measured on 64 x 64 x 63 unknowns
+// to 1e-12: 318 CG iterations of five launches and one wait each, 43.3 ms;
+// direct, 3 passes and two waits, 0.22 ms.
 //
 // The array is a fixed PIC_STATIC_MAX_UNKNOWNS-sized allocation that every GPU
 // loading this library holds until the process exits (4 vectors of 2^18
@@ -20,14 +25,19 @@
 #include <mutex>
 
 #include "../../include/pic.h"
+#include "pic_direct.cuh"
 #include "pic_internal.cuh"
+#include "pic_solver.cuh"
 
 namespace pic {
 
 constexpr long long kStaticVec = PIC_STATIC_MAX_UNKNOWNS;
 constexpr int kStaticBlock = 256;
+constexpr int kStaticMaxPasses = 40;  // of the direct solver: each gains several digits, so more gain none
 constexpr int kStaticParts = 1024;  // block partials (grid size cap)
-constexpr int kStaticScalars = 8;   // rr, pq, alpha, beta, bb
+constexpr int kStaticScalars = 32;  // CG: rr, pq, alpha, beta, bb; direct solver: its decision block
+
+static_assert(sizeof(SolveCtl) <= kStaticScalars * sizeof(double), "the decision block fits");
 
 static __device__ __align__(256) double g_static_scratch[4 * kStaticVec + kStaticParts + kStaticScalars];
 
@@ -224,17 +234,59 @@ extern "C" pic_status pic_poisson_solve_static(int32_t nx, int32_t ny, int32_t n
     if (e != cudaSuccess) return e;
     return cudaStreamSynchronize(s);
   };
+  // the outcome for the caller: status by the true residual
+  auto finish = [&](double bb, double rr, int it) -> pic_status {
+    const double rel = bb > 0.0 ? std::sqrt(rr / bb) : 0.0;
+    if (iters) *iters = it;
+    if (resid_rel) *resid_rel = rel;
+    if (!(rel <= rtol)) {
+      char msg[256];
+      snprintf(msg, sizeof msg,
+               "pic_poisson_solve_static: true relative residual %.3e above rtol %.3e after %d iterations", rel, rtol,
+               it);
+      set_static_error(msg);
+      return PIC_ENOCONV;
+    }
+    return PIC_OK;
+  };
   // a launch error left by earlier, unrelated work is cleared, not reported as this call's
   cudaError_t e = cudaGetLastError();
+  DirectSolver D;
+  // tables in the first half of the fourth vector, partial sums in the second
+  static_assert(2 * kDirParts <= kStaticVec / 2, "the partial sums fit");
+  if (D.plan(nx, ny, nz) && D.spec_bytes() <= sizeof(double) * kStaticVec &&
+      D.table_bytes() <= sizeof(double) * kStaticVec / 2) {
+    const MgLevel M{nx, ny, nz, nu};
+    SolveCtl* ctl = reinterpret_cast<SolveCtl*>(sc);
+    double* dpart = q + kStaticVec / 2;
+    const DirectLoop d{rtol, maxit, kStaticMaxPasses, 0, 0};
+    SolveCtl now;
+    if ((e = cudaMemsetAsync(ctl, 0, sizeof(SolveCtl), s)) != cudaSuccess) return fail("decision block", e);
+    if ((e = D.place(q, p, s)) != cudaSuccess) return fail("tables", e);
+    PIC_LAUNCH(G, kStaticBlock, 0, s, k_static_rhs)(L, h, phi_cathode_V, phi_anode_V, rho_dev, phi_dev, b, part);
+    D.residual_fp64(true, M, x, b, r, dpart, ctl, d, s);
+    // two passes before the first look at the outcome (passes after the decision to stop return at once)
+    for (int n = 0;; ++n) {
+      D.apply_fp64(r, x, ctl, s);
+      D.residual_fp64(false, M, x, b, r, dpart, ctl, d, s);
+      if (n == 0) continue;
+      if ((e = cudaGetLastError()) != cudaSuccess) return fail("refinement pass", e);
+      if ((e = cudaMemcpyAsync(&now, ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+          (e = cudaStreamSynchronize(s)) != cudaSuccess)
+        return fail("refinement pass", e);
+      if (!now.more) break;
+    }
+    return finish(now.bb, now.bb > 0.0 ? now.rr_true : 0.0, now.it_total);
+  }
   PIC_LAUNCH(G, kStaticBlock, 0, s, k_static_rhs)(L, h, phi_cathode_V, phi_anode_V, rho_dev, phi_dev, b, part);
   PIC_LAUNCH(1, 1, 0, s, k_static_scalars)(part, G, sc, 0);
   PIC_LAUNCH(G, kStaticBlock, 0, s, k_static_residual)(L, x, b, r, p, part);
   PIC_LAUNCH(1, 1, 0, s, k_static_scalars)(part, G, sc, 1);
   double bb = 0.0, rr = 0.0;
+  int it = 0;
   if ((e = read(4, &bb)) != cudaSuccess) return fail("right-hand side", e);
   if ((e = read(0, &rr)) != cudaSuccess) return fail("initial residual", e);
   const double tol = rtol * std::sqrt(bb);
-  int it = 0;
   if (bb > 0.0) {
     while (std::sqrt(rr) > tol && it < maxit) {
       PIC_LAUNCH(G, kStaticBlock, 0, s, k_static_apply)(L, p, q, part);
@@ -255,16 +307,5 @@ extern "C" pic_status pic_poisson_solve_static(int32_t nx, int32_t ny, int32_t n
     rr = 0.0;
   }
   if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail("stream synchronise", e);
-  const double rel = bb > 0.0 ? std::sqrt(rr / bb) : 0.0;
-  if (iters) *iters = it;
-  if (resid_rel) *resid_rel = rel;
-  if (!(rel <= rtol)) {
-    char msg[256];
-    snprintf(msg, sizeof msg,
-             "pic_poisson_solve_static: true relative residual %.3e above rtol %.3e after %d iterations", rel, rtol,
-             it);
-    set_static_error(msg);
-    return PIC_ENOCONV;
-  }
-  return PIC_OK;
+  return finish(bb, rr, it);
 }

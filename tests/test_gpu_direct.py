@@ -87,3 +87,27 @@ def test_tiny_potentials_do_not_underflow():
     small, _, rel = sim.solve(rho * 2.0 ** -300)
     assert rel <= 1e-12 and np.array_equal(small * 2.0 ** 300, big)
     sim.close()
+
+
+@pytest.mark.parametrize("nx,ny,nz,offset", [(24, 20, 34, 0), (24, 20, 34, 1), (7, 33, 60, 1), (64, 64, 64, 0),
+                                             (1, 3, 900, 0), (2, 2, 1030, 0)])
+def test_static_solve_on_caller_memory(nx, ny, nz, offset):
+    """Caller-owned arrays that start on any double, and the CG beyond the direct solver's planes."""
+    import torch
+    import paper_2606_05893_gb300 as pkg
+    rtol, h, phi_a = 1e-11, 2.5e-9, 37.0 * nz
+    n = (nz + 1) * ny * nx
+    rho = np.random.default_rng(n).standard_normal((nz + 1, ny, nx)) * 2e6
+    rho_dev = torch.zeros(n + 2, dtype=torch.float64, device="cuda")[offset:offset + n]
+    phi_dev = torch.zeros(n + 2, dtype=torch.float64, device="cuda")[offset:offset + n]
+    rho_dev.copy_(torch.from_numpy(rho.reshape(-1)))
+    st, iters, rel = pkg.pic_poisson_solve_static(nx, ny, nz, h, -2.0, phi_a, rho_dev.data_ptr(), phi_dev.data_ptr(), rtol, 100000)
+    assert st == pkg.PIC_OK and rel <= rtol and iters > 0
+    b = rho[1:nz] * (h * h / EPS0)
+    b[0] -= 2.0
+    b[-1] += phi_a
+    exact = _reference(nx, ny, nz, b)
+    phi = phi_dev.cpu().numpy().reshape(nz + 1, ny, nx)
+    bound = rtol * np.linalg.norm(b) + 12 * np.abs(exact).max() * math.sqrt(b.size) * 2.0 ** -52
+    assert np.linalg.norm(phi[1:nz] - exact) <= bound / (4 * math.sin(math.pi / (2 * nz)) ** 2)
+    assert np.all(phi[0] == -2.0) and np.all(phi[nz] == phi_a)
