@@ -19,7 +19,10 @@
 // the FP32 rate. A block holds 16 lines of an axis with the line index innermost
 // in shared memory, so every butterfly access of a half warp is one contiguous
 // 128-byte row whatever the radix (rows of 17 float2 in x, where the loads
-// transpose). Spectra stay in the order the passes leave them in (digit
+// transpose). What is left is latency: a tile is loaded by asynchronous copies,
+// all in flight at once, and the last kernel loads what it adds to in batches
+// before it stores (256x256x512: k_dir_xi 281 -> 170 us, k_dir_z with its pivots
+// in shared memory, two blocks an SM instead of one, 108 -> 71). Spectra stay in the order the passes leave them in (digit
 // reversed): the tridiagonal kernel only needs each column's eigenvalue.
 #include <algorithm>
 #include <cmath>
@@ -211,6 +214,16 @@ __device__ __forceinline__ float2* fft_tile(float2* Z, float2* Z2, const float2*
   return Z;
 }
 
+// Global to shared memory without a register in between, so that a thread has
+// its whole share of the tile in flight at once.
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "n"(BYTES)
+               : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 __device__ __forceinline__ void load_tw(float2* tw, const AxisPlan& A) {
   for (int m = threadIdx.x; m < A.n; m += kFftThreads) tw[m] = __ldg(A.tw + m);
 }
@@ -238,10 +251,20 @@ __global__ void __launch_bounds__(kFftThreads) k_dir_xf(DirectArgs a, const T* _
     const long long r = row0 + 2 * l;
     const T* pa = in + r * n;
     const bool va = r < a.rows, vb = r + 1 < a.rows;
-#pragma unroll 4
+    if constexpr (sizeof(T) == 4) {
+      if (vb) {
+        for (int i = lane; i < n; i += 32) {
+          copy_async<4>(&Z[i * kLpX + l].x, pa + i);
+          copy_async<4>(&Z[i * kLpX + l].y, pa + n + i);
+        }
+        continue;
+      }
+    }
+#pragma unroll 8
     for (int i = lane; i < n; i += 32)
       Z[i * kLpX + l] = make_float2(va ? scaled(pa[i], scale) : 0.f, vb ? scaled(pa[n + i], scale) : 0.f);
   }
+  if constexpr (sizeof(T) == 4) copy_async_wait();
   __syncthreads();
   Z = fft_tile<false, kLpX, POW2>(Z, Z + n * kLpX, tw, a.x);
   // the two rows' spectra from their packed line: A = (Z_f + conj Z_-f) / 2, B = (Z_f - conj Z_-f) / 2i
@@ -298,9 +321,11 @@ __global__ void __launch_bounds__(kFftThreads) k_dir_y(DirectArgs a, const Solve
   const int col0 = blockIdx.x * kDirLines, l = threadIdx.x & (kDirLines - 1);
   const bool in = col0 + l < a.C;
   float2* g = reinterpret_cast<float2*>(a.spec) + (long long)blockIdx.y * n * a.C + col0 + l;
-#pragma unroll 8
-  for (int y = threadIdx.x / kDirLines; y < n; y += kFftThreads / kDirLines)
-    Z[y * kLpY + l] = in ? g[(long long)y * a.C] : make_float2(0.f, 0.f);
+  for (int y = threadIdx.x / kDirLines; y < n; y += kFftThreads / kDirLines) {
+    if (in) copy_async<8>(&Z[y * kLpY + l], g + (long long)y * a.C);
+    else Z[y * kLpY + l] = make_float2(0.f, 0.f);
+  }
+  copy_async_wait();
   __syncthreads();
   const bool split = a.packed && col0 == 0;
   if (INV && split) {
@@ -318,14 +343,17 @@ __global__ void __launch_bounds__(kFftThreads) k_dir_y(DirectArgs a, const Solve
 }
 
 // What the last inverse transform does with d (already normalised): mixed,
-// (hi, lo) += d renormalised; FP64, x += d / scale.
+// (hi, lo) += d renormalised; FP64, x += d / scale. Loads and stores are apart,
+// so that a thread's loads are all in flight before its first store.
 struct AddMixed {
   float *hi, *lo;
   double phi_c, dphi_dk;
-  __device__ __forceinline__ void add(long long u, float d, double) const {
+  using Val = float2;
+  __device__ __forceinline__ Val load(long long u) const { return make_float2(hi[u], lo[u]); }
+  __device__ __forceinline__ void store(long long u, Val v, float d, double) const {
     float s, e;
-    two_sum(hi[u], d, s, e);
-    e = __fadd_rn(e, lo[u]);
+    two_sum(v.x, d, s, e);
+    e = __fadd_rn(e, v.y);
     const float h2 = __fadd_rn(s, e);
     hi[u] = h2;
     lo[u] = __fsub_rn(e, __fsub_rn(h2, s));
@@ -339,7 +367,11 @@ struct AddMixed {
 };
 struct Add64 {
   double* x;
-  __device__ __forceinline__ void add(long long u, float d, double inv_scale) const { x[u] += (double)d * inv_scale; }
+  using Val = double;
+  __device__ __forceinline__ Val load(long long u) const { return x[u]; }
+  __device__ __forceinline__ void store(long long u, Val v, float d, double inv_scale) const {
+    x[u] = v + (double)d * inv_scale;
+  }
   __device__ __forceinline__ void zero(long long u, int) const { x[u] = 0.0; }
 };
 
@@ -363,7 +395,7 @@ __global__ void __launch_bounds__(kFftThreads) k_dir_xi(DirectArgs a, Add add, c
   for (int l = w; l < kDirLines; l += kFftThreads / 32) {
     const long long r = row0 + 2 * l;
     const bool va = r < a.rows, vb = r + 1 < a.rows;
-#pragma unroll 2
+#pragma unroll 4
     for (int f = lane; f < a.C; f += 32) {
       const float2 A = va ? spec[r * a.C + f] : make_float2(0.f, 0.f);
       const float2 B = vb ? spec[(r + 1) * a.C + f] : make_float2(0.f, 0.f);
@@ -382,11 +414,25 @@ __global__ void __launch_bounds__(kFftThreads) k_dir_xi(DirectArgs a, Add add, c
   for (int l = w; l < kDirLines; l += kFftThreads / 32) {
     const long long r = row0 + 2 * l;
     const bool va = r < a.rows, vb = r + 1 < a.rows;
-#pragma unroll 4
-    for (int i = lane; i < n; i += 32) {
-      const float2 d = Z[i * kLpX + l];
-      if (va) add.add(r * n + i, d.x * a.norm, inv_scale);
-      if (vb) add.add((r + 1) * n + i, d.y * a.norm, inv_scale);
+    if (!va) break;
+    constexpr int B = 4;  // points of both rows a thread loads before it stores any
+    for (int i0 = lane; i0 < n; i0 += 32 * B) {
+      typename Add::Val xa[B] = {}, xb[B] = {};
+#pragma unroll
+      for (int q = 0; q < B; ++q) {
+        const int i = i0 + 32 * q;
+        if (i >= n) break;
+        xa[q] = add.load(r * n + i);
+        if (vb) xb[q] = add.load((r + 1) * n + i);
+      }
+#pragma unroll
+      for (int q = 0; q < B; ++q) {
+        const int i = i0 + 32 * q;
+        if (i >= n) break;
+        const float2 d = Z[i * kLpX + l];
+        add.store(r * n + i, xa[q], d.x * a.norm, inv_scale);
+        if (vb) add.store((r + 1) * n + i, xb[q], d.y * a.norm, inv_scale);
+      }
     }
   }
 }
@@ -399,8 +445,8 @@ __global__ void __launch_bounds__(kFftThreads) k_dir_xi(DirectArgs a, Add add, c
 // the chunks' first and last values then satisfy a recurrence that warp 0 solves
 // along the chunks, and each warp adds the response to its two outer neighbours.
 // Planes stay in registers in between, so the spectrum is read and written once.
-template <int M, int THREADS>
-__global__ void __launch_bounds__(THREADS) k_dir_z(DirectArgs a, const SolveCtl* c) {
+template <int M, int THREADS, int BLOCKS>
+__global__ void __launch_bounds__(THREADS, BLOCKS) k_dir_z(DirectArgs a, const SolveCtl* c) {
   pdl_enter();
   if (c->stopped) return;
   extern __shared__ float zs[];
@@ -409,30 +455,28 @@ __global__ void __launch_bounds__(THREADS) k_dir_z(DirectArgs a, const SolveCtl*
   float* sE = sF + 32 * W;       // last value with zero neighbours, then the left neighbour's value
   float* sD = sE + 32 * W;       // response of the first value to the right neighbour
   float* sV = sD + 32 * W;
-  float* sC = sV + 32 * W;       // [M][32] the pivots, where registers do not hold them
+  float* sC = sV + 32 * W;       // [M][32] the pivots and, after them, their product
   const int col = blockIdx.x * 32 + lane;
   const bool in = col < a.plane;
   const int k0 = w * M, len = min(M, a.P - k0);
   float* g = a.spec + (long long)k0 * a.plane + col;
-  constexpr bool kShared = THREADS > 512;  // 64 registers a thread hold the planes alone
-  float y[M], cr[M] = {};
-  auto cp = [&](int k) -> float {
-    if constexpr (kShared) return *(volatile float*)(sC + 32 * k);  // reloaded at each use
-    else return cr[k];
-  };
+  float y[M];
+  // reloaded at each use: registers then hold the planes alone
+  auto cp = [&](int k) -> float { return *(volatile float*)(sC + 32 * k); };
 #pragma unroll
   for (int k = 0; k < M; ++k) y[k] = in && k < len ? g[(long long)k * a.plane] : 0.f;
-  const float lam = in ? __ldg(a.lam + col) : 1.f;
-  float s = lam + 1.f, b = 1.f;
-#pragma unroll
-  for (int k = 0; k < M; ++k) {
-    const float v = 1.f / (1.f + s);
-    if (kShared) sC[32 * k] = v;  // every warp writes the same value
-    else cr[k] = v;
-    s = fmaf(s, v, lam);
-    b *= v;
+  if (w == 0) {
+    const float lam = in ? __ldg(a.lam + col) : 1.f;
+    float s = lam + 1.f, b = 1.f;
+    for (int k = 0; k < M; ++k) {
+      const float v = 1.f / (1.f + s);
+      sC[32 * k] = v;
+      s = fmaf(s, v, lam);
+      b *= v;
+    }
+    sC[32 * M] = b;
   }
-  if (kShared) __syncwarp();
+  __syncthreads();
   float t = 0.f;
 #pragma unroll
   for (int k = 0; k < M; ++k) {
@@ -450,12 +494,10 @@ __global__ void __launch_bounds__(THREADS) k_dir_z(DirectArgs a, const SolveCtl*
     // and the far end), L the left chunk's E, R the right chunk's F. With
     // L = u + v F: F = (pF + a u + b R) / (1 - a v), and u, v of the next chunk.
     const int last = a.P - (W - 1) * M;  // planes of the last chunk
-    float alast = cp(0);
-#pragma unroll
-    for (int k = 1; k < M; ++k) alast = k < last ? cp(k) : alast;
+    const float alast = cp(last - 1), afull = cp(M - 1), b = cp(M);
     float u = 0.f, v = 0.f;
     for (int q = 0; q < W; ++q) {
-      const float aq = q == W - 1 ? alast : cp(M - 1), bq = q == W - 1 ? 0.f : b;
+      const float aq = q == W - 1 ? alast : afull, bq = q == W - 1 ? 0.f : b;
       const float inv = 1.f / fmaf(-aq, v, 1.f);
       const float F = fmaf(aq, u, sF[32 * q]) * inv, D = bq * inv, pE = sE[32 * q];
       sF[32 * q] = F;
@@ -617,7 +659,7 @@ __device__ __forceinline__ void vstore(T* p, const T (&v)[V]) {
 // through kc planes: a plane is loaded once as the upper neighbour and kept in
 // registers as the centre and the lower one, so a point costs one load of its
 // own plane instead of three.
-constexpr int kResX = 32, kResY = 8;
+constexpr int kResThreads = 256;  // 8, 16 or 32 lanes along x, the rest along y
 struct ResGeom {
   Lv L;
   int kc;         // planes per block
@@ -628,14 +670,14 @@ struct ResGeom {
 // comment of the MIXED solver), r.r and, FIRST, b.b with the folded electrode
 // terms. V = 4 where rows are whole float4s.
 template <int V, bool FIRST>
-__global__ void __launch_bounds__(kResX* kResY) k_dir_resid_ff(ResGeom G, const float* __restrict__ hi,
+__global__ void __launch_bounds__(kResThreads) k_dir_resid_ff(ResGeom G, const float* __restrict__ hi,
                                                               const float* __restrict__ lo, const float* __restrict__ f,
                                                               float* __restrict__ r, float fold_first, float fold_last,
                                                               double* part, SolveCtl* c, DirectLoop d) {
   pdl_enter();
   if (!FIRST && c->stopped) return;
   const Lv& L = G.L;
-  const int i = (blockIdx.x * kResX + threadIdx.x) * V, j = blockIdx.y * kResY + threadIdx.y;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) * V, j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k0 = blockIdx.z * G.kc, kend = min(k0 + G.kc, L.nz - 1);
   float rr = 0.f, bb = 0.f;
   if (i < L.nx && j < L.ny) {
@@ -716,13 +758,13 @@ __global__ void __launch_bounds__(kResX* kResY) k_dir_resid_ff(ResGeom G, const 
 
 // r = b - A x in FP64, r.r and, FIRST, b.b
 template <int V, bool FIRST>
-__global__ void __launch_bounds__(kResX* kResY) k_dir_resid64(ResGeom G, const double* __restrict__ x,
+__global__ void __launch_bounds__(kResThreads) k_dir_resid64(ResGeom G, const double* __restrict__ x,
                                                              const double* __restrict__ b, double* __restrict__ r,
                                                              double* part, SolveCtl* c, DirectLoop d) {
   pdl_enter();
   if (!FIRST && c->stopped) return;
   const Lv& L = G.L;
-  const int i = (blockIdx.x * kResX + threadIdx.x) * V, j = blockIdx.y * kResY + threadIdx.y;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) * V, j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k0 = blockIdx.z * G.kc, kend = min(k0 + G.kc, L.nz - 1);
   double rr = 0.0, bb = 0.0;
   if (i < L.nx && j < L.ny) {
@@ -935,32 +977,39 @@ void apply(const DirectSolver& D, const T* r, const Add& add, const SolveCtl* c,
   const dim3 gx((unsigned)((a.rows + 2 * kDirLines - 1) / (2 * kDirLines)));
   const dim3 gy((a.C + kDirLines - 1) / kDirLines, a.P);
   const dim3 gz((a.plane + 31) / 32);
-  const size_t zsm = sizeof(float) * 32 * (4 * D.zw + (D.zw > 16 ? D.zm : 0));
+  const size_t zsm = sizeof(float) * 32 * (4 * D.zw + D.zm + 1);
   if (a.x.pow2) SOLVER_LAUNCH(gx, kFftThreads, D.smem_x, s, k_dir_xf<T, true>)(a, r, c);
   else SOLVER_LAUNCH(gx, kFftThreads, D.smem_x, s, k_dir_xf<T, false>)(a, r, c);
   if (a.y.pow2) SOLVER_LAUNCH(gy, kFftThreads, D.smem_y, s, k_dir_y<false, true>)(a, c);
   else SOLVER_LAUNCH(gy, kFftThreads, D.smem_y, s, k_dir_y<false, false>)(a, c);
-  if (D.zm == 16) SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<16, 512>)(a, c);
-  else if (D.zw <= 16) SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<32, 512>)(a, c);
-  else SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<32, 1024>)(a, c);
+  if (D.zm == 16) SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<16, 512, 3>)(a, c);
+  else if (D.zw <= 16) SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<32, 512, 2>)(a, c);
+  else SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<32, 1024, 1>)(a, c);
   if (a.y.pow2) SOLVER_LAUNCH(gy, kFftThreads, D.smem_y, s, k_dir_y<true, true>)(a, c);
   else SOLVER_LAUNCH(gy, kFftThreads, D.smem_y, s, k_dir_y<true, false>)(a, c);
   if (a.x.pow2) SOLVER_LAUNCH(gx, kFftThreads, D.smem_x, s, k_dir_xi<Add, true>)(a, add, c);
   else SOLVER_LAUNCH(gx, kFftThreads, D.smem_x, s, k_dir_xi<Add, false>)(a, add, c);
 }
 
-// planes per block of the residual kernels: a few blocks per SM, at most 8 planes
-// (longer marches save little: 1 + 2 / kc plane loads per point)
-ResGeom res_geom(const MgLevel& M, int V, dim3* grid) {
+// points per thread: a vector of a row, or one where vectors would leave SMs without a block
+int res_vec(const MgLevel& M, int V, bool aligned) {
+  return aligned && M.nu >= 2ll * sm_count() * kResThreads * V ? V : 1;
+}
+
+// block shape and planes per block of the residual kernels: a few blocks per SM,
+// at most 8 planes (longer marches save little: 1 + 2 / kc plane loads per point)
+ResGeom res_geom(const MgLevel& M, int V, dim3* grid, dim3* block) {
   ResGeom G{lv_of(M), 1, M.nu};
-  const int P = M.nz - 1;
-  const unsigned gx = (unsigned)((M.nx / V + kResX - 1) / kResX), gy = (unsigned)((M.ny + kResY - 1) / kResY);
+  const int P = M.nz - 1, vx = M.nx / V;
+  const unsigned bx = vx <= 8 ? 8 : (vx <= 16 ? 16 : 32), by = kResThreads / bx;
+  const unsigned gx = (vx + bx - 1) / bx, gy = (M.ny + by - 1) / by;
   int kc = 8;
   while (kc > 1 && (long long)gx * gy * ((P + kc - 1) / kc) < 6ll * sm_count()) kc >>= 1;
   // the partial sums of a block are a double2 each
   while ((long long)gx * gy * ((P + kc - 1) / kc) > kDirParts) kc *= 2;
   G.kc = kc;
   *grid = dim3(gx, gy, (unsigned)((P + kc - 1) / kc));
+  *block = dim3(bx, by);
   return G;
 }
 
@@ -979,10 +1028,9 @@ void DirectSolver::residual_mixed(bool first, const MgLevel& M, const float* hi,
                                   float fold_first, float fold_last, double* part, SolveCtl* c, const DirectLoop& d,
                                   cudaStream_t s) const {
   // float4 rows: hi starts one plane into phi32, so its rows are aligned when nx is a multiple of 4
-  const bool v4 = M.nx % 4 == 0;
-  dim3 g;
-  const ResGeom G = res_geom(M, v4 ? 4 : 1, &g);
-  const dim3 b(kResX, kResY);
+  const bool v4 = res_vec(M, 4, M.nx % 4 == 0) == 4;
+  dim3 g, b;
+  const ResGeom G = res_geom(M, v4 ? 4 : 1, &g, &b);
   if (v4 && first)
     SOLVER_LAUNCH(g, b, 0, s, k_dir_resid_ff<4, true>)(G, hi, lo, f, r, fold_first, fold_last, part, c, d);
   else if (v4)
@@ -996,10 +1044,9 @@ void DirectSolver::residual_mixed(bool first, const MgLevel& M, const float* hi,
 void DirectSolver::residual_fp64(bool first, const MgLevel& M, const double* x, const double* b, double* r, double* part,
                                  SolveCtl* c, const DirectLoop& d, cudaStream_t s) const {
   // double2 rows: the caller's own array may start anywhere on a double
-  const bool v2 = M.nx % 2 == 0 && ((uintptr_t)x | (uintptr_t)b | (uintptr_t)r) % 16 == 0;
-  dim3 g;
-  const ResGeom G = res_geom(M, v2 ? 2 : 1, &g);
-  const dim3 bl(kResX, kResY);
+  const bool v2 = res_vec(M, 2, M.nx % 2 == 0 && ((uintptr_t)x | (uintptr_t)b | (uintptr_t)r) % 16 == 0) == 2;
+  dim3 g, bl;
+  const ResGeom G = res_geom(M, v2 ? 2 : 1, &g, &bl);
   if (v2 && first) SOLVER_LAUNCH(g, bl, 0, s, k_dir_resid64<2, true>)(G, x, b, r, part, c, d);
   else if (v2) SOLVER_LAUNCH(g, bl, 0, s, k_dir_resid64<2, false>)(G, x, b, r, part, c, d);
   else if (first) SOLVER_LAUNCH(g, bl, 0, s, k_dir_resid64<1, true>)(G, x, b, r, part, c, d);
