@@ -39,7 +39,8 @@ namespace pic {
 
 namespace {
 
-constexpr int kFftThreads = 128;
+constexpr int kFftThreads = 256;  // most threads of an FFT block: x tiles above 128 points (k_dir_xi 170 -> 148 us
+                                  // at 256x256x512); the others 128 (y tiles with 256: 55 -> 65 us)
 constexpr int kLpX = kDirLines + 1;  // row pitch (float2) of the x tiles
 constexpr int kLpY = kDirLines;
 
@@ -133,7 +134,7 @@ __device__ __forceinline__ void dft_odd(float2 (&v)[R], const float2* w, int ste
 template <int R, bool INV, int LP>
 __device__ __forceinline__ void fft_pass(float2* Z, const float2* tw, int n, int L, const FastDiv& dM) {
   const int M = dM.d, nb = n / R, step = n / L, st = M * LP;
-  for (int t = threadIdx.x; t < nb * kDirLines; t += kFftThreads) {
+  for (int t = threadIdx.x; t < nb * kDirLines; t += blockDim.x) {
     const int l = t & (kDirLines - 1), b = t / kDirLines;
     const int s = fdiv(b, dM), j = b - s * M;
     float2* z = Z + (s * L + j) * LP + l;
@@ -159,7 +160,7 @@ __device__ __forceinline__ void fft_pass(float2* Z, const float2* tw, int n, int
 template <bool INV, int LP>
 __device__ void fft_pass_any(const float2* Z, float2* Z2, const float2* tw, int n, int R, int L, const FastDiv& dM) {
   const int M = dM.d, step = n / L, root = n / R;
-  for (int t = threadIdx.x; t < n * kDirLines; t += kFftThreads) {
+  for (int t = threadIdx.x; t < n * kDirLines; t += blockDim.x) {
     const int l = t & (kDirLines - 1), e = t / kDirLines;
     const int qs = fdiv(e, dM), j = e - qs * M;  // e = (s R + q) M + j
     const int s = qs / R, q = qs - s * R;
@@ -225,7 +226,7 @@ __device__ __forceinline__ void copy_async(void* dst, const void* src) {
 __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 __device__ __forceinline__ void load_tw(float2* tw, const AxisPlan& A) {
-  for (int m = threadIdx.x; m < A.n; m += kFftThreads) tw[m] = __ldg(A.tw + m);
+  for (int m = threadIdx.x; m < A.n; m += blockDim.x) tw[m] = __ldg(A.tw + m);
 }
 
 // Rows 2q and 2q + 1 as real and imaginary part; scale applied in FP64 to FP64 input.
@@ -236,7 +237,7 @@ __device__ __forceinline__ float scaled(T v, double scale) {
 }
 
 template <class T, bool POW2>
-__global__ void __launch_bounds__(kFftThreads) k_dir_xf(DirectArgs a, const T* __restrict__ in, const SolveCtl* c) {
+__global__ void __launch_bounds__(kFftThreads, 3) k_dir_xf(DirectArgs a, const T* __restrict__ in, const SolveCtl* c) {
   pdl_enter();
   if (c->stopped) return;
   extern __shared__ __align__(16) float2 sm[];
@@ -247,7 +248,7 @@ __global__ void __launch_bounds__(kFftThreads) k_dir_xf(DirectArgs a, const T* _
   const long long row0 = 2ll * kDirLines * blockIdx.x;
   const double scale = sizeof(T) == 8 ? c->scale : 1.0;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int l = w; l < kDirLines; l += kFftThreads / 32) {
+  for (int l = w; l < kDirLines; l += (int)blockDim.x / 32) {
     const long long r = row0 + 2 * l;
     const T* pa = in + r * n;
     const bool va = r < a.rows, vb = r + 1 < a.rows;
@@ -269,7 +270,7 @@ __global__ void __launch_bounds__(kFftThreads) k_dir_xf(DirectArgs a, const T* _
   Z = fft_tile<false, kLpX, POW2>(Z, Z + n * kLpX, tw, a.x);
   // the two rows' spectra from their packed line: A = (Z_f + conj Z_-f) / 2, B = (Z_f - conj Z_-f) / 2i
   float2* out = reinterpret_cast<float2*>(a.spec);
-  for (int l = w; l < kDirLines; l += kFftThreads / 32) {
+  for (int l = w; l < kDirLines; l += (int)blockDim.x / 32) {
     const long long r = row0 + 2 * l;
     if (r >= a.rows) break;
     const bool vb = r + 1 < a.rows;
@@ -296,7 +297,7 @@ __global__ void __launch_bounds__(kFftThreads) k_dir_xf(DirectArgs a, const T* _
 // and -g are combined into the two coefficients' own spectra (and back).
 template <bool INV>
 __device__ __forceinline__ void split_packed(float2* Z, const AxisPlan& A) {
-  for (int g = 1 + threadIdx.x; 2 * g < A.n; g += kFftThreads) {
+  for (int g = 1 + threadIdx.x; 2 * g < A.n; g += blockDim.x) {
     float2 &p = Z[__ldg(A.pos + g) * kLpY], &m = Z[__ldg(A.pos + A.n - g) * kLpY];
     const float2 u = p, v = m;
     if (!INV) {
@@ -310,7 +311,7 @@ __device__ __forceinline__ void split_packed(float2* Z, const AxisPlan& A) {
 }
 
 template <bool INV, bool POW2>
-__global__ void __launch_bounds__(kFftThreads) k_dir_y(DirectArgs a, const SolveCtl* c) {
+__global__ void __launch_bounds__(kFftThreads, 3) k_dir_y(DirectArgs a, const SolveCtl* c) {
   pdl_enter();
   if (c->stopped) return;
   extern __shared__ __align__(16) float2 sm[];
@@ -321,7 +322,7 @@ __global__ void __launch_bounds__(kFftThreads) k_dir_y(DirectArgs a, const Solve
   const int col0 = blockIdx.x * kDirLines, l = threadIdx.x & (kDirLines - 1);
   const bool in = col0 + l < a.C;
   float2* g = reinterpret_cast<float2*>(a.spec) + (long long)blockIdx.y * n * a.C + col0 + l;
-  for (int y = threadIdx.x / kDirLines; y < n; y += kFftThreads / kDirLines) {
+  for (int y = threadIdx.x / kDirLines; y < n; y += (int)blockDim.x / kDirLines) {
     if (in) copy_async<8>(&Z[y * kLpY + l], g + (long long)y * a.C);
     else Z[y * kLpY + l] = make_float2(0.f, 0.f);
   }
@@ -339,7 +340,7 @@ __global__ void __launch_bounds__(kFftThreads) k_dir_y(DirectArgs a, const Solve
   }
   if (!in) return;
 #pragma unroll 8
-  for (int y = threadIdx.x / kDirLines; y < n; y += kFftThreads / kDirLines) g[(long long)y * a.C] = Z[y * kLpY + l];
+  for (int y = threadIdx.x / kDirLines; y < n; y += (int)blockDim.x / kDirLines) g[(long long)y * a.C] = Z[y * kLpY + l];
 }
 
 // What the last inverse transform does with d (already normalised): mixed,
@@ -376,14 +377,14 @@ struct Add64 {
 };
 
 template <class Add, bool POW2>
-__global__ void __launch_bounds__(kFftThreads) k_dir_xi(DirectArgs a, Add add, const SolveCtl* c) {
+__global__ void __launch_bounds__(kFftThreads, 3) k_dir_xi(DirectArgs a, Add add, const SolveCtl* c) {
   pdl_enter();
   const long long row0 = 2ll * kDirLines * blockIdx.x;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int n = a.nx;
   if (c->stopped) {
     if (c->bb != 0.0) return;
-    for (long long r = row0 + w; r < row0 + 2 * kDirLines && r < a.rows; r += kFftThreads / 32)  // b = 0: x = 0
+    for (long long r = row0 + w; r < row0 + 2 * kDirLines && r < a.rows; r += (int)blockDim.x / 32)  // b = 0: x = 0
       for (int i = lane; i < n; i += 32) add.zero(r * n + i, (int)(r / a.ny));
     return;
   }
@@ -392,7 +393,7 @@ __global__ void __launch_bounds__(kFftThreads) k_dir_xi(DirectArgs a, Add add, c
   float2* Z = sm + n;
   load_tw(tw, a.x);
   const float2* spec = reinterpret_cast<const float2*>(a.spec);
-  for (int l = w; l < kDirLines; l += kFftThreads / 32) {
+  for (int l = w; l < kDirLines; l += (int)blockDim.x / 32) {
     const long long r = row0 + 2 * l;
     const bool va = r < a.rows, vb = r + 1 < a.rows;
 #pragma unroll 4
@@ -411,7 +412,7 @@ __global__ void __launch_bounds__(kFftThreads) k_dir_xi(DirectArgs a, Add add, c
   __syncthreads();
   Z = fft_tile<true, kLpX, POW2>(Z, Z + n * kLpX, tw, a.x);
   const double inv_scale = c->inv_scale;
-  for (int l = w; l < kDirLines; l += kFftThreads / 32) {
+  for (int l = w; l < kDirLines; l += (int)blockDim.x / 32) {
     const long long r = row0 + 2 * l;
     const bool va = r < a.rows, vb = r + 1 < a.rows;
     if (!va) break;
@@ -977,18 +978,19 @@ void apply(const DirectSolver& D, const T* r, const Add& add, const SolveCtl* c,
   const dim3 gx((unsigned)((a.rows + 2 * kDirLines - 1) / (2 * kDirLines)));
   const dim3 gy((a.C + kDirLines - 1) / kDirLines, a.P);
   const dim3 gz((a.plane + 31) / 32);
+  const int tx = a.nx > 128 ? kFftThreads : kFftThreads / 2, ty = kFftThreads / 2;
   const size_t zsm = sizeof(float) * 32 * (4 * D.zw + D.zm + 1);
-  if (a.x.pow2) SOLVER_LAUNCH(gx, kFftThreads, D.smem_x, s, k_dir_xf<T, true>)(a, r, c);
-  else SOLVER_LAUNCH(gx, kFftThreads, D.smem_x, s, k_dir_xf<T, false>)(a, r, c);
-  if (a.y.pow2) SOLVER_LAUNCH(gy, kFftThreads, D.smem_y, s, k_dir_y<false, true>)(a, c);
-  else SOLVER_LAUNCH(gy, kFftThreads, D.smem_y, s, k_dir_y<false, false>)(a, c);
+  if (a.x.pow2) SOLVER_LAUNCH(gx, tx, D.smem_x, s, k_dir_xf<T, true>)(a, r, c);
+  else SOLVER_LAUNCH(gx, tx, D.smem_x, s, k_dir_xf<T, false>)(a, r, c);
+  if (a.y.pow2) SOLVER_LAUNCH(gy, ty, D.smem_y, s, k_dir_y<false, true>)(a, c);
+  else SOLVER_LAUNCH(gy, ty, D.smem_y, s, k_dir_y<false, false>)(a, c);
   if (D.zm == 16) SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<16, 512, 3>)(a, c);
   else if (D.zw <= 16) SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<32, 512, 2>)(a, c);
   else SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<32, 1024, 1>)(a, c);
-  if (a.y.pow2) SOLVER_LAUNCH(gy, kFftThreads, D.smem_y, s, k_dir_y<true, true>)(a, c);
-  else SOLVER_LAUNCH(gy, kFftThreads, D.smem_y, s, k_dir_y<true, false>)(a, c);
-  if (a.x.pow2) SOLVER_LAUNCH(gx, kFftThreads, D.smem_x, s, k_dir_xi<Add, true>)(a, add, c);
-  else SOLVER_LAUNCH(gx, kFftThreads, D.smem_x, s, k_dir_xi<Add, false>)(a, add, c);
+  if (a.y.pow2) SOLVER_LAUNCH(gy, ty, D.smem_y, s, k_dir_y<true, true>)(a, c);
+  else SOLVER_LAUNCH(gy, ty, D.smem_y, s, k_dir_y<true, false>)(a, c);
+  if (a.x.pow2) SOLVER_LAUNCH(gx, tx, D.smem_x, s, k_dir_xi<Add, true>)(a, add, c);
+  else SOLVER_LAUNCH(gx, tx, D.smem_x, s, k_dir_xi<Add, false>)(a, add, c);
 }
 
 // points per thread: a vector of a row, or one where vectors would leave SMs without a block

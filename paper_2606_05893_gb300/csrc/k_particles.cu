@@ -875,7 +875,7 @@ __global__ void k_resolve_apply(ApplyArgs<S> a) {
     a.ev_head[c] = -1;
     a.cand_head[c] = -1;
   }
-  // the last block to finish commits the step's counts (every block has read them)
+  // the last block to finish commits the step's counts (every block has read them) and ends the step
   __shared__ bool s_last;
   __threadfence();
   __syncthreads();
@@ -884,6 +884,7 @@ __global__ void k_resolve_apply(ApplyArgs<S> a) {
   if (s_last && threadIdx.x == 0) {
     __threadfence();
     resolve_commit(a.cnt, a.commit);
+    step_end(a.cnt, a.circ);
     a.cnt->resolve_ticket = 0u;
   }
 }

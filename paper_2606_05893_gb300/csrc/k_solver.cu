@@ -1563,6 +1563,7 @@ __global__ void __launch_bounds__(256) k_phi_from_ff(Lv L, const float* __restri
                                                      double* __restrict__ x, double phi_c, double dphi_dk) {
   pdl_enter();
   const double vac = phi_c + dphi_dk * (double)(blockIdx.z + 1);
+
   ROWS3(L, L.nx) {
     if (!in_x) continue;
     const int u = k * L.pl + j * L.nx + i;

@@ -840,6 +840,20 @@ NextDeposit next_deposit_of(const Instance* I, bool on) {
   return nd;
 }
 
+template <class T>
+StepClear<T> step_clear(const Instance* I, T* rho_next) {
+  StepClear<T> sc{};
+  sc.cnt = I->cnt;
+  sc.nsp = I->nsp;
+  sc.rho = rho_next;
+  sc.background = (T)I->cfg.rho_background;
+  for (int s = 0; s < I->nsp; ++s) {
+    sc.out[s] = I->cur[s] ^ 1;
+    if (I->ncount_next[s]) sc.ncount[sc.nclear++] = I->ncount_next[s];
+  }
+  return sc;
+}
+
 template <class S>
 pic_status step_instance(pic_handle* h, Instance* I) {
   cudaStream_t st = I->stream;
@@ -918,13 +932,6 @@ pic_status step_instance(pic_handle* h, Instance* I) {
     }
 
   }
-  // this step's kernels accumulate the next deposit here
-  if (I->mixed)
-    launch_fill32(I->rho32_next, g.nnode, (float)I->cfg.rho_background, st);
-  else
-    launch_fill64(I->rho64_next, g.nnode, I->cfg.rho_background, st);
-  for (int s = 0; s < I->nsp; ++s)
-    if (I->ncount_next[s]) CK(h, cudaMemsetAsync(I->ncount_next[s], 0, sizeof(int32_t) * g.ncell, st));
   T.end(st);
   // a4 Poisson solve
   T.begin(PIC_PH_SOLVE, st);
@@ -961,17 +968,15 @@ pic_status step_instance(pic_handle* h, Instance* I) {
   {
     const int ft = field_count_target(I);
     const int32_t* nc = ft >= 0 ? I->ncount[ft] : nullptr;
+    // with it the accumulators that this step's kernels add to
     if (I->mixed)
-      launch_efield32f(g, I->phi32, I->E32, nc, st);
+      launch_efield32f(g, I->phi32, I->E32, nc, step_clear<float>(I, I->rho32_next), st);
     else
-      launch_efield64(g, I->phi, I->E64, nc, st);
+      launch_efield64(g, I->phi, I->E64, nc, step_clear<double>(I, I->rho64_next), st);
   }
   T.end(st);
 
   // a6-a8 + a10 push / absorb / collide / compact: charged species first, then neutrals
-  int outb[kMaxSpecies];
-  for (int s = 0; s < I->nsp; ++s) outb[s] = I->cur[s] ^ 1;
-  launch_step_begin(I->cnt, outb, I->nsp, st);
   for (int pass = 0; pass < 2; ++pass) {
     for (int s = 0; s < I->nsp; ++s) {
       const bool neutral = I->species[s].role == PIC_NEUTRAL;
@@ -1079,10 +1084,12 @@ pic_status step_instance(pic_handle* h, Instance* I) {
     rc.n_cap = ap.n_cap;
     rc.ev_cap = I->ev_cap;
     rc.weighted = I->weighted ? 1 : 0;
-    launch_resolve_apply<S>(ap, rb, st);  // with the commit and the list-head reset
+    ap.circ = I->circ;
+    launch_resolve_apply<S>(ap, rb, st);  // with the commit, the list-head reset and the end of the step
     T.end(st);
+  } else {
+    launch_step_end(I->cnt, I->circ, st);
   }
-  launch_step_end(I->cnt, I->circ, st);
   for (int s = 0; s < I->nsp; ++s) I->cur[s] ^= 1;
   I->step += 1;
   I->next_valid = true;

@@ -516,10 +516,37 @@ struct McArgs {
   int count_in_field;  // all channels share one target: its cell count rides in E.w
 };
 
-struct StepBegin {
+// What a step's particle kernels add to, readied by the field kernel before
+// them: the next step's density and neutral counts, and the step's counters.
+template <class T>
+struct StepClear {
+  DevCounters* cnt;
   int nsp;
-  int out[kMaxSpecies];
+  int out[kMaxSpecies];  // output buffer of every species
+  T* rho;                // next density, over the nodes
+  T background;
+  int nclear;            // neutral species
+  int32_t* ncount[kMaxSpecies];
 };
+template <class T>
+__device__ __forceinline__ void step_begin(const StepClear<T>& sc) {
+  DevCounters* cnt = sc.cnt;
+  for (int s = 0; s < sc.nsp; ++s) cnt->n[sc.out[s]][s] = 0;
+  cnt->n_events = 0;
+  cnt->n_success = 0;
+  cnt->n_success_cx = 0;
+  cnt->n_cands = 0;
+  cnt->q_cathode_step = 0.0;
+  cnt->q_anode_step = 0.0;
+}
+// The step is complete: the circuit moves the anode, the step index advances.
+__device__ __forceinline__ void step_end(DevCounters* cnt, const Circuit& c) {
+  if (c.on) {
+    const double dv = (c.dt * (c.V0 - cnt->anode_V) / c.R + cnt->q_anode_step) / c.C;
+    cnt->anode_V += dv;
+  }
+  cnt->step += 1u;
+}
 
 struct InjSrc {
   int species;
@@ -630,6 +657,7 @@ struct ApplyArgs {
   int32_t* ev_head;      // per-cell list heads, emptied for the next step
   int32_t* cand_head;
   ResolveCommit commit;  // applied by the launch's last block
+  Circuit circ;          // and the end of the step
 };
 
 
@@ -667,11 +695,12 @@ void launch_rhs(const Grid& g, const DevCounters* cnt, const double* rho64, cons
                 cudaStream_t st);
 void launch_rhs_f32(const Grid& g, const DevCounters* cnt, const double* rho64, const float* rho32, float* f,
                     float* phi32, cudaStream_t st);
-void launch_efield64(const Grid& g, const double* phi, double4_32a* E, const int32_t* ncount, cudaStream_t st);
-void launch_efield32f(const Grid& g, const float* phi32, float4* E, const int32_t* ncount, cudaStream_t st);
+void launch_efield64(const Grid& g, const double* phi, double4_32a* E, const int32_t* ncount,
+                     const StepClear<double>& sc, cudaStream_t st);
+void launch_efield32f(const Grid& g, const float* phi32, float4* E, const int32_t* ncount, const StepClear<float>& sc,
+                      cudaStream_t st);
 void launch_phi_planes(const Grid& g, const DevCounters* cnt, double* phi, cudaStream_t st);
 void launch_planes_from_ff(const Grid& g, const float* phi32, double* phi, cudaStream_t st);
-void launch_step_begin(DevCounters* cnt, const int* out_buf, int nsp, cudaStream_t st);
 
 template <class S>
 void launch_load(const Grid& g, S st, DevCounters* cnt, int cur, int species, long long cap, const double* x,
