@@ -75,6 +75,7 @@ struct unet_handle {
   unet::Tensor GD0, GD0A, GU0, GE0S, GE0, GE0A, GD1, GD1A, GU1, GE1S, GP1, GE1, GE1A, GD2, GD2A, GU2, GE2S, GP2, GE2,
       GE2A, GE3, GE3A, GP3;
   std::vector<void*> allocs;
+  float* flat = nullptr;    // weights or gradients in the caller's order (copies in and out)
   float* y = nullptr;       // D x H x W output of the last forward
   float* dy = nullptr;      // scratch output gradient
   float* xin = nullptr;     // 2 x D x H x W input scratch (warm start)
@@ -484,6 +485,16 @@ static int grid_for(long long n, int block = 256) {
 #define ULAUNCH(grid, block, smem, stream, ...) (++g_ew_launches), __VA_ARGS__<<<grid, block, smem, stream>>>
 static unsigned long long g_ew_launches = 0;
 
+static int sm_count() {
+  static const int n = [] {
+    int dev = 0, c = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev);
+    return c > 0 ? c : 152;
+  }();
+  return n;
+}
+
 static int pow2_cols(int c) {
   int p = 32;
   while (p < c) p <<= 1;
@@ -568,6 +579,13 @@ static void conv_impl(unet_handle* n, int l, bool dgrad, const Tensor& s0, const
     z.Zc = 256 / (a.T * cout);
     if (z.Zc > 8) z.Zc = 8;
     if (z.Zc > v.D) z.Zc = v.D;
+    z.u_begin = v.Wp + 1;
+    z.u_end = (long long)v.H * v.Wp + v.W + 1;
+    // volumes that leave SMs without a CTA: one tile, then shorter plane columns
+    // (they read (Zc + 2) / Zc input planes per output plane, so not below 4)
+    auto ctas = [&]() { return ((z.u_end - z.u_begin + 128 * a.T - 1) / (128 * a.T)) * ((v.D + z.Zc - 1) / z.Zc); };
+    if (a.T == 2 && ctas() < sm_count()) a.T = 1;
+    if (z.Zc == 8 && ctas() < sm_count()) z.Zc = 4;
     a.R = 128 * a.T + 2 * v.Wp + 2;
     a.a_bytes = (uint32_t)a.R * 32u;
     z.bz_bytes = 9u * 2u * 3u * (uint32_t)cout * 16u;
@@ -576,8 +594,6 @@ static void conv_impl(unet_handle* n, int l, bool dgrad, const Tensor& s0, const
     z.a_region = (uint32_t)a.nstage * a.a_bytes;
     a.stage_bytes = a.a_bytes;
     a.tmem_cols = (uint32_t)pow2_cols(a.T * z.Zc * cout);
-    z.u_begin = v.Wp + 1;
-    z.u_end = (long long)v.H * v.Wp + v.W + 1;
     launch_conv3z(z, st);
     return;
   }
@@ -604,12 +620,17 @@ static void conv_impl(unet_handle* n, int l, bool dgrad, const Tensor& s0, const
   int T = 256 / cout;
   if (T < 1) T = 1;
   if (T > kMaxTiles) T = kMaxTiles;
+  // volumes that leave SMs without a CTA: fewer tiles, then fewer output channels per CTA
+  const long long tiles = (v.r_end - v.r_begin + 127) / 128;
+  while (T > 1 && (tiles + T - 1) / T < sm_count()) T /= 2;
+  a.nc = cout;
+  while (T == 1 && a.nc % 32 == 0 && tiles * (cout / a.nc) * 2 <= sm_count()) a.nc /= 2;
   int ns = 0;
   uint32_t stage = 0;
   for (;; T /= 2) {
     a.R = 128 * T + 2 * v.Wp + 2;
     a.a_bytes = (uint32_t)a.R * 32u;
-    a.b_bytes = (uint32_t)(9 * 2 * cout * 16);
+    a.b_bytes = (uint32_t)(9 * 2 * a.nc * 16);
     stage = ((a.a_bytes + a.b_bytes + 127u) / 128u) * 128u;
     ns = (int)(100u * 1024u / stage);
     if (ns >= 2 || T == 1) break;
@@ -618,7 +639,7 @@ static void conv_impl(unet_handle* n, int l, bool dgrad, const Tensor& s0, const
   a.T = T;
   a.nstage = ns;
   a.stage_bytes = stage;
-  a.tmem_cols = (uint32_t)pow2_cols(T * cout);
+  a.tmem_cols = (uint32_t)pow2_cols(T * a.nc);
   a.err = n->err;
   launch_conv3(a, st);
 }
@@ -768,35 +789,67 @@ static pic_status check_err(unet_handle* n) {
   return PIC_OK;
 }
 
-// host flat (oracle order: w[co][ci][a][b][c] per layer, then out) <-> device [27][cout][cin_store]
-static void host_to_store(const LayerDef& d, int cin_s, const float* src, std::vector<float>& dst) {
-  dst.assign(27ull * d.cout * cin_s, 0.f);
-  for (int co = 0; co < d.cout; ++co)
-    for (int ci = 0; ci < d.cin; ++ci)
-      for (int t = 0; t < 27; ++t) dst[((size_t)t * d.cout + co) * cin_s + ci] = src[((size_t)co * d.cin + ci) * 27 + t];
+// The caller's flat order (w[co][ci][a][b][c] per layer, then the output layer)
+// against the store's [27][cout][cin] per layer, cin padded to whole chunks.
+// Reordered on the device: the host's loops over 1.4 million values in strides
+// took as long as the whole backward pass of a small volume.
+struct FlatMap {
+  long long store[kNL], flat[kNL + 1];  // first value of every layer
+  int cin[kNL], cin_s[kNL], cout[kNL];
+  long long store_out;  // the output layer
+};
+static FlatMap flat_map(const unet_handle* n) {
+  FlatMap m{};
+  long long off = 0, hoff = 0;
+  for (int l = 0; l < kNL; ++l) {
+    const Layer& L = n->L[l];
+    m.store[l] = off;
+    m.flat[l] = hoff;
+    m.cin[l] = L.def.cin;
+    m.cin_s[l] = L.cin;
+    m.cout[l] = L.def.cout;
+    off += L.nw();
+    hoff += 27ll * L.def.cin * L.def.cout;
+  }
+  m.store_out = off;
+  m.flat[kNL] = hoff;
+  return m;
 }
+// TO_FLAT: flat = store; else store = flat (its padding channels are not written)
+template <bool TO_FLAT>
+__global__ void k_reorder(const __grid_constant__ FlatMap m, float* flat, float* store) {
+  const long long n = m.flat[kNL] + kOutC;
+  for (long long u = (long long)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += (long long)gridDim.x * blockDim.x) {
+    int l = 0;
+    while (l < kNL && u >= m.flat[l + 1]) ++l;
+    long long at;
+    if (l == kNL) {
+      at = m.store_out + (u - m.flat[kNL]);
+    } else {
+      const unsigned r = (unsigned)(u - m.flat[l]), q = r / 27u, t = r - 27u * q;
+      const unsigned co = q / (unsigned)m.cin[l], ci = q - co * (unsigned)m.cin[l];
+      at = m.store[l] + ((long long)t * m.cout[l] + co) * m.cin_s[l] + ci;
+    }
+    if (TO_FLAT) flat[u] = store[at];
+    else store[at] = flat[u];
+  }
+}
+
+// one layer's gradient in the caller's order (test hook)
 static void store_to_host(const LayerDef& d, int cin_s, const float* src, float* dst) {
   for (int co = 0; co < d.cout; ++co)
     for (int ci = 0; ci < d.cin; ++ci)
       for (int t = 0; t < 27; ++t) dst[((size_t)co * d.cin + ci) * 27 + t] = src[((size_t)t * d.cout + co) * cin_s + ci];
 }
 
-static pic_status copy_out(unet_handle* n, const float* dev_base, float* host, int64_t cnt) {
+static pic_status copy_out(unet_handle* n, float* dev_base, float* host, int64_t cnt) {
   if (!n || !host || cnt != num_weights()) return fail(n, PIC_EINVAL, "unet: need a handle and %lld values",
                                                         (long long)num_weights());
-  std::vector<float> buf(n->n_store);
-  if (cudaMemcpyAsync(buf.data(), dev_base, sizeof(float) * n->n_store, cudaMemcpyDeviceToHost, n->stream) !=
-          cudaSuccess ||
+  ULAUNCH(grid_for(cnt), 256, 0, n->stream, k_reorder<true>)(flat_map(n), n->flat, dev_base);
+  if (cudaGetLastError() != cudaSuccess ||
+      cudaMemcpyAsync(host, n->flat, sizeof(float) * cnt, cudaMemcpyDeviceToHost, n->stream) != cudaSuccess ||
       cudaStreamSynchronize(n->stream) != cudaSuccess)
     return fail(n, PIC_ECUDA, "unet: copy failed");
-  size_t off = 0, hoff = 0;
-  for (int l = 0; l < kNL; ++l) {
-    const Layer& L = n->L[l];
-    store_to_host(L.def, L.cin, buf.data() + off, host + hoff);
-    off += L.nw();
-    hoff += 27ull * L.def.cin * L.def.cout;
-  }
-  memcpy(host + hoff, buf.data() + off, sizeof(float) * kOutC);
   return PIC_OK;
 }
 
@@ -958,7 +1011,8 @@ extern "C" pic_status unet_create(int32_t D, int32_t H, int32_t W, void* cuda_st
   ns += kOutC;
   n->n_store = ns;
   n->wbuf = (float*)dev_alloc(sizeof(float) * 4 * ns);
-  ok = ok && n->wbuf;
+  n->flat = (float*)dev_alloc(sizeof(float) * num_weights());
+  ok = ok && n->wbuf && n->flat;
   if (ok) {
     long long off = 0;
     for (int l = 0; l < kNL; ++l) {
@@ -1052,21 +1106,11 @@ extern "C" pic_status unet_destroy(unet_handle* n) {
 extern "C" pic_status unet_set_weights(unet_handle* n, const float* host, int64_t cnt) {
   if (!n || !host || cnt != num_weights()) return fail(n, PIC_EINVAL, "unet_set_weights: need %lld values",
                                                        (long long)num_weights());
-  std::vector<float> buf;
-  std::vector<float> all(n->n_store, 0.f);
-  size_t off = 0, hoff = 0;
-  for (int l = 0; l < kNL; ++l) {
-    const Layer& L = n->L[l];
-    host_to_store(L.def, L.cin, host + hoff, buf);
-    memcpy(all.data() + off, buf.data(), sizeof(float) * buf.size());
-    off += L.nw();
-    hoff += 27ull * L.def.cin * L.def.cout;
-  }
-  memcpy(all.data() + off, host + hoff, sizeof(float) * kOutC);
-  if (cudaMemcpyAsync(n->wbuf, all.data(), sizeof(float) * n->n_store, cudaMemcpyHostToDevice, n->stream) !=
-          cudaSuccess ||
+  if (cudaMemcpyAsync(n->flat, host, sizeof(float) * cnt, cudaMemcpyHostToDevice, n->stream) != cudaSuccess ||
+      cudaMemsetAsync(n->wbuf, 0, sizeof(float) * n->n_store, n->stream) != cudaSuccess ||
       cudaMemsetAsync(n->wbuf + 2 * n->n_store, 0, sizeof(float) * 2 * n->n_store, n->stream) != cudaSuccess)
     return fail(n, PIC_ECUDA, "unet_set_weights: copy failed");
+  ULAUNCH(grid_for(cnt), 256, 0, n->stream, k_reorder<false>)(flat_map(n), n->flat, n->wbuf);
   n->adam_t = 0;
   rebuild_images(n, n->stream);
   if (cudaStreamSynchronize(n->stream) != cudaSuccess) return fail(n, PIC_ECUDA, "unet_set_weights: CUDA error");

@@ -16,6 +16,9 @@
 //   warps then read the accumulators (tcgen05.ld, lane = row) and write the
 //   interior rows as BF16 with the optional ReLU or ReLU-mask of the backward
 //   pass. Stages are double/triple buffered on full/empty mbarriers.
+//   Small volumes take fewer tiles per CTA and split the output channels over
+//   CTAs (each then copies its rows of the weight image), so that more SMs share
+//   the work; every output still sums its products in the same order.
 // Weight gradient: dw[tap][co][ci] = sum_r in[r + off(tap)][ci] dz[r][co], an
 //   MMA with M = 128 input channels (one tile of 16 channel blocks; rows past
 //   the tensor's channels are computed and dropped), N = cout and K = voxel rows,
@@ -66,6 +69,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3(const __grid_constant
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long r0 = a.v.r_begin + (long long)blockIdx.x * 128 * a.T;
   const int nst = 3 * a.nchunk;
+  const int n0 = blockIdx.y * a.nc;  // first output channel of this CTA
   if (threadIdx.x == 0) {
     for (int i = 0; i < a.nstage; ++i) {
       tc::mbar_init(&full[i], 1);
@@ -104,13 +108,20 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3(const __grid_constant
       const long long start = r0 + (long long)(dz - 1) * a.v.P - a.v.Wp - 1;
       tc::bulk_g2s(A, src + (g0 * a.v.rows + start) * 8, (uint32_t)a.R * 16u, &full[b]);
       tc::bulk_g2s(A + (size_t)a.R * 16, src + ((g0 + 1) * a.v.rows + start) * 8, (uint32_t)a.R * 16u, &full[b]);
-      tc::bulk_g2s(B, a.wimg + (size_t)s * (a.b_bytes / 2), a.b_bytes, &full[b]);
+      const __nv_bfloat16* wst = a.wimg + (size_t)s * 18u * (size_t)a.cout * 8u;
+      if (a.nc == a.cout) {
+        tc::bulk_g2s(B, wst, a.b_bytes, &full[b]);
+      } else {  // this CTA's rows of every tap and channel block
+        const uint32_t nb = (uint32_t)a.nc * 16u;
+        for (int q = 0; q < 18; ++q)
+          tc::bulk_g2s(B + (size_t)q * nb, wst + ((size_t)q * a.cout + n0) * 8u, nb, &full[b]);
+      }
       issued = s + 1;
     }
   } else if (warp == 1 && lane == 0) {
     // MMA issuer
-    const uint32_t idesc = tc::idesc_bf16(128, a.cout, 0, 0);
-    const uint32_t lbo_a = (uint32_t)a.R * 16u, lbo_b = (uint32_t)a.cout * 16u;
+    const uint32_t idesc = tc::idesc_bf16(128, a.nc, 0, 0);
+    const uint32_t lbo_a = (uint32_t)a.R * 16u, lbo_b = (uint32_t)a.nc * 16u;
     int s = 0;
     for (; s < nst; ++s) {
       const int b = s % a.nstage;
@@ -128,7 +139,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3(const __grid_constant
         const uint32_t shift = (uint32_t)(dy * a.v.Wp + dx) * 16u;
         for (int t = 0; t < a.T; ++t) {
           const uint64_t ad = tc::sdesc(A + shift + (uint32_t)t * 2048u, lbo_a, 128);
-          tc::mma_bf16(tmem + (uint32_t)(t * a.cout), ad, bd, idesc, (s | tap) != 0 ? 1u : 0u);
+          tc::mma_bf16(tmem + (uint32_t)(t * a.nc), ad, bd, idesc, (s | tap) != 0 ? 1u : 0u);
         }
       }
       tc::mma_commit(&empty[b]);
@@ -149,13 +160,13 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3(const __grid_constant
     for (int t = 0; t < a.T; ++t) {
       const long long r = r0 + (long long)t * 128 + m;
       const bool inside = row_interior(a.v, r);
-      for (int c0 = 0; c0 < a.cout; c0 += 16) {
+      for (int c0 = 0; c0 < a.nc; c0 += 16) {
         float v[16];
-        tc::tmem_ld16(tmem + lane_base + (uint32_t)(t * a.cout + c0), v);
+        tc::tmem_ld16(tmem + lane_base + (uint32_t)(t * a.nc + c0), v);
         if (!inside) continue;
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
-          const int gidx = (c0 >> 3) + half;
+          const int gidx = ((n0 + c0) >> 3) + half;
           const bool first = gidx < a.dgroups0;
           const long long gl = first ? gidx : gidx - a.dgroups0;
           float* f = v + 8 * half;
@@ -567,7 +578,7 @@ void launch_conv3(const ConvArgs& a, cudaStream_t s) {
   const long long grid = (rows + 128ll * a.T - 1) / (128ll * a.T);
   const size_t smem = smem_floor((size_t)a.nstage * a.stage_bytes + 256, a.tmem_cols);
   ++g_launches;
-  k_conv3<<<(unsigned)grid, kConvThreads, smem, s>>>(a);
+  k_conv3<<<dim3((unsigned)grid, a.cout / a.nc), kConvThreads, smem, s>>>(a);
 }
 
 void launch_conv3z(const ConvZArgs& z, cudaStream_t s) {

@@ -54,6 +54,7 @@ struct ConvArgs {
   int nchunk0;  // chunks taken from src0 (blocks 2c, 2c+1); the rest from src1
   const __nv_bfloat16* wimg;  // [3][nchunk][9][2][cout][8]
   int cout;
+  int nc;        // output channels per CTA (blockIdx.y takes channels [nc y, nc (y + 1)))
   __nv_bfloat16* dst0;
   __nv_bfloat16* dst1;
   int dgroups0;  // output blocks [0, dgroups0) to dst0, the rest to dst1
