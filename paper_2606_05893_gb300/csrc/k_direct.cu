@@ -275,14 +275,15 @@ __global__ void __launch_bounds__(kFftThreads, 3) k_dir_xf(DirectArgs a, const T
     if (r >= a.rows) break;
     const bool vb = r + 1 < a.rows;
     for (int f = lane; f < a.C; f += 32) {
+      const int2 at = __ldg(a.col + f);
       float2 A, B;
       if (f == 0) {
         const float2 z0 = Z[l];
-        const float2 zh = a.packed ? Z[__ldg(a.x.pos + n / 2) * kLpX + l] : make_float2(0.f, 0.f);
+        const float2 zh = a.packed ? Z[at.y * kLpX + l] : make_float2(0.f, 0.f);
         A = make_float2(z0.x, zh.x);
         B = make_float2(z0.y, zh.y);
       } else {
-        const float2 p = Z[__ldg(a.x.pos + f) * kLpX + l], m = Z[__ldg(a.x.pos + n - f) * kLpX + l];
+        const float2 p = Z[at.x * kLpX + l], m = Z[at.y * kLpX + l];
         A = make_float2(0.5f * (p.x + m.x), 0.5f * (p.y - m.y));
         B = make_float2(0.5f * (p.y + m.y), 0.5f * (m.x - p.x));
       }
@@ -400,12 +401,13 @@ __global__ void __launch_bounds__(kFftThreads, 3) k_dir_xi(DirectArgs a, Add add
     for (int f = lane; f < a.C; f += 32) {
       const float2 A = va ? spec[r * a.C + f] : make_float2(0.f, 0.f);
       const float2 B = vb ? spec[(r + 1) * a.C + f] : make_float2(0.f, 0.f);
+      const int2 at = __ldg(a.col + f);
       if (f == 0) {
         Z[l] = make_float2(A.x, B.x);
-        if (a.packed) Z[__ldg(a.x.pos + n / 2) * kLpX + l] = make_float2(A.y, B.y);
+        if (a.packed) Z[at.y * kLpX + l] = make_float2(A.y, B.y);
       } else {  // Z_f = A + i B, Z_-f = conj A + i conj B
-        Z[__ldg(a.x.pos + f) * kLpX + l] = make_float2(A.x - B.y, A.y + B.x);
-        Z[__ldg(a.x.pos + n - f) * kLpX + l] = make_float2(A.x + B.y, B.x - A.y);
+        Z[at.x * kLpX + l] = make_float2(A.x - B.y, A.y + B.x);
+        Z[at.y * kLpX + l] = make_float2(A.x + B.y, B.x - A.y);
       }
     }
   }
@@ -862,9 +864,28 @@ __device__ __forceinline__ double axis_lambda(int n, int f) {  // 2 - 2 cos(2 pi
   return 4.0 * s * s;
 }
 
-// twiddles, positions and eigenvalues of a plan, formed in FP64 and rounded once
+// Twiddles, positions, columns and eigenvalues of a plan, formed in FP64 and
+// rounded once. Columns of x (frequencies 0..C - 1) are ordered by position: the
+// lanes that gather (k_dir_xf) or scatter (k_dir_xi) them then walk runs of
+// neighbouring rows of the tile, where frequency order jumps by a whole radix
+// and meets the same bank 8 (128 points) or 16 times (256).
 __global__ void k_dir_tables(DirectArgs a) {
   const int t = (int)gtid(), n = (int)gstride();
+  extern __shared__ int sh[];  // frequency of every position of x, its inverse, frequency of every column
+  int *freqx = sh, *posx = sh + a.nx, *colf = posx + a.nx;
+  for (int p = threadIdx.x; p < a.nx; p += blockDim.x) {
+    const int f = axis_freq(a.x, p);
+    freqx[p] = f;
+    posx[f] = p;
+  }
+  __syncthreads();
+  for (int p = threadIdx.x; p < a.nx; p += blockDim.x) {
+    if (freqx[p] >= a.C) continue;
+    int c = 0;
+    for (int q = 0; q < p; ++q) c += freqx[q] < a.C ? 1 : 0;
+    colf[c] = freqx[p];
+  }
+  __syncthreads();
 #pragma unroll
   for (int axis = 0; axis < 2; ++axis) {
     const AxisPlan& A = axis == 0 ? a.x : a.y;
@@ -875,8 +896,12 @@ __global__ void k_dir_tables(DirectArgs a) {
       const_cast<int*>(A.pos)[axis_freq(A, m)] = m;
     }
   }
+  for (int c = t; c < a.C; c += n) {
+    const int f = colf[c];
+    const_cast<int2*>(a.col)[c] = make_int2(posx[f], posx[f > 0 ? a.nx - f : (a.packed ? a.nx / 2 : 0)]);
+  }
   for (int u = t; u < a.plane / 2; u += n) {
-    const int p = u / a.C, q = u - p * a.C;
+    const int p = u / a.C, q = colf[u - p * a.C];
     const int g = axis_freq(a.y, p);
     const double ly = axis_lambda(a.ny, g);
     double l0 = axis_lambda(a.nx, q), l1 = l0;
@@ -925,7 +950,8 @@ bool DirectSolver::plan(int nx, int ny, int nz) {
 }
 
 size_t DirectSolver::table_bytes() const {
-  return (sizeof(float2) + sizeof(int)) * (size_t)(a.nx + a.ny) + sizeof(float) * (size_t)a.plane;
+  return (sizeof(float2) + sizeof(int)) * (size_t)(a.nx + a.ny) + 8 + sizeof(int2) * (size_t)a.C +
+         sizeof(float) * (size_t)a.plane;
 }
 size_t DirectSolver::spec_bytes() const { return sizeof(float) * (size_t)a.plane * a.P; }
 
@@ -935,7 +961,8 @@ cudaError_t DirectSolver::place(void* tables_mem, void* spec_mem, cudaStream_t s
   a.y.tw = a.x.tw + a.nx;
   a.x.pos = (const int*)(a.y.tw + a.ny);
   a.y.pos = a.x.pos + a.nx;
-  a.lam = (const float*)(a.y.pos + a.ny);
+  a.col = (const int2*)(t + (sizeof(float2) * (a.nx + a.ny) + sizeof(int) * (a.nx + a.ny) + 7) / 8 * 8);
+  a.lam = (const float*)(a.col + a.C);
   a.spec = (float*)spec_mem;
   cudaError_t e;
   if ((e = allow_smem(k_dir_xf<float, true>)) || (e = allow_smem(k_dir_xf<float, false>)) ||
@@ -946,7 +973,7 @@ cudaError_t DirectSolver::place(void* tables_mem, void* spec_mem, cudaStream_t s
       (e = allow_smem(k_dir_xi<Add64, true>)) || (e = allow_smem(k_dir_xi<Add64, false>)))
     return e;
   const int n = std::max(std::max(a.nx, a.ny), a.plane / 2);
-  PIC_LAUNCH(std::min((n + 127) / 128, 1024), 128, 0, s, k_dir_tables)(a);
+  PIC_LAUNCH(std::min((n + 127) / 128, 1024), 128, sizeof(int) * (2 * a.nx + a.C), s, k_dir_tables)(a);
   return cudaGetLastError();
 }
 

@@ -37,6 +37,7 @@ struct DirectArgs {
   long long rows;  // ny P rows of x
   float norm;      // 1 / (nx ny)
   AxisPlan x, y;
+  const int2* col;   // [C] where column c's frequency f and -f end up (columns in the order of the former)
   const float* lam;  // [plane] x and y eigenvalue of every float of a spectral plane
   float* spec;       // [P][ny][C] float2
 };
