@@ -387,10 +387,10 @@ __global__ void k_load(Grid g, S st, DevCounters* cnt, int cur, int species, lon
   for (long long i = gtid(); i < n; i += gstride()) {
     const unsigned long long slot = base + i;
     if (slot >= (unsigned long long)cap) continue;
-    store_write(st, g, slot, x[3 * i], x[3 * i + 1], x[3 * i + 2], v[3 * i], v[3 * i + 1], v[3 * i + 2],
-                pid0 + (uint32_t)i, mw ? mw[i] : 1u);
+    const auto p = make_particle(st, g, x[3 * i], x[3 * i + 1], x[3 * i + 2], v[3 * i], v[3 * i + 1], v[3 * i + 2],
+                                 pid0 + (uint32_t)i, mw ? mw[i] : 1u);
+    store_write_p(st, slot, p);
     if (nd.on) {  // the next step's deposit is being accumulated: add this particle
-      const auto p = store_read(st, g, slot);
       if (neutral) atomicAdd(&nd.ncount[species][cell_now(g, p)], (int)p.mw);
       else if (nd.qw_h3[species] != 0.0) deposit_one(g, p, nd.rho32, nd.rho64, nd.qw_h3[species]);
     }

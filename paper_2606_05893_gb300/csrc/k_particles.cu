@@ -273,9 +273,9 @@ __global__ void k_inject(InjectArgs<S> a) {
       vz = s.sig * fabs(n3);
       z = u01_64(d3.x, d3.y) * vz * a.g.dt;
     }
-    store_write(a.st[s.species], a.g, slot, x, y, z, vx, vy, vz, pid);
+    const auto p = make_particle(a.st[s.species], a.g, x, y, z, vx, vy, vz, pid);
+    store_write_p(a.st[s.species], slot, p);
     if (a.nd.on) {  // the next step's deposit is being accumulated: add this particle
-      const auto p = store_read(a.st[s.species], a.g, slot);
       if (a.role[s.species] == ROLE_NEUTRAL) atomicAdd(&a.nd.ncount[s.species][cell_now(a.g, p)], 1);
       else if (a.nd.qw_h3[s.species] != 0.0) deposit_one(a.g, p, a.nd.rho32, a.nd.rho64, a.nd.qw_h3[s.species]);
     }
@@ -312,17 +312,28 @@ __global__ void k_inject(InjectArgs<S> a) {
 // The neutral count likewise (the group's size). FP64 store: plain FP64
 // atomics (summing doubles across lanes would load the narrow FP64 pipe).
 // Every lane of the warp calls it.
+// Shared memory of a push block (one for whichever species the block pushes).
+struct PushShared {
+  unsigned int wcnt[kPushWarps];
+  unsigned long long base;
+  // per-thread tallies, each touched by its own thread only (no atomics, no
+  // registers held): absorbed at cathode / anode, their sum of v^2, elastic
+  // collisions; reduced once per block at the end
+  // (with variable weights v^2 is weighted by the multiplicity, and rows 3, 4
+  // sum the absorbed multiplicities for the charge)
+  double tv2[2][kPushBlock];
+  unsigned int tn[5][kPushBlock];
+  float w[kPushWarps][8 * 32];  // a warp's deposit weights, [corner][lane] (conflict-free rows of 32 words)
+};
 template <bool CHARGED, bool NEUTRAL>
-__device__ __forceinline__ void next_deposit(const PushArgs<StoreMx>& a, const ParticleMx& p, bool stored) {
+__device__ __forceinline__ void next_deposit(const PushArgs<StoreMx>& a, const ParticleMx& p, bool stored, PushShared& sh) {
   const int lane = threadIdx.x & 31;
   // a lane without a particle gets a key of its own (negative: never a cell)
   const int key = stored ? p.cell : -1 - lane;
   const unsigned grp = __match_any_sync(0xffffffffu, key);
   const bool lead = stored && (__ffs(grp) - 1) == lane;
   if (CHARGED) {
-    // this warp's weights, [corner][lane] (conflict-free rows of 32 words)
-    __shared__ float s_w[kPushWarps][8 * 32];
-    float* sw = s_w[threadIdx.x >> 5];
+    float* sw = sh.w[threadIdx.x >> 5];
     float w[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (stored) {
       cic_weights(p.ox, p.oy, p.oz, w);
@@ -358,7 +369,7 @@ __device__ __forceinline__ void next_deposit(const PushArgs<StoreMx>& a, const P
   }
 }
 template <bool CHARGED, bool NEUTRAL>
-__device__ __forceinline__ void next_deposit(const PushArgs<Store64>& a, const Particle64& p, bool stored) {
+__device__ __forceinline__ void next_deposit(const PushArgs<Store64>& a, const Particle64& p, bool stored, PushShared&) {
   if (!stored) return;
   if (CHARGED) deposit_one(a.g, p, nullptr, a.nd.rho64, a.nd.qw_h3[a.species]);
   if (NEUTRAL) atomicAdd(&a.nd.ncount[a.species][cell_now(a.g, p)], (int)p.mw);
@@ -381,21 +392,16 @@ __device__ __noinline__ void log_cathode_hit(const HitLog& h, uint32_t pid, int 
 }
 
 template <class S, bool CHARGED, bool MCC, bool NEUTRAL>
-__global__ void __launch_bounds__(kPushBlock, PTraits<S>::kMinBlocks) k_push(PushArgs<S> a) {
+__device__ __forceinline__ void push_block(const PushArgs<S>& a, PushShared& sh) {
   // Each thread advances kIlp particles per round (their loads are issued
   // together, so the memory latency of one hides behind the others). Output
   // slots are reserved once per block and round (one global atomic per
   // kIlp * 256 particles); absorption statistics and elastic counts accumulate
   // in shared memory and reach HBM once per block.
-  __shared__ unsigned int s_wcnt[kPushWarps];
-  __shared__ unsigned long long s_base;
-  // per-thread tallies, each touched by its own thread only (no atomics, no
-  // registers held): absorbed at cathode / anode, their sum of v^2, elastic
-  // collisions; reduced once per block at the end
-  // (with variable weights v^2 is weighted by the multiplicity, and rows 3, 4
-  // sum the absorbed multiplicities for the charge)
-  __shared__ double s_tv2[2][kPushBlock];
-  __shared__ unsigned int s_tn[5][kPushBlock];
+  unsigned int* s_wcnt = sh.wcnt;
+  unsigned long long& s_base = sh.base;
+  auto& s_tv2 = sh.tv2;
+  auto& s_tn = sh.tn;
   const int tx = threadIdx.x;
   s_tv2[0][tx] = s_tv2[1][tx] = 0.0;
   s_tn[0][tx] = s_tn[1][tx] = s_tn[2][tx] = s_tn[3][tx] = s_tn[4][tx] = 0u;
@@ -549,7 +555,7 @@ __global__ void __launch_bounds__(kPushBlock, PTraits<S>::kMinBlocks) k_push(Pus
     // count) at x^{n+1} of every particle kept
     if (a.nd.on) {
 #pragma unroll
-      for (int u = 0; u < kIlp; ++u) next_deposit<CHARGED, NEUTRAL>(a, p[u], stored[u]);
+      for (int u = 0; u < kIlp; ++u) next_deposit<CHARGED, NEUTRAL>(a, p[u], stored[u], sh);
     }
   }
   // block totals of the tallies by warp 0: counts in integers, the FP64 sums of
@@ -597,6 +603,23 @@ __global__ void __launch_bounds__(kPushBlock, PTraits<S>::kMinBlocks) k_push(Pus
     }
     if (lane == 0 && nel) atomicAdd(&a.cnt->n_el, (unsigned long long)nel);
   }
+}
+
+template <class S, bool CHARGED, bool MCC, bool NEUTRAL>
+__global__ void __launch_bounds__(kPushBlock, PTraits<S>::kMinBlocks) k_push(const __grid_constant__ PushArgs<S> a) {
+  __shared__ PushShared sh;
+  push_block<S, CHARGED, MCC, NEUTRAL>(a, sh);
+}
+
+// Two charged species in one launch (blockIdx.y): neither reads what the other
+// writes, their sums are atomics either way, and a species that fills only part
+// of the GPU, or ends in a nearly empty wave, leaves the rest to the other.
+template <class S, bool MCC0, bool MCC1>
+__global__ void __launch_bounds__(kPushBlock, PTraits<S>::kMinBlocks)
+    k_push_pair(const __grid_constant__ PushArgs<S> a0, const __grid_constant__ PushArgs<S> a1) {
+  __shared__ PushShared sh;
+  if (blockIdx.y == 0) push_block<S, true, MCC0, false>(a0, sh);
+  else push_block<S, true, MCC1, false>(a1, sh);
 }
 
 // ---------------------------------------------------------------------------
@@ -668,7 +691,11 @@ __global__ void __launch_bounds__(kRankWarps * 32) k_resolve_rank(ResolveArgs a)
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const unsigned int ne = min(a.cnt->n_events, (unsigned int)a.ev_cap);
   const unsigned int nc = min(a.cnt->n_cands, (unsigned int)a.cand_cap);
-  if (blockIdx.x == 0 && threadIdx.x == 0) a.cnt->ev_sort_n = ne;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    a.cnt->ev_sort_n = ne;
+    *a.order.small = ne <= kSmallEvents ? 1 : 0;
+    if (a.order.use_graph) cudaGraphSetConditional(a.order.handle, ne > kSmallEvents ? 1u : 0u);
+  }
   if ((unsigned long long)ne * nc > kScanWork) {
     for (long long e = gtid(); e < ne; e += gstride()) {
       const uint32_t cell = a.ev[e].cell, pid = a.ev[e].pid;
@@ -773,12 +800,27 @@ __global__ void k_resolve_apply(ApplyArgs<S> a) {
   const unsigned long long ni_out = a.cnt->n[a.i_out][a.i_species];
   const unsigned long long nn_out = a.cnt->n[a.n_out][a.n_species];
   const uint32_t pid0 = a.cnt->next_pid;
-  // event r on block r mod G (as for injection: each event's FP64 kinematics
+  const unsigned int ne = min(a.cnt->n_events, (unsigned int)a.commit.ev_cap);
+  // few events: each thread takes one and finds its place r among the successful
+  // ones (the keys are unique and put those first); more: in the sorted order
+  const bool few = ne <= kSmallEvents;
+  // event q on block q mod G (as for injection: each event's FP64 kinematics
   // then run on their own SM's FP64 pipe instead of queueing on one)
-  for (long long r = blockIdx.x + (long long)gridDim.x * threadIdx.x; r < ns;
-       r += (long long)gridDim.x * blockDim.x) {
-    if (!PIC_BOUNDS(a.sorted_vals[r] < (uint32_t)a.ev_cap, a.cnt)) continue;
-    const Event ev = a.ev[a.sorted_vals[r]];
+  for (long long q = blockIdx.x + (long long)gridDim.x * threadIdx.x; q < (few ? ne : ns);
+       q += (long long)gridDim.x * blockDim.x) {
+    long long r = q;
+    uint32_t e = (uint32_t)q;
+    if (few) {
+      if (a.ev[e].victim < 0) continue;  // suppressed
+      const unsigned long long key = a.sort_keys[e];
+      r = 0;
+#pragma unroll 8
+      for (unsigned int t = 0; t < ne; ++t) r += a.sort_keys[t] < key ? 1 : 0;
+    } else {
+      e = a.sorted_vals[q];
+    }
+    if (!PIC_BOUNDS(e < (uint32_t)a.ev_cap, a.cnt)) continue;
+    const Event ev = a.ev[e];
     if (!PIC_BOUNDS(ev.victim >= 0 && ev.victim < a.cand_cap &&
                         (long long)ev.slot < (ev.kind == XS_CHARGE_EXCHANGE ? a.i_cap : a.e_cap),
                     a.cnt))
@@ -869,7 +911,6 @@ __global__ void k_resolve_apply(ApplyArgs<S> a) {
   }
   // the per-cell list heads of this step's events (and so of its candidates) go
   // back to empty; nothing in this kernel reads them
-  const unsigned int ne = min(a.cnt->n_events, (unsigned int)a.commit.ev_cap);
   for (long long e = gtid(); e < ne; e += gstride()) {
     const uint32_t c = a.ev[e].cell;
     a.ev_head[c] = -1;
@@ -909,6 +950,15 @@ void launch_push(const PushArgs<S>& a, int role, bool mcc, int grid, cudaStream_
 }
 
 
+template <class S>
+void launch_push_pair(const PushArgs<S>& a0, bool mcc0, const PushArgs<S>& a1, bool mcc1, int grid, cudaStream_t st) {
+  const dim3 g(grid, 2);
+  if (mcc0 && mcc1) PIC_LAUNCH(g, 256, 0, st, k_push_pair<S, true, true>)(a0, a1);
+  else if (mcc0) PIC_LAUNCH(g, 256, 0, st, k_push_pair<S, true, false>)(a0, a1);
+  else if (mcc1) PIC_LAUNCH(g, 256, 0, st, k_push_pair<S, false, true>)(a0, a1);
+  else PIC_LAUNCH(g, 256, 0, st, k_push_pair<S, false, false>)(a0, a1);
+}
+
 void launch_resolve_rank(const ResolveArgs& a, int grid, cudaStream_t st) {
   PIC_LAUNCH(grid, kRankWarps * 32, 0, st, k_resolve_rank)(a);
 }
@@ -921,6 +971,8 @@ template void launch_inject<Store64>(const InjectArgs<Store64>&, int, cudaStream
 template void launch_inject<StoreMx>(const InjectArgs<StoreMx>&, int, cudaStream_t);
 template void launch_push<Store64>(const PushArgs<Store64>&, int, bool, int, cudaStream_t);
 template void launch_push<StoreMx>(const PushArgs<StoreMx>&, int, bool, int, cudaStream_t);
+template void launch_push_pair<Store64>(const PushArgs<Store64>&, bool, const PushArgs<Store64>&, bool, int, cudaStream_t);
+template void launch_push_pair<StoreMx>(const PushArgs<StoreMx>&, bool, const PushArgs<StoreMx>&, bool, int, cudaStream_t);
 template void launch_resolve_apply<Store64>(const ApplyArgs<Store64>&, int, cudaStream_t);
 template void launch_resolve_apply<StoreMx>(const ApplyArgs<StoreMx>&, int, cudaStream_t);
 

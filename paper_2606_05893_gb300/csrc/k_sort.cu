@@ -133,95 +133,73 @@ __global__ void __launch_bounds__(kSortBlock) k_radix_scatter(const unsigned lon
 // ranks every pair against all others (ties by input position, so the order is
 // the stable one), writes it at its rank in the buffers the radix passes would
 // end in, and sets *done so that those passes return at once.
-constexpr int kSmallSort = 2048;
-// In a recorded graph the radix passes sit in a conditional IF node whose
-// condition this kernel sets (use_graph): they are launched only when needed.
-__global__ void __launch_bounds__(1024) k_small_sort(const unsigned long long* __restrict__ kin,
-                                                     const uint32_t* __restrict__ vin,
-                                                     unsigned long long* __restrict__ kout,
-                                                     uint32_t* __restrict__ vout, const unsigned long long* n_dev,
-                                                     long long n_max, int* done, cudaGraphConditionalHandle h_radix,
-                                                     int use_graph) {
-  __shared__ unsigned long long sk[kSmallSort];
-  const long long n = min((long long)*n_dev, n_max);
-  if (use_graph && threadIdx.x == 0) cudaGraphSetConditional(h_radix, n > kSmallSort ? 1u : 0u);
-  if (n > kSmallSort) {
-    if (threadIdx.x == 0) *done = 0;
-    return;
-  }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) sk[i] = kin[i];
-  __syncthreads();
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const unsigned long long k = sk[i];
-    int rank = 0;
-    for (int j = 0; j < n; ++j) {
-      const unsigned long long kj = sk[j];
-      rank += (kj < k || (kj == k && j < i)) ? 1 : 0;
-    }
-    kout[rank] = k;
-    vout[rank] = vin[i];
-  }
-  if (threadIdx.x == 0) *done = 1;
-}
-
+// ---------------------------------------------------------------------------
+// Order of a step's events. Up to kSmallEvents the resolve's apply kernel ranks
+// each event against all others itself; larger lists take the radix passes. Which
+// of the two is known on the device only: the rank kernel sets `order.small`, so
+// that the passes return at once, or, in a step being recorded, the condition of
+// the IF node they sit in, so that they are not launched at all.
+// ---------------------------------------------------------------------------
 static int radix_passes(const SortBuffers& b, const unsigned long long* n_dev, int bit0, int bit1, cudaStream_t s,
                         const int* skip);
 
-// When s is capturing (a step being recorded), the small path's kernel decides
-// through a conditional IF node whether the radix passes run at all.
-static cudaError_t radix_if_node(const SortBuffers& b, const unsigned long long* n_dev, int bit0, int bit1,
+static bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusActive;
+}
+
+EventOrder event_order_begin(const SortBuffers& b, cudaStream_t s) {
+  EventOrder o{};
+  o.small = b.small_done;
+  cudaStreamCaptureStatus status;
+  cudaGraph_t g;
+  if (capturing(s) && cudaStreamGetCaptureInfo(s, &status, nullptr, &g, nullptr, nullptr, nullptr) == cudaSuccess &&
+      cudaGraphConditionalHandleCreate(&o.handle, g, 0u, cudaGraphCondAssignDefault) == cudaSuccess)
+    o.use_graph = 1;
+  return o;
+}
+
+static cudaError_t radix_if_node(const SortBuffers& b, const EventOrder& o, const unsigned long long* n_dev, int bits,
                                  cudaStream_t s) {
+  if (!o.use_graph) return cudaErrorIllegalState;
   cudaStreamCaptureStatus status;
   cudaGraph_t g;
   const cudaGraphNode_t* deps = nullptr;
   const cudaGraphEdgeData* edges = nullptr;
   size_t ndeps = 0;
-  cudaError_t e = cudaStreamGetCaptureInfo(s, &status, nullptr, &g, &deps, &edges, &ndeps);
-  if (e != cudaSuccess) return e;
-  cudaGraphConditionalHandle h;
-  if ((e = cudaGraphConditionalHandleCreate(&h, g, 0u, cudaGraphCondAssignDefault))) return e;
-  PIC_LAUNCH(1, 1024, 0, s, k_small_sort)(b.ka, b.va, b.kb, b.vb, n_dev, b.n_max, b.small_done, h, 1);
-  if ((e = cudaGetLastError())) return e;
+  cudaError_t e;
   if ((e = cudaStreamGetCaptureInfo(s, &status, nullptr, &g, &deps, &edges, &ndeps))) return e;
   cudaGraphNodeParams np = {};
   np.type = cudaGraphNodeTypeConditional;
-  np.conditional.handle = h;
+  np.conditional.handle = o.handle;
   np.conditional.type = cudaGraphCondTypeIf;
   np.conditional.size = 1;
   cudaGraphNode_t node;
   if ((e = cudaGraphAddNode(&node, g, deps, edges, ndeps, &np))) return e;
   cudaGraph_t body = np.conditional.phGraph_out[0];
   if ((e = cudaStreamBeginCaptureToGraph(b.aux, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed))) return e;
-  radix_passes(b, n_dev, bit0, bit1, b.aux, nullptr);
+  radix_passes(b, n_dev, 0, bits, b.aux, nullptr);
   cudaGraph_t tmp;
   const cudaError_t e1 = cudaStreamEndCapture(b.aux, &tmp);
   if ((e = cudaGetLastError()) || (e = e1)) return e;
   return cudaStreamUpdateCaptureDependencies(s, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
 }
 
-int radix_sort_pairs(const SortBuffers& b, const unsigned long long* n_dev, int bit0, int bit1, cudaStream_t s,
-                     bool small_path) {
-  const int passes = (bit1 - bit0 + 7) / 8;
-  const int* skip = nullptr;
-  // the small path writes where an odd number of passes ends (kb, vb); an even
-  // number would end in the input buffers, which the ranking still reads
-  if (small_path && (passes & 1)) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (b.aux && cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusActive) {
-      if (radix_if_node(b, n_dev, bit0, bit1, s) != cudaSuccess) {
-        // a half-built node must not be replayed: synchronising a capturing
-        // stream is illegal and invalidates the capture, so the recording
-        // fails and the instance steps directly from then on
-        cudaStreamSynchronize(s);
-        cudaGetLastError();
-      }
-      return 1;
-    }
-    const cudaGraphConditionalHandle none = 0;
-    PIC_LAUNCH(1, 1024, 0, s, k_small_sort)(b.ka, b.va, b.kb, b.vb, n_dev, b.n_max, b.small_done, none, 0);
-    skip = b.small_done;
+int event_order_end(const SortBuffers& b, const EventOrder& o, const unsigned long long* n_dev, int bits,
+                    cudaStream_t s) {
+  if (!capturing(s)) return radix_passes(b, n_dev, 0, bits, s, b.small_done);
+  if (radix_if_node(b, o, n_dev, bits, s) != cudaSuccess) {
+    // a half-built node must not be replayed: synchronising a capturing
+    // stream is illegal and invalidates the capture, so the recording
+    // fails and the instance steps directly from then on
+    cudaStreamSynchronize(s);
+    cudaGetLastError();
   }
-  return radix_passes(b, n_dev, bit0, bit1, s, skip);
+  return ((bits + 7) / 8) & 1;
+}
+
+int radix_sort_pairs(const SortBuffers& b, const unsigned long long* n_dev, int bit0, int bit1, cudaStream_t s) {
+  return radix_passes(b, n_dev, bit0, bit1, s, nullptr);
 }
 
 static int radix_passes(const SortBuffers& b, const unsigned long long* n_dev, int bit0, int bit1, cudaStream_t s,

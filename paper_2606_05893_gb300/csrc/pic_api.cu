@@ -977,6 +977,8 @@ pic_status step_instance(pic_handle* h, Instance* I) {
   T.end(st);
 
   // a6-a8 + a10 push / absorb / collide / compact: charged species first, then neutrals
+  PushArgs<S> first{};  // a charged species waiting for a second one to share its launch
+  int first_s = -1;
   for (int pass = 0; pass < 2; ++pass) {
     for (int s = 0; s < I->nsp; ++s) {
       const bool neutral = I->species[s].role == PIC_NEUTRAL;
@@ -1012,10 +1014,22 @@ pic_status step_instance(pic_handle* h, Instance* I) {
         a.ev_head = nullptr;  // no victims in this species
       }
       const int role = I->species[s].role;
+      if (!neutral && !T.on) {  // two charged species a launch, unless each is timed
+        if (first_s < 0) {
+          first = a;
+          first_s = s;
+        } else {
+          launch_push_pair<S>(first, first.mc.nch > 0, a, mcc, blocks, st);
+          first_s = -1;
+        }
+        continue;
+      }
       T.begin(role == PIC_ELECTRON ? PIC_PH_PUSH_ELECTRON : (role == PIC_ION ? PIC_PH_PUSH_ION : PIC_PH_PUSH_NEUTRAL), st);
       launch_push<S>(a, neutral ? ROLE_NEUTRAL : ROLE_ELECTRON, mcc, blocks, st);
       T.end(st);
     }
+    if (first_s >= 0) launch_push<S>(first, ROLE_ELECTRON, first.mc.nch > 0, blocks, st);
+    first_s = -1;
   }
 
   // a9 resolve of ionizations and charge exchanges
@@ -1033,8 +1047,9 @@ pic_status step_instance(pic_handle* h, Instance* I) {
     r.sort_keys = I->evsort.ka;
     r.sort_vals = I->evsort.va;
     const int rb = std::min(blocks, (I->ev_cap + 255) / 256);
+    r.order = event_order_begin(I->evsort, st);
     launch_resolve_rank(r, rb, st);
-    const int where = radix_sort_pairs(I->evsort, &I->cnt->ev_sort_n, 0, 40, st, true);
+    const int where = event_order_end(I->evsort, r.order, &I->cnt->ev_sort_n, 40, st);
     ApplyArgs<S> ap{};
     ap.g = g;
     ap.cnt = I->cnt;
@@ -1043,6 +1058,7 @@ pic_status step_instance(pic_handle* h, Instance* I) {
     ap.cand = I->cand;
     ap.cand_cap = I->cand_cap;
     ap.sorted_vals = where ? I->evsort.vb : I->evsort.va;
+    ap.sort_keys = I->evsort.ka;
     ap.key = key;
     // the ionization fixes electrons, victims and ions; without it the exchange
     // fixes victims and ions (validation makes the two agree when both exist)

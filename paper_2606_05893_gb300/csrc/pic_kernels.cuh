@@ -439,37 +439,42 @@ __device__ __forceinline__ void store_write_v(const StoreMx& s, long long i, con
 __device__ __forceinline__ void store_kill(const Store64& s, long long i) { s.pid[i] = kPidDead; }
 __device__ __forceinline__ void store_kill(const StoreMx& s, long long i) { s.pid[i] = kPidDead; }
 
-// Write from FP64 values (injection, host upload).
-__device__ __forceinline__ void store_write(const Store64& s, const Grid& g, long long i, double x, double y, double z,
-                                            double vx, double vy, double vz, uint32_t pid, uint32_t mw = 1u) {
-  (void)g;
-  if (s.mw) s.mw[i] = mw;
-  s.x[i] = x;
-  s.y[i] = y;
-  s.z[i] = z;
-  s.vx[i] = vx;
-  s.vy[i] = vy;
-  s.vz[i] = vz;
-  s.pid[i] = pid;
-}
+// A particle from FP64 values (injection, host upload), as the store keeps it.
 __device__ __forceinline__ float offset_of(double gcoord, int cell) {
   float o = (float)(gcoord - (double)cell);
   if (o >= 1.f) o = 0x1.fffffep-1f;
   if (o < 0.f) o = 0.f;
   return o;
 }
-__device__ __forceinline__ void store_write(const StoreMx& s, const Grid& g, long long i, double x, double y, double z,
-                                            double vx, double vy, double vz, uint32_t pid, uint32_t mw = 1u) {
-  if (s.mw) s.mw[i] = mw;
+__device__ __forceinline__ Particle64 make_particle(const Store64&, const Grid& g, double x, double y, double z, double vx,
+                                                    double vy, double vz, uint32_t pid, uint32_t mw = 1u) {
+  Particle64 p;
+  p.x = x;
+  p.y = y;
+  p.z = z;
+  p.vx = vx;
+  p.vy = vy;
+  p.vz = vz;
+  p.pid = pid;
+  p.mw = mw;
+  p.l = locate64(g, x, y, z);
+  p.cell = ((long long)p.l.k * g.ny + p.l.j) * g.nx + p.l.i;
+  return p;
+}
+__device__ __forceinline__ ParticleMx make_particle(const StoreMx&, const Grid& g, double x, double y, double z, double vx,
+                                                    double vy, double vz, uint32_t pid, uint32_t mw = 1u) {
+  ParticleMx p;
   const Loc l = locate64(g, x, y, z);
-  s.cell[i] = (l.k * g.ny + l.j) * g.nx + l.i;
-  s.ox[i] = offset_of(x * g.inv_h, l.i);
-  s.oy[i] = offset_of(y * g.inv_h, l.j);
-  s.oz[i] = offset_of(z * g.inv_h, l.k);
-  s.vx[i] = (float)vx;
-  s.vy[i] = (float)vy;
-  s.vz[i] = (float)vz;
-  s.pid[i] = pid;
+  p.cell = (l.k * g.ny + l.j) * g.nx + l.i;
+  p.ox = offset_of(x * g.inv_h, l.i);
+  p.oy = offset_of(y * g.inv_h, l.j);
+  p.oz = offset_of(z * g.inv_h, l.k);
+  p.vx = (float)vx;
+  p.vy = (float)vy;
+  p.vz = (float)vz;
+  p.pid = pid;
+  p.mw = mw;
+  return p;
 }
 // Read as FP64 values (host download).
 __device__ __forceinline__ void store_get(const Store64& s, const Grid& g, long long i, double* x, double* v,
@@ -605,6 +610,14 @@ struct PushArgs {
   HitLog hits;
 };
 
+// How the rank kernel tells the radix passes of the events whether they run.
+constexpr unsigned kSmallEvents = 2048;  // events that the apply kernel ranks itself
+struct EventOrder {
+  int* small;     // set to 1 for at most kSmallEvents events, else 0
+  int use_graph;  // a recorded step: the IF node's condition instead
+  cudaGraphConditionalHandle handle;
+};
+
 struct ResolveArgs {
   DevCounters* cnt;
   Event* ev;
@@ -616,6 +629,7 @@ struct ResolveArgs {
   int32_t* cand_head;
   unsigned long long* sort_keys;
   uint32_t* sort_vals;
+  EventOrder order;
 };
 
 // Buffers and capacities the resolve commit updates (species < 0: absent).
@@ -638,7 +652,8 @@ struct ApplyArgs {
   int ev_cap;
   const Cand* cand;
   int cand_cap;
-  const uint32_t* sorted_vals;
+  const uint32_t* sorted_vals;           // events in apply order (more than kSmallEvents)
+  const unsigned long long* sort_keys;  // of every event
   XsDev ch[kMaxXsec];
   uint2 key;
   S e_st;                  // ionization: electrons (e_species < 0 without an ionization channel)
@@ -682,6 +697,8 @@ void launch_inject(const InjectArgs<S>& a, int grid, cudaStream_t st);
 void launch_step_end(DevCounters* cnt, const Circuit& c, cudaStream_t st);
 template <class S>
 void launch_push(const PushArgs<S>& a, int role, bool mcc, int grid, cudaStream_t st);
+template <class S>
+void launch_push_pair(const PushArgs<S>& a0, bool mcc0, const PushArgs<S>& a1, bool mcc1, int grid, cudaStream_t st);
 void launch_resolve_rank(const ResolveArgs& a, int grid, cudaStream_t st);
 template <class S>
 void launch_resolve_apply(const ApplyArgs<S>& a, int grid, cudaStream_t st);
@@ -745,13 +762,14 @@ struct SortBuffers {
   uint32_t *va, *vb;
   uint32_t* hist;      // 256 * nblocks(n_max)
   uint32_t* digit_tot; // 256
-  int* small_done;     // set when the single-block path sorted the input
+  int* small_done;     // set when the radix passes are not needed (EventOrder)
   long long n_max;
   cudaStream_t aux;    // capture stream of the radix passes inside a recorded step (small path)
 };
 long long sort_hist_entries(long long n_max);
-int radix_sort_pairs(const SortBuffers& b, const unsigned long long* n_dev, int bit0, int bit1, cudaStream_t s,
-                     bool small_path = false);
+EventOrder event_order_begin(const SortBuffers& b, cudaStream_t s);
+int event_order_end(const SortBuffers& b, const EventOrder& o, const unsigned long long* n_dev, int bits, cudaStream_t s);
+int radix_sort_pairs(const SortBuffers& b, const unsigned long long* n_dev, int bit0, int bit1, cudaStream_t s);
 // exclusive scan of int32 counts[n] into int64 out[n+1] (out[n] = total)
 size_t scan_temp_bytes(long long n);
 void exclusive_scan_i32_i64(const int32_t* counts, long long n, long long* out, void* temp, cudaStream_t s);
