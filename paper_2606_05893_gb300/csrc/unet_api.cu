@@ -135,92 +135,103 @@ __device__ __forceinline__ void decode(const Vol& v, long long n, int& d, int& j
   i = (int)(rem - (long long)j * v.W);
 }
 
+// Elementwise passes over a volume: a block takes whole rows of voxels (threadIdx.x
+// along the row, so indices cost one 32-bit division a thread), blockIdx.y one
+// 8-channel block, so that small volumes of many channels fill the GPU too (with
+// all channel blocks in one thread's loop, 12 us at 4x4x4 voxels of 128 channels).
+#define VOXEL_ROW(v, d, j, i)                                                              \
+  const int row_ = blockIdx.x * blockDim.y + threadIdx.y;                                  \
+  if (row_ >= (v).D * (v).H) return;                                                       \
+  const int d = row_ / (v).H, j = row_ - d * (v).H;                                        \
+  for (int i = threadIdx.x; i < (v).W; i += blockDim.x)
+static dim3 row_block(const Vol& v) {
+  unsigned tx = 4;
+  while (tx < (unsigned)v.W && tx < 128) tx <<= 1;
+  return dim3(tx, 256 / tx);
+}
+static dim3 row_grid(const Vol& v, int G) {
+  const unsigned ty = row_block(v).y;
+  return dim3(((unsigned)(v.D * v.H) + ty - 1) / ty, G);
+}
+
 // input (2 channels, dense FP32) -> block 0 of the level-0 input tensor
-__global__ void k_pack_x(Vol v, const float* __restrict__ x, __nv_bfloat16* X) {
+__global__ void __launch_bounds__(256) k_pack_x(Vol v, const float* __restrict__ x, __nv_bfloat16* X) {
   const long long nv = (long long)v.D * v.H * v.W;
-  VOXELS(v, n) {
-    int d, j, i;
-    decode(v, n, d, j, i);
+  VOXEL_ROW(v, d, j, i) {
+    const long long n = (long long)row_ * v.W + i;
     float f[8] = {x[n], x[nv + n], 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     st_row(X, v, 0, vrow(v, d, j, i), pack8(f));
   }
 }
 
-// out[coarse] = mean of the 8 children (all blocks)
-__global__ void k_pool(Vol vf, Vol vc, int G, const __nv_bfloat16* in, __nv_bfloat16* out) {
-  VOXELS(vc, n) {
-    int d, j, i;
-    decode(vc, n, d, j, i);
-    for (int g = 0; g < G; ++g) {
-      float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      for (int c = 0; c < 8; ++c) {
-        float f[8];
-        unpack8(ld_row(in, vf, g, vrow(vf, 2 * d + (c >> 2), 2 * j + ((c >> 1) & 1), 2 * i + (c & 1))), f);
+// the 8 children of coarse voxel (d, j, i) summed in order, one channel block
+__device__ __forceinline__ void sum_children(const Vol& vf, int g, int d, int j, int i, const __nv_bfloat16* in, float* acc) {
+  uint4 u[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] += f[k];
-      }
+  for (int c = 0; c < 8; ++c) u[c] = ld_row(in, vf, g, vrow(vf, 2 * d + (c >> 2), 2 * j + ((c >> 1) & 1), 2 * i + (c & 1)));
 #pragma unroll
-      for (int k = 0; k < 8; ++k) acc[k] *= 0.125f;
-      st_row(out, vc, g, vrow(vc, d, j, i), pack8(acc));
-    }
+  for (int k = 0; k < 8; ++k) acc[k] = 0.f;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    float f[8];
+    unpack8(u[c], f);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc[k] += f[k];
+  }
+}
+
+// out[coarse] = mean of the 8 children
+__global__ void __launch_bounds__(256) k_pool(Vol vf, Vol vc, const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ out) {
+  const int g = blockIdx.y;
+  VOXEL_ROW(vc, d, j, i) {
+    float acc[8];
+    sum_children(vf, g, d, j, i, in, acc);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc[k] *= 0.125f;
+    st_row(out, vc, g, vrow(vc, d, j, i), pack8(acc));
   }
 }
 
 // out[fine] = in[parent]
-__global__ void k_upsample(Vol vc, Vol vf, int G, const __nv_bfloat16* in, __nv_bfloat16* out) {
-  VOXELS(vf, n) {
-    int d, j, i;
-    decode(vf, n, d, j, i);
-    const long long rc = vrow(vc, d >> 1, j >> 1, i >> 1), rf = vrow(vf, d, j, i);
-    for (int g = 0; g < G; ++g) st_row(out, vf, g, rf, ld_row(in, vc, g, rc));
-  }
+__global__ void __launch_bounds__(256) k_upsample(Vol vc, Vol vf, const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ out) {
+  const int g = blockIdx.y;
+  VOXEL_ROW(vf, d, j, i) st_row(out, vf, g, vrow(vf, d, j, i), ld_row(in, vc, g, vrow(vc, d >> 1, j >> 1, i >> 1)));
 }
 
 // adjoint of upsampling: out[coarse] = sum of the 8 children of in
-__global__ void k_upsample_back(Vol vf, Vol vc, int G, const __nv_bfloat16* in, __nv_bfloat16* out) {
-  VOXELS(vc, n) {
-    int d, j, i;
-    decode(vc, n, d, j, i);
-    for (int g = 0; g < G; ++g) {
-      float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      for (int c = 0; c < 8; ++c) {
-        float f[8];
-        unpack8(ld_row(in, vf, g, vrow(vf, 2 * d + (c >> 2), 2 * j + ((c >> 1) & 1), 2 * i + (c & 1))), f);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] += f[k];
-      }
-      st_row(out, vc, g, vrow(vc, d, j, i), pack8(acc));
-    }
+__global__ void __launch_bounds__(256) k_upsample_back(Vol vf, Vol vc, const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ out) {
+  const int g = blockIdx.y;
+  VOXEL_ROW(vc, d, j, i) {
+    float acc[8];
+    sum_children(vf, g, d, j, i, in, acc);
+    st_row(out, vc, g, vrow(vc, d, j, i), pack8(acc));
   }
 }
 
 // gradient at an encoder output: out[fine] = (skip[fine] + dp[parent] / 8) where e[fine] > 0
-__global__ void k_pool_back(Vol vf, Vol vc, int G, const __nv_bfloat16* skip, const __nv_bfloat16* dp,
-                            const __nv_bfloat16* e, __nv_bfloat16* out) {
-  VOXELS(vf, n) {
-    int d, j, i;
-    decode(vf, n, d, j, i);
+__global__ void __launch_bounds__(256) k_pool_back(Vol vf, Vol vc, const __nv_bfloat16* __restrict__ skip,
+                                                   const __nv_bfloat16* __restrict__ dp, const __nv_bfloat16* __restrict__ e,
+                                                   __nv_bfloat16* __restrict__ out) {
+  const int g = blockIdx.y;
+  VOXEL_ROW(vf, d, j, i) {
     const long long rf = vrow(vf, d, j, i), rc = vrow(vc, d >> 1, j >> 1, i >> 1);
-    for (int g = 0; g < G; ++g) {
-      float s[8], p[8], m[8];
-      unpack8(ld_row(skip, vf, g, rf), s);
-      unpack8(ld_row(dp, vc, g, rc), p);
-      unpack8(ld_row(e, vf, g, rf), m);
+    float s[8], p[8], m[8];
+    unpack8(ld_row(skip, vf, g, rf), s);
+    unpack8(ld_row(dp, vc, g, rc), p);
+    unpack8(ld_row(e, vf, g, rf), m);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) s[k] = m[k] > 0.f ? s[k] + 0.125f * p[k] : 0.f;
-      st_row(out, vf, g, rf, pack8(s));
-    }
+    for (int k = 0; k < 8; ++k) s[k] = m[k] > 0.f ? s[k] + 0.125f * p[k] : 0.f;
+    st_row(out, vf, g, rf, pack8(s));
   }
 }
 
 // output layer: y = sum_c w[c] d0[c]
-__global__ void k_out_fwd(Vol v, const __nv_bfloat16* d0, const float* __restrict__ w, float* y) {
+__global__ void __launch_bounds__(256) k_out_fwd(Vol v, const __nv_bfloat16* __restrict__ d0, const float* __restrict__ w, float* __restrict__ y) {
   __shared__ float ws[kOutC];
-  if (threadIdx.x < kOutC) ws[threadIdx.x] = w[threadIdx.x];
+  const int t = threadIdx.y * blockDim.x + threadIdx.x;
+  if (t < kOutC) ws[t] = w[t];
   __syncthreads();
-  VOXELS(v, n) {
-    int d, j, i;
-    decode(v, n, d, j, i);
+  VOXEL_ROW(v, d, j, i) {
     const long long r = vrow(v, d, j, i);
     float a[8], b[8];
     unpack8(ld_row(d0, v, 0, r), a);
@@ -228,7 +239,7 @@ __global__ void k_out_fwd(Vol v, const __nv_bfloat16* d0, const float* __restric
     float s = 0.f;
 #pragma unroll
     for (int k = 0; k < 8; ++k) s += ws[k] * a[k] + ws[8 + k] * b[k];
-    y[n] = s;
+    y[(long long)row_ * v.W + i] = s;
   }
 }
 
@@ -689,28 +700,28 @@ static void rebuild_images(unet_handle* n, cudaStream_t st) {
 
 static cudaError_t forward(unet_handle* n, const float* x, float* y, cudaStream_t st) {
   const Vol* V = n->vol;
-  ULAUNCH(grid_for((long long)V[0].D * V[0].H * V[0].W), 256, 0, st, k_pack_x)(V[0], x, n->X.p);
+  ULAUNCH(row_grid(V[0], 1), row_block(V[0]), 0, st, k_pack_x)(V[0], x, n->X.p);
   conv(n, E0A, false, n->X, nullptr, n->E0A, nullptr, nullptr, nullptr, true, st);
   conv(n, E0B, false, n->E0A, nullptr, n->E0, nullptr, nullptr, nullptr, true, st);
-  ULAUNCH(grid_for((long long)V[1].D * V[1].H * V[1].W), 256, 0, st, k_pool)(V[0], V[1], 2, n->E0.p, n->P1.p);
+  ULAUNCH(row_grid(V[1], 2), row_block(V[1]), 0, st, k_pool)(V[0], V[1], n->E0.p, n->P1.p);
   conv(n, E1A, false, n->P1, nullptr, n->E1A, nullptr, nullptr, nullptr, true, st);
   conv(n, E1B, false, n->E1A, nullptr, n->E1, nullptr, nullptr, nullptr, true, st);
-  ULAUNCH(grid_for((long long)V[2].D * V[2].H * V[2].W), 256, 0, st, k_pool)(V[1], V[2], 4, n->E1.p, n->P2.p);
+  ULAUNCH(row_grid(V[2], 4), row_block(V[2]), 0, st, k_pool)(V[1], V[2], n->E1.p, n->P2.p);
   conv(n, E2A, false, n->P2, nullptr, n->E2A, nullptr, nullptr, nullptr, true, st);
   conv(n, E2B, false, n->E2A, nullptr, n->E2, nullptr, nullptr, nullptr, true, st);
-  ULAUNCH(grid_for((long long)V[3].D * V[3].H * V[3].W), 256, 0, st, k_pool)(V[2], V[3], 8, n->E2.p, n->P3.p);
+  ULAUNCH(row_grid(V[3], 8), row_block(V[3]), 0, st, k_pool)(V[2], V[3], n->E2.p, n->P3.p);
   conv(n, E3A, false, n->P3, nullptr, n->E3A, nullptr, nullptr, nullptr, true, st);
   conv(n, E3B, false, n->E3A, nullptr, n->E3, nullptr, nullptr, nullptr, true, st);
-  ULAUNCH(grid_for((long long)V[2].D * V[2].H * V[2].W), 256, 0, st, k_upsample)(V[3], V[2], 16, n->E3.p, n->U2.p);
+  ULAUNCH(row_grid(V[2], 16), row_block(V[2]), 0, st, k_upsample)(V[3], V[2], n->E3.p, n->U2.p);
   conv(n, D2A, false, n->U2, &n->E2, n->D2A, nullptr, nullptr, nullptr, true, st);
   conv(n, D2B, false, n->D2A, nullptr, n->D2, nullptr, nullptr, nullptr, true, st);
-  ULAUNCH(grid_for((long long)V[1].D * V[1].H * V[1].W), 256, 0, st, k_upsample)(V[2], V[1], 8, n->D2.p, n->U1.p);
+  ULAUNCH(row_grid(V[1], 8), row_block(V[1]), 0, st, k_upsample)(V[2], V[1], n->D2.p, n->U1.p);
   conv(n, D1A, false, n->U1, &n->E1, n->D1A, nullptr, nullptr, nullptr, true, st);
   conv(n, D1B, false, n->D1A, nullptr, n->D1, nullptr, nullptr, nullptr, true, st);
-  ULAUNCH(grid_for((long long)V[0].D * V[0].H * V[0].W), 256, 0, st, k_upsample)(V[1], V[0], 4, n->D1.p, n->U0.p);
+  ULAUNCH(row_grid(V[0], 4), row_block(V[0]), 0, st, k_upsample)(V[1], V[0], n->D1.p, n->U0.p);
   conv(n, D0A, false, n->U0, &n->E0, n->D0A, nullptr, nullptr, nullptr, true, st);
   conv(n, D0B, false, n->D0A, nullptr, n->D0, nullptr, nullptr, nullptr, true, st);
-  ULAUNCH(grid_for((long long)V[0].D * V[0].H * V[0].W), 256, 0, st, k_out_fwd)(V[0], n->D0.p, n->wout, y);
+  ULAUNCH(row_grid(V[0], 1), row_block(V[0]), 0, st, k_out_fwd)(V[0], n->D0.p, n->wout, y);
   return cudaGetLastError();
 }
 
@@ -730,39 +741,39 @@ static cudaError_t backward(unet_handle* n, const float* dy, const float* t, int
   conv(n, D0B, true, n->GD0, nullptr, n->GD0A, nullptr, &n->D0A, nullptr, false, st);
   wgrad(n, D0A, n->U0, &n->E0, n->GD0A, st);
   conv(n, D0A, true, n->GD0A, nullptr, n->GU0, &n->GE0S, &n->U0, &n->E0, false, st);
-  ULAUNCH(grid_for((long long)V[1].D * V[1].H * V[1].W), 256, 0, st, k_upsample_back)(V[0], V[1], 4, n->GU0.p, n->GD1.p);
+  ULAUNCH(row_grid(V[1], 4), row_block(V[1]), 0, st, k_upsample_back)(V[0], V[1], n->GU0.p, n->GD1.p);
   // level 1 decoder
   wgrad(n, D1B, n->D1A, nullptr, n->GD1, st);
   conv(n, D1B, true, n->GD1, nullptr, n->GD1A, nullptr, &n->D1A, nullptr, false, st);
   wgrad(n, D1A, n->U1, &n->E1, n->GD1A, st);
   conv(n, D1A, true, n->GD1A, nullptr, n->GU1, &n->GE1S, &n->U1, &n->E1, false, st);
-  ULAUNCH(grid_for((long long)V[2].D * V[2].H * V[2].W), 256, 0, st, k_upsample_back)(V[1], V[2], 8, n->GU1.p, n->GD2.p);
+  ULAUNCH(row_grid(V[2], 8), row_block(V[2]), 0, st, k_upsample_back)(V[1], V[2], n->GU1.p, n->GD2.p);
   // level 2 decoder
   wgrad(n, D2B, n->D2A, nullptr, n->GD2, st);
   conv(n, D2B, true, n->GD2, nullptr, n->GD2A, nullptr, &n->D2A, nullptr, false, st);
   wgrad(n, D2A, n->U2, &n->E2, n->GD2A, st);
   conv(n, D2A, true, n->GD2A, nullptr, n->GU2, &n->GE2S, &n->U2, &n->E2, false, st);
-  ULAUNCH(grid_for((long long)V[3].D * V[3].H * V[3].W), 256, 0, st, k_upsample_back)(V[2], V[3], 16, n->GU2.p, n->GE3.p);
+  ULAUNCH(row_grid(V[3], 16), row_block(V[3]), 0, st, k_upsample_back)(V[2], V[3], n->GU2.p, n->GE3.p);
   // level 3
   wgrad(n, E3B, n->E3A, nullptr, n->GE3, st);
   conv(n, E3B, true, n->GE3, nullptr, n->GE3A, nullptr, &n->E3A, nullptr, false, st);
   wgrad(n, E3A, n->P3, nullptr, n->GE3A, st);
   conv(n, E3A, true, n->GE3A, nullptr, n->GP3, nullptr, nullptr, nullptr, false, st);
-  ULAUNCH(grid_for((long long)V[2].D * V[2].H * V[2].W), 256, 0, st, k_pool_back)(V[2], V[3], 8, n->GE2S.p, n->GP3.p,
+  ULAUNCH(row_grid(V[2], 8), row_block(V[2]), 0, st, k_pool_back)(V[2], V[3], n->GE2S.p, n->GP3.p,
                                                                                    n->E2.p, n->GE2.p);
   // level 2 encoder
   wgrad(n, E2B, n->E2A, nullptr, n->GE2, st);
   conv(n, E2B, true, n->GE2, nullptr, n->GE2A, nullptr, &n->E2A, nullptr, false, st);
   wgrad(n, E2A, n->P2, nullptr, n->GE2A, st);
   conv(n, E2A, true, n->GE2A, nullptr, n->GP2, nullptr, nullptr, nullptr, false, st);
-  ULAUNCH(grid_for((long long)V[1].D * V[1].H * V[1].W), 256, 0, st, k_pool_back)(V[1], V[2], 4, n->GE1S.p, n->GP2.p,
+  ULAUNCH(row_grid(V[1], 4), row_block(V[1]), 0, st, k_pool_back)(V[1], V[2], n->GE1S.p, n->GP2.p,
                                                                                    n->E1.p, n->GE1.p);
   // level 1 encoder
   wgrad(n, E1B, n->E1A, nullptr, n->GE1, st);
   conv(n, E1B, true, n->GE1, nullptr, n->GE1A, nullptr, &n->E1A, nullptr, false, st);
   wgrad(n, E1A, n->P1, nullptr, n->GE1A, st);
   conv(n, E1A, true, n->GE1A, nullptr, n->GP1, nullptr, nullptr, nullptr, false, st);
-  ULAUNCH(grid_for(nv0), 256, 0, st, k_pool_back)(V[0], V[1], 2, n->GE0S.p, n->GP1.p, n->E0.p, n->GE0.p);
+  ULAUNCH(row_grid(V[0], 2), row_block(V[0]), 0, st, k_pool_back)(V[0], V[1], n->GE0S.p, n->GP1.p, n->E0.p, n->GE0.p);
   // level 0 encoder
   wgrad(n, E0B, n->E0A, nullptr, n->GE0, st);
   conv(n, E0B, true, n->GE0, nullptr, n->GE0A, nullptr, &n->E0A, nullptr, false, st);

@@ -89,32 +89,39 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv3(const __grid_constant
   tc::fence_after_sync();
   const uint32_t tmem = *tslot;
   int issued = 0;
-  if (warp == 0 && lane == 0) {
-    // producer: one input slab (two 8-channel blocks) and one weight image per stage
+  if (warp == 0) {
+    // producer: one input slab (two 8-channel blocks) and one weight image per
+    // stage; lane 0 waits and copies, and where the CTA takes part of the output
+    // channels the lanes copy the image's 18 pieces side by side (one lane issuing
+    // them all bounded the kernel at few voxels of many channels)
     for (int s = 0; s < nst; ++s) {
       const int b = s % a.nstage;
-      if (s >= a.nstage && !tc::mbar_wait(&empty[b], ((s / a.nstage) - 1) & 1, kWaitNs)) {
-        atomicOr(a.err, kErrWaitProducer);
-        *abort_flag = 1;
-        break;
+      int go = 1;
+      if (lane == 0) {
+        if (s >= a.nstage && !tc::mbar_wait(&empty[b], ((s / a.nstage) - 1) & 1, kWaitNs)) {
+          atomicOr(a.err, kErrWaitProducer);
+          *abort_flag = 1;
+        }
+        go = !*abort_flag;
       }
-      if (*abort_flag) break;
+      if (!__shfl_sync(0xffffffffu, go, 0)) break;
       const int dz = s / a.nchunk, c = s - dz * a.nchunk;
       uint8_t* A = smem + (size_t)b * a.stage_bytes;
       uint8_t* B = A + a.a_bytes;
-      tc::mbar_arrive_expect_tx(&full[b], a.a_bytes + a.b_bytes);
-      const __nv_bfloat16* src = c < a.nchunk0 ? a.src0 : a.src1;
-      const long long g0 = 2ll * (c < a.nchunk0 ? c : c - a.nchunk0);
-      const long long start = r0 + (long long)(dz - 1) * a.v.P - a.v.Wp - 1;
-      tc::bulk_g2s(A, src + (g0 * a.v.rows + start) * 8, (uint32_t)a.R * 16u, &full[b]);
-      tc::bulk_g2s(A + (size_t)a.R * 16, src + ((g0 + 1) * a.v.rows + start) * 8, (uint32_t)a.R * 16u, &full[b]);
       const __nv_bfloat16* wst = a.wimg + (size_t)s * 18u * (size_t)a.cout * 8u;
-      if (a.nc == a.cout) {
-        tc::bulk_g2s(B, wst, a.b_bytes, &full[b]);
-      } else {  // this CTA's rows of every tap and channel block
+      if (lane == 0) {
+        tc::mbar_arrive_expect_tx(&full[b], a.a_bytes + a.b_bytes);
+        const __nv_bfloat16* src = c < a.nchunk0 ? a.src0 : a.src1;
+        const long long g0 = 2ll * (c < a.nchunk0 ? c : c - a.nchunk0);
+        const long long start = r0 + (long long)(dz - 1) * a.v.P - a.v.Wp - 1;
+        tc::bulk_g2s(A, src + (g0 * a.v.rows + start) * 8, (uint32_t)a.R * 16u, &full[b]);
+        tc::bulk_g2s(A + (size_t)a.R * 16, src + ((g0 + 1) * a.v.rows + start) * 8, (uint32_t)a.R * 16u, &full[b]);
+        if (a.nc == a.cout) tc::bulk_g2s(B, wst, a.b_bytes, &full[b]);
+      }
+      __syncwarp();  // the copies below count on the expectation above
+      if (a.nc != a.cout && lane < 18) {  // this CTA's rows of every tap and channel block
         const uint32_t nb = (uint32_t)a.nc * 16u;
-        for (int q = 0; q < 18; ++q)
-          tc::bulk_g2s(B + (size_t)q * nb, wst + ((size_t)q * a.cout + n0) * 8u, nb, &full[b]);
+        tc::bulk_g2s(B + (size_t)lane * nb, wst + ((size_t)lane * a.cout + n0) * 8u, nb, &full[b]);
       }
       issued = s + 1;
     }
@@ -610,9 +617,11 @@ void launch_wgrad(const WgradArgs& a, cudaStream_t s) {
   }
   const int gy = a.taps == 9 ? 3 : 9;
   const int gz = (a.gin + 15) / 16;
-  long long gx = (2ll * sms + gy * gz - 1) / (gy * gz);
-  gx = std::max(1ll, std::min(gx, a.nchunks));
   const size_t smem = smem_floor((size_t)a.smem_main + 256, a.tmem_cols);
+  // one wave: as many CTAs as are resident at once (rounding up left two CTAs for
+  // a wave of their own)
+  const long long per_sm = std::max<long long>(1, std::min<long long>(512 / a.tmem_cols, kSmemPerSM / (smem + 1024)));
+  const long long gx = std::max(1ll, std::min(per_sm * sms / (gy * gz), a.nchunks));
   ++g_launches;
   k_wgrad<<<dim3((unsigned)gx, gy, gz), kConvThreads, smem, s>>>(a);
 }
