@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kSortBlock) k_radix_scatter(const unsigned lon
 static int radix_passes(const SortBuffers& b, const unsigned long long* n_dev, int bit0, int bit1, cudaStream_t s,
                         const int* skip);
 
-static bool capturing(cudaStream_t s) {
+bool capturing(cudaStream_t s) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   return cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusActive;
 }
@@ -159,8 +159,7 @@ EventOrder event_order_begin(const SortBuffers& b, cudaStream_t s) {
   return o;
 }
 
-static cudaError_t radix_if_node(const SortBuffers& b, const EventOrder& o, const unsigned long long* n_dev, int bits,
-                                 cudaStream_t s) {
+cudaError_t if_node(const EventOrder& o, cudaStream_t s, cudaStream_t aux, const std::function<void(cudaStream_t)>& body) {
   if (!o.use_graph) return cudaErrorIllegalState;
   cudaStreamCaptureStatus status;
   cudaGraph_t g;
@@ -176,25 +175,25 @@ static cudaError_t radix_if_node(const SortBuffers& b, const EventOrder& o, cons
   np.conditional.size = 1;
   cudaGraphNode_t node;
   if ((e = cudaGraphAddNode(&node, g, deps, edges, ndeps, &np))) return e;
-  cudaGraph_t body = np.conditional.phGraph_out[0];
-  if ((e = cudaStreamBeginCaptureToGraph(b.aux, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed))) return e;
-  radix_passes(b, n_dev, 0, bits, b.aux, nullptr);
+  cudaGraph_t in = np.conditional.phGraph_out[0];
+  if ((e = cudaStreamBeginCaptureToGraph(aux, in, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed))) return e;
+  body(aux);
   cudaGraph_t tmp;
-  const cudaError_t e1 = cudaStreamEndCapture(b.aux, &tmp);
+  const cudaError_t e1 = cudaStreamEndCapture(aux, &tmp);
   if ((e = cudaGetLastError()) || (e = e1)) return e;
   return cudaStreamUpdateCaptureDependencies(s, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
+}
+
+void invalidate_capture(cudaStream_t s) {
+  cudaStreamSynchronize(s);
+  cudaGetLastError();
 }
 
 int event_order_end(const SortBuffers& b, const EventOrder& o, const unsigned long long* n_dev, int bits,
                     cudaStream_t s) {
   if (!capturing(s)) return radix_passes(b, n_dev, 0, bits, s, b.small_done);
-  if (radix_if_node(b, o, n_dev, bits, s) != cudaSuccess) {
-    // a half-built node must not be replayed: synchronising a capturing
-    // stream is illegal and invalidates the capture, so the recording
-    // fails and the instance steps directly from then on
-    cudaStreamSynchronize(s);
-    cudaGetLastError();
-  }
+  if (if_node(o, s, b.aux, [&](cudaStream_t t) { radix_passes(b, n_dev, 0, bits, t, nullptr); }) != cudaSuccess)
+    invalidate_capture(s);
   return ((bits + 7) / 8) & 1;
 }
 
@@ -312,7 +311,8 @@ __global__ void __launch_bounds__(kSortBlock) k_seg_sort_big(long long ncell, co
                                                              const unsigned long long* n_dev,
                                                              const unsigned long long* __restrict__ v,
                                                              uint32_t* __restrict__ perm,
-                                                             const int32_t* __restrict__ big, SegCtl* ctl) {
+                                                             const int32_t* __restrict__ big, SegCtl* ctl,
+                                                             cudaGraphConditionalHandle h_radix, int use_graph) {
   __shared__ unsigned long long sv[kSegBig];
   const long long n = (long long)*n_dev;
   const int nbig = ctl->nbig;
@@ -322,7 +322,10 @@ __global__ void __launch_bounds__(kSortBlock) k_seg_sort_big(long long ncell, co
     const long long b = c < ncell ? cs[c + 1] : n;
     const int m = (int)(b - a);
     if (m > kSegBig) {  // the same m in every thread: the block skips together
-      if (threadIdx.x == 0) ctl->overflow = 1;
+      if (threadIdx.x == 0) {
+        ctl->overflow = 1;
+        if (use_graph) cudaGraphSetConditional(h_radix, 1u);
+      }
       continue;
     }
     __syncthreads();  // the previous bucket's readers are done with sv
@@ -351,79 +354,119 @@ void launch_seg_scatter(long long ncell, long long n_max, const unsigned long lo
 }
 
 void launch_seg_sort(long long ncell, const long long* cell_start, const unsigned long long* n_dev,
-                     const unsigned long long* vals, uint32_t* perm, int32_t* big, SegCtl* ctl, cudaStream_t s) {
+                     const unsigned long long* vals, uint32_t* perm, int32_t* big, SegCtl* ctl, cudaStream_t s,
+                     const EventOrder& radix) {
   PIC_LAUNCH(seg_grid(ncell), kSortBlock, 0, s, k_seg_sort)(ncell, cell_start, n_dev, vals, perm, big, ctl);
   PIC_LAUNCH(8 * sm_count(), kSortBlock, 0, s, k_seg_sort_mid)(ncell, cell_start, n_dev, vals, perm, big, ctl);
-  PIC_LAUNCH(2 * sm_count(), kSortBlock, 0, s, k_seg_sort_big)(ncell, cell_start, n_dev, vals, perm, big, ctl);
+  PIC_LAUNCH(2 * sm_count(), kSortBlock, 0, s, k_seg_sort_big)(ncell, cell_start, n_dev, vals, perm, big, ctl,
+                                                                     radix.handle, radix.use_graph);
 }
 
 // ---------------------------------------------------------------------------
-// exclusive scan int32 -> int64 (three kernels: tile sums, scan of sums, tiles)
+// exclusive scan int32 -> int64 (three kernels: tile sums, scan of sums, tiles).
+// Bound by memory (4 B read twice, 8 B written per count): a warp reads whole
+// 512-byte rows of int4 and writes rows of longlong2 (16 consecutive counts a
+// thread touched 32 lines a load)
 // ---------------------------------------------------------------------------
 constexpr int kScanBlock = 256;
 constexpr int kScanItems = 16;
 constexpr int kScanTile = kScanBlock * kScanItems;
+constexpr int kScanSumsBlock = 1024;
 
 size_t scan_temp_bytes(long long n) {
   const long long tiles = (n + kScanTile - 1) / kScanTile + 1;
   return (size_t)tiles * sizeof(long long);
 }
 
-__device__ __forceinline__ long long block_incl_scan(long long v, long long* sm) {
-  sm[threadIdx.x] = v;
+// sum of v over the threads before this one, and over all (the result is the
+// same for every thread's use of total)
+template <int BLOCK>
+__device__ __forceinline__ long long block_excl_scan(long long v, long long& total) {
+  __shared__ long long sm[BLOCK / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  long long inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  if (lane == 31) sm[w] = inc;
   __syncthreads();
-  for (int o = 1; o < kScanBlock; o <<= 1) {
-    const long long a = threadIdx.x >= o ? sm[threadIdx.x - o] : 0;
-    __syncthreads();
-    sm[threadIdx.x] += a;
-    __syncthreads();
+  long long before = 0, all = 0;
+#pragma unroll
+  for (int q = 0; q < BLOCK / 32; ++q) {
+    before += q < w ? sm[q] : 0;
+    all += sm[q];
   }
-  return sm[threadIdx.x];
+  __syncthreads();  // sm is reused
+  total = all;
+  return before + inc - v;
 }
 
-__global__ void k_scan_tiles(const int32_t* __restrict__ c, long long n, long long* __restrict__ tile_sum) {
-  __shared__ long long sm[kScanBlock];
-  const long long t0 = (long long)blockIdx.x * kScanTile;
-  long long s = 0;
-  for (int k = 0; k < kScanItems; ++k) {
-    const long long i = t0 + (long long)threadIdx.x * kScanItems + k;
-    if (i < n) s += c[i];
-  }
-  const long long inc = block_incl_scan(s, sm);
-  if (threadIdx.x == kScanBlock - 1) tile_sum[blockIdx.x] = inc;
+// the tile's counts, four neighbours a thread and row (0 beyond n)
+__device__ __forceinline__ int4 scan_load(const int32_t* __restrict__ c, long long n, long long i) {
+  if (i + 4 <= n) return *reinterpret_cast<const int4*>(c + i);
+  return make_int4(i < n ? c[i] : 0, i + 1 < n ? c[i + 1] : 0, i + 2 < n ? c[i + 2] : 0, 0);
 }
 
-__global__ void k_scan_sums(long long* tile_sum, int ntiles) {
-  __shared__ long long sm[kScanBlock];
+__global__ void __launch_bounds__(kScanBlock) k_scan_tiles(const int32_t* __restrict__ c, long long n,
+                                                           long long* __restrict__ tile_sum) {
+  const long long t0 = (long long)blockIdx.x * kScanTile + 4 * threadIdx.x;
+  long long s = 0, total;
+#pragma unroll
+  for (int q = 0; q < kScanItems / 4; ++q) {
+    const int4 v = scan_load(c, n, t0 + 4ll * kScanBlock * q);
+    s += ((long long)v.x + v.y) + ((long long)v.z + v.w);
+  }
+  block_excl_scan<kScanBlock>(s, total);
+  if (threadIdx.x == 0) tile_sum[blockIdx.x] = total;
+}
+
+__global__ void __launch_bounds__(kScanSumsBlock) k_scan_sums(long long* tile_sum, int ntiles) {
   long long carry = 0;
-  for (int b0 = 0; b0 < ntiles; b0 += kScanBlock) {
-    const int i = b0 + threadIdx.x;
-    const long long v = i < ntiles ? tile_sum[i] : 0;
-    const long long inc = block_incl_scan(v, sm);
-    if (i < ntiles) tile_sum[i] = carry + inc - v;  // exclusive
-    __syncthreads();
-    carry += sm[kScanBlock - 1];
-    __syncthreads();
+  for (int b0 = 0; b0 < ntiles; b0 += 4 * kScanSumsBlock) {
+    const int i = b0 + 4 * threadIdx.x;
+    long long v[4], s = 0, total;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      v[q] = i + q < ntiles ? tile_sum[i + q] : 0;
+      s += v[q];
+    }
+    long long at = carry + block_excl_scan<kScanSumsBlock>(s, total);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (i + q < ntiles) tile_sum[i + q] = at;  // exclusive
+      at += v[q];
+    }
+    carry += total;
   }
   if (threadIdx.x == 0) tile_sum[ntiles] = carry;
 }
 
-__global__ void k_scan_apply(const int32_t* __restrict__ c, long long n, const long long* __restrict__ tile_sum,
-                             long long* __restrict__ out, int ntiles) {
-  __shared__ long long sm[kScanBlock];
-  const long long t0 = (long long)blockIdx.x * kScanTile;
-  long long loc[kScanItems];
-  long long s = 0;
-  for (int k = 0; k < kScanItems; ++k) {
-    const long long i = t0 + (long long)threadIdx.x * kScanItems + k;
-    loc[k] = s;
-    if (i < n) s += c[i];
-  }
-  const long long inc = block_incl_scan(s, sm);
-  const long long off = tile_sum[blockIdx.x] + inc - s;
-  for (int k = 0; k < kScanItems; ++k) {
-    const long long i = t0 + (long long)threadIdx.x * kScanItems + k;
-    if (i < n) out[i] = off + loc[k];
+__global__ void __launch_bounds__(kScanBlock) k_scan_apply(const int32_t* __restrict__ c, long long n,
+                                                           const long long* __restrict__ tile_sum,
+                                                           long long* __restrict__ out, int ntiles) {
+  const long long t0 = (long long)blockIdx.x * kScanTile + 4 * threadIdx.x;
+  int4 v[kScanItems / 4];
+#pragma unroll
+  for (int q = 0; q < kScanItems / 4; ++q) v[q] = scan_load(c, n, t0 + 4ll * kScanBlock * q);
+  long long off = tile_sum[blockIdx.x];
+#pragma unroll
+  for (int q = 0; q < kScanItems / 4; ++q) {
+    const long long i = t0 + 4ll * kScanBlock * q;
+    long long total;
+    const long long s = ((long long)v[q].x + v[q].y) + ((long long)v[q].z + v[q].w);
+    const long long o0 = off + block_excl_scan<kScanBlock>(s, total);
+    const long long o1 = o0 + v[q].x, o2 = o1 + v[q].y, o3 = o2 + v[q].z;
+    if (i + 4 <= n) {
+      reinterpret_cast<longlong2*>(out + i)[0] = make_longlong2(o0, o1);
+      reinterpret_cast<longlong2*>(out + i)[1] = make_longlong2(o2, o3);
+    } else {
+      if (i < n) out[i] = o0;
+      if (i + 1 < n) out[i + 1] = o1;
+      if (i + 2 < n) out[i + 2] = o2;
+    }
+    off += total;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = tile_sum[ntiles];
 }
@@ -436,7 +479,7 @@ void exclusive_scan_i32_i64(const int32_t* counts, long long n, long long* out, 
     return;
   }
   PIC_LAUNCH(ntiles, kScanBlock, 0, s, k_scan_tiles)(counts, n, ts);
-  PIC_LAUNCH(1, kScanBlock, 0, s, k_scan_sums)(ts, ntiles);
+  PIC_LAUNCH(1, kScanSumsBlock, 0, s, k_scan_sums)(ts, ntiles);
   PIC_LAUNCH(ntiles, kScanBlock, 0, s, k_scan_apply)(counts, n, ts, out, ntiles);
 }
 

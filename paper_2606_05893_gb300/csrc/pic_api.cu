@@ -215,10 +215,10 @@ struct Instance {
   InjectPlan* plan = nullptr;
   bool plan_dirty = true;
   bool plan_used = false;
-  // recorded steps: one graph per (store parity, rho parity), replayed for every
-  // step that neither sorts, nor times phases, nor deposits from scratch
-  cudaGraphExec_t step_exec[4]{};
-  unsigned long long step_kernels[4]{};  // kernel nodes recorded in each
+  // recorded steps: one graph per (store parity, rho parity, sort or not),
+  // replayed for every step that neither times phases nor deposits from scratch
+  cudaGraphExec_t step_exec[8]{};
+  unsigned long long step_kernels[8]{};  // kernel nodes recorded in each
   bool graphs_ok = true;
   cudaStream_t cap_stream = nullptr;  // private stream for recording
   cudaEvent_t cap_done = nullptr;     // end of this instance's branch in a recorded ensemble step
@@ -778,24 +778,19 @@ McArgs mc_args(Instance* I, int proj) {
   return m;
 }
 
-// a2: sort every species by (cell, pid)
+// a2: sort every species by (cell, pid). Nothing is read back: whether a bucket is
+// too large for one block (the species then takes the radix sort of its whole key)
+// is known on the device, and the radix passes sit in an IF node of a recorded
+// step; a step that is not recorded reads it once per species instead.
 template <class S>
 pic_status sort_instance(pic_handle* h, Instance* I) {
   cudaStream_t st = I->stream;
-  CK(h, cudaMemcpyAsync(I->host_cnt, I->cnt, sizeof(DevCounters), cudaMemcpyDeviceToHost, st));
-  CK(h, cudaStreamSynchronize(st));
-  const int pid_bits = std::max(1, bits_for(I->host_cnt->next_pid));
+  const bool rec = capturing(st);
   const int cell_bits = bits_for((unsigned long long)I->g.ncell);
-  const int key_bits = std::min(64, cell_bits + pid_bits);
+  const int key_bits = std::min(64, cell_bits + 32);
   for (int s = 0; s < I->nsp; ++s) {
     const int c = I->cur[s];
     unsigned long long* ndev = &I->cnt->n[c][s];
-    if (I->host_cnt->n[c][s] == 0) {  // nothing to move: offsets all zero; buffers flip as for every species
-      CK(h, cudaMemsetAsync(I->cell_start[s], 0, sizeof(long long) * (I->g.ncell + 1), st));
-      launch_sort_commit(I->cnt, c, s, st);
-      I->cur[s] = c ^ 1;
-      continue;
-    }
     // bucket path: slots, offsets, scatter, per-bucket sort by (pid, index)
     CK(h, cudaMemsetAsync(I->cell_count, 0, sizeof(int32_t) * I->g.ncell, st));
     CK(h, cudaMemsetAsync(I->seg_ctl, 0, sizeof(SegCtl), st));
@@ -804,18 +799,25 @@ pic_status sort_instance(pic_handle* h, Instance* I) {
     exclusive_scan_i32_i64(I->cell_count, I->g.ncell, I->cell_start[s], I->scan_tmp, st);
     launch_seg_scatter(I->g.ncell, I->cap[s], ndev, I->csort.ka, I->csort.va, I->cell_start[s], I->csort.kb,
                        I->csort.vb, st);
-    launch_seg_sort(I->g.ncell, I->cell_start[s], ndev, I->csort.kb, I->csort.vb, I->seg_big, I->seg_ctl, st);
-    CK(h, cudaMemcpyAsync(I->seg_host, I->seg_ctl, sizeof(SegCtl), cudaMemcpyDeviceToHost, st));
-    CK(h, cudaStreamSynchronize(st));
+    const EventOrder o = event_order_begin(I->csort, st);
+    launch_seg_sort(I->g.ncell, I->cell_start[s], ndev, I->csort.kb, I->csort.vb, I->seg_big, I->seg_ctl, st, o);
     const uint32_t* perm = I->csort.vb;
-    if (I->seg_host->overflow) {
-      // a bucket too large for one block: LSD radix sort of the key (cell, pid)
-      launch_cell_keys<S>(I->g, store_of<S>(I, s, c), I->cap[s], ndev, pid_bits, I->csort.ka, I->csort.va, nullptr,
-                          st);
-      SortBuffers b = I->csort;
-      b.n_max = I->cap[s];
-      const int where = radix_sort_pairs(b, ndev, 0, ((key_bits + 7) / 8) * 8, st);
-      perm = where ? b.vb : b.va;
+    // a bucket too large for one block: LSD radix sort of the key (cell, pid)
+    SortBuffers b = I->csort;
+    b.n_max = I->cap[s];
+    auto radix = [&](cudaStream_t t) -> int {
+      launch_cell_keys<S>(I->g, store_of<S>(I, s, c), I->cap[s], ndev, 32, I->csort.ka, I->csort.va, nullptr, t);
+      return radix_sort_pairs(b, ndev, 0, ((key_bits + 7) / 8) * 8, t);
+    };
+    if (rec) {
+      auto body = [&](cudaStream_t t) {
+        if (radix(t) == 0) cudaMemcpyAsync(b.vb, b.va, sizeof(uint32_t) * b.n_max, cudaMemcpyDeviceToDevice, t);
+      };
+      if (if_node(o, st, I->csort.aux, body) != cudaSuccess) invalidate_capture(st);
+    } else {
+      CK(h, cudaMemcpyAsync(I->seg_host, I->seg_ctl, sizeof(SegCtl), cudaMemcpyDeviceToHost, st));
+      CK(h, cudaStreamSynchronize(st));
+      if (I->seg_host->overflow) perm = radix(st) ? b.vb : b.va;
     }
     launch_gather<S>(store_of<S>(I, s, c), store_of<S>(I, s, c ^ 1), perm, ndev, I->cap[s], st);
     launch_sort_commit(I->cnt, c, s, st);
@@ -1195,9 +1197,18 @@ struct HostStepState {
   }
 };
 
+bool sort_due(const Instance* I) {
+  return I->cfg.sort_interval > 0 && I->step % (uint32_t)I->cfg.sort_interval == 0;
+}
+
 // The host-side effect of replaying a recorded step (what step_instance does
-// to the host state of a step that neither sorts nor deposits from scratch).
+// to the host state of a step that does not deposit from scratch).
 void advance_replayed(Instance* I) {
+  if (sort_due(I)) {
+    for (int s = 0; s < I->nsp; ++s) I->cur[s] ^= 1;
+    I->sorted_once = true;
+    I->host_fresh = false;
+  }
   std::swap(I->rho32, I->rho32_next);
   std::swap(I->rho64, I->rho64_next);
   for (int s = 0; s < I->nsp; ++s) std::swap(I->ncount[s], I->ncount_next[s]);
@@ -1206,22 +1217,18 @@ void advance_replayed(Instance* I) {
   I->step += 1;
 }
 
-bool sort_due(const Instance* I) {
-  return I->cfg.sort_interval > 0 && I->step % (uint32_t)I->cfg.sort_interval == 0;
-}
-
 // a step of this instance qualifies for a recorded graph (its own or the ensemble's)
 bool step_recordable(const Instance* I) {
-  return I->graphs_ok && I->next_valid && !sort_due(I) && !I->timer.on && I->solver.exec != nullptr;
+  return I->graphs_ok && I->next_valid && !I->timer.on && I->solver.exec != nullptr;
 }
 
 uint32_t graph_key(const Instance* I) {
   const void* rho_now = I->mixed ? (const void*)I->rho32 : (const void*)I->rho64;
-  return (uint32_t)((I->cur[0] & 1) | (rho_now == I->rho_first ? 2 : 0));
+  return (uint32_t)((I->cur[0] & 1) | (rho_now == I->rho_first ? 2 : 0) | (sort_due(I) ? 4 : 0));
 }
 
 // One step of one instance: replayed from a recorded graph when the step neither
-// sorts nor times phases nor deposits from scratch, else enqueued directly (and
+// times phases nor deposits from scratch, else enqueued directly (and
 // recorded first when it qualifies). Recording runs the same enqueue code with a
 // private stream in capture mode, so the host-side state advances exactly as in
 // a direct step; a replay advances it the same way.
@@ -1302,7 +1309,7 @@ bool ensemble_recordable(const pic_handle* h) {
 bool run_ensemble_step(pic_handle* h) {
   std::vector<uint32_t> key;
   key.reserve(h->inst.size());
-  for (const auto* I : h->inst) key.push_back(graph_key(I) | (I->graph_epoch << 2));
+  for (const auto* I : h->inst) key.push_back(graph_key(I) | (I->graph_epoch << 3));
   for (auto& g : h->ens) {
     if (g.key != key) continue;
     count_graph(g.kernels);

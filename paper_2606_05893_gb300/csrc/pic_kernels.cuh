@@ -2,6 +2,8 @@
 // declarations shared by the kernel translation units and the host runtime.
 #pragma once
 
+#include <functional>
+
 #include "pic_internal.cuh"
 
 namespace pic {
@@ -755,7 +757,8 @@ void launch_seg_scatter(long long ncell, long long n_max, const unsigned long lo
                         const unsigned long long* words, const uint32_t* pids, const long long* cell_start,
                         unsigned long long* out, uint32_t* perm, cudaStream_t s);
 void launch_seg_sort(long long ncell, const long long* cell_start, const unsigned long long* n_dev,
-                     const unsigned long long* vals, uint32_t* perm, int32_t* big, SegCtl* ctl, cudaStream_t s);
+                     const unsigned long long* vals, uint32_t* perm, int32_t* big, SegCtl* ctl, cudaStream_t s,
+                     const EventOrder& radix);
 
 struct SortBuffers {
   unsigned long long *ka, *kb;
@@ -767,6 +770,13 @@ struct SortBuffers {
   cudaStream_t aux;    // capture stream of the radix passes inside a recorded step (small path)
 };
 long long sort_hist_entries(long long n_max);
+bool capturing(cudaStream_t s);
+// An IF node on o's handle at the capture position of s, its body captured on aux.
+cudaError_t if_node(const EventOrder& o, cudaStream_t s, cudaStream_t aux, const std::function<void(cudaStream_t)>& body);
+// A half-built node must not be replayed: synchronising a capturing stream is
+// illegal and invalidates the capture, so the recording fails and the instance
+// steps directly from then on.
+void invalidate_capture(cudaStream_t s);
 EventOrder event_order_begin(const SortBuffers& b, cudaStream_t s);
 int event_order_end(const SortBuffers& b, const EventOrder& o, const unsigned long long* n_dev, int bits, cudaStream_t s);
 int radix_sort_pairs(const SortBuffers& b, const unsigned long long* n_dev, int bit0, int bit1, cudaStream_t s);

@@ -108,3 +108,40 @@ def test_autotuner_times_every_candidate_from_the_same_state():
     assert sim.moments(0)["step"] == before[0]["step"]
     sim.step(2)
     sim.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_recorded_sort_of_an_overfull_cell(pkg, precision):
+    """Sort steps are recorded too; a cell of more than 4096 particles sends its species to the radix
+    sort, which sits in a conditional node there. Steps with and without recording end alike."""
+    from tests._cases import bare
+    wl = bare(nx=4, ny=4, nz=8, weight=1e-6, capacity=1 << 14, phi_a=1.0)
+    wl.sort_interval = 2
+    rng = np.random.default_rng(3)
+
+    def cloud(n):
+        dense = (np.array([1, 2, 3]) + 0.05 + 0.9 * rng.random((n, 3))) * wl.h
+        return np.concatenate([dense, rng.random((500, 3)) * np.array(wl.L)]), rng.standard_normal((n + 500, 3)) * 10.0
+
+    wl.preload = [cloud(5000), cloud(20), cloud(4500)]
+    a = pkg.Simulation(wl, precision=precision, cg_rtol=1e-12)
+    b = pkg.Simulation(wl, precision=precision, cg_rtol=1e-12)
+    pkg.pic_set_profiling(b.h, True)  # timed steps are always enqueued directly
+    a.step(9)
+    b.step(9)
+    for sp in range(3):
+        xa, va, pa = a.particles(sp)
+        xb, vb, pb = b.particles(sp)
+        oa, ob = np.argsort(pa), np.argsort(pb)
+        assert np.array_equal(pa[oa], pb[ob]) and len(np.unique(pa)) == pa.size
+        # deposits sum in another order: FP64 rounding, or the mixed store's parity bounds per step
+        tol_x, tol_v = (1e-10 * max(wl.L), 1e-10) if precision == 0 else (9 * 1e-5 * wl.h, 9 * 1e-5)
+        assert np.abs(xa[oa] - xb[ob]).max() <= tol_x
+        assert np.abs(va[oa] - vb[ob]).max() <= tol_v * np.abs(va).max()
+    a.sort_now()
+    x, v, pid = a.particles(0)
+    cell = np.minimum((x / wl.h).astype(int), np.array([3, 3, 7]))
+    key = (cell[:, 2] * 4 + cell[:, 1]) * 4 + cell[:, 0]
+    assert np.all(np.lexsort((pid, key)) == np.arange(pid.size))
+    a.close()
+    b.close()
