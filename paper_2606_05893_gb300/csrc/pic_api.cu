@@ -94,6 +94,8 @@ namespace {
 
 constexpr int kPushBlocksPerSM = 8;
 constexpr long long kStageHost = 65536;  // largest upload staged on the host (returns before the device runs it)
+constexpr size_t kParticleBytes = 6 * sizeof(double) + 2 * sizeof(uint32_t);  // x, v, pid, multiplicity
+constexpr size_t kSolveKeep = 64ull << 20;
 constexpr int kPhases = PIC_NPHASES;
 
 // CUDA-event timing of the phases of a step on the handle's stream.
@@ -275,6 +277,12 @@ struct Instance {
   double* stage_v = nullptr;
   uint32_t* stage_m = nullptr;  // multiplicities of an upload
   long long stage_cap = 0;
+  // small downloads of particles (kStageHost at most) and solves of a caller's
+  // density (kSolveKeep bytes at most) keep their buffers between calls: allocating
+  // and freeing them took longer than the work
+  void* dl_dev = nullptr;
+  void* dl_host = nullptr;  // pinned
+  void* solve_ws = nullptr;
   // small uploads go through pinned host staging and return without waiting
   // for the device (kStageHost particles at most)
   double* hstage = nullptr;      // x then v, 6 doubles per particle (pinned)
@@ -418,6 +426,9 @@ void free_instance(Instance* I) {
   dev_free(I->stage_x);
   dev_free(I->stage_v);
   dev_free(I->stage_m);
+  dev_free(I->dl_dev);
+  if (I->dl_host) cudaFreeHost(I->dl_host);
+  dev_free(I->solve_ws);
   if (I->hstage) cudaFreeHost(I->hstage);
   if (I->hstage_done) cudaEventDestroy(I->hstage_done);
   I->timer.release();
@@ -1850,27 +1861,38 @@ static pic_status get_particles(pic_handle* h, int32_t inst, int32_t species, in
   *n = live;
   if (cap < live) return fail(h, PIC_EINVAL, "cap %lld below count %lld", (long long)cap, live);
   if (slots == 0) return PIC_OK;
-  double *dx = nullptr, *dv = nullptr;
-  uint32_t *dp = nullptr, *dm = nullptr;
-  CK(h, dalloc(&dx, 3 * (size_t)slots));
-  CK(h, dalloc(&dv, 3 * (size_t)slots));
-  CK(h, dalloc(&dp, (size_t)slots));
-  if (mw) CK(h, dalloc(&dm, (size_t)slots));
+  // one block x, v, pid, multiplicity on the device, copied to the host at once
+  const size_t bytes = (size_t)slots * kParticleBytes;
+  const bool keep = slots <= kStageHost;
+  char *dev = nullptr, *host = nullptr;
+  std::vector<char> big;
+  if (keep) {
+    if (!I->dl_dev) CK(h, dev_malloc(&I->dl_dev, kStageHost * kParticleBytes));
+    if (!I->dl_host) CK(h, cudaMallocHost(&I->dl_host, kStageHost * kParticleBytes));
+    dev = (char*)I->dl_dev;
+    host = (char*)I->dl_host;
+  } else {
+    CK(h, dev_malloc((void**)&dev, bytes));
+    big.resize(bytes);
+    host = big.data();
+  }
+  auto at = [&](char* base, int part) -> char* {  // 0 x, 1 v, 2 pid, 3 multiplicity
+    const size_t d = 3 * sizeof(double) * (size_t)slots;
+    return base + (part < 2 ? part * d : 2 * d + (part - 2) * sizeof(uint32_t) * (size_t)slots);
+  };
+  double *dx = (double*)at(dev, 0), *dv = (double*)at(dev, 1);
+  uint32_t *dp = (uint32_t*)at(dev, 2), *dm = mw ? (uint32_t*)at(dev, 3) : nullptr;
   const int c = I->cur[species];
   if (I->mixed) launch_download<StoreMx>(I->g, I->smx[species][c], slots, dx, dv, dp, dm, h->stream);
   else launch_download<Store64>(I->g, I->s64[species][c], slots, dx, dv, dp, dm, h->stream);
-  std::vector<double> hx(3 * slots), hv(3 * slots);
-  std::vector<uint32_t> hp(slots), hm(mw ? slots : 0);
-  cudaMemcpyAsync(hx.data(), dx, sizeof(double) * 3 * slots, cudaMemcpyDeviceToHost, h->stream);
-  cudaMemcpyAsync(hv.data(), dv, sizeof(double) * 3 * slots, cudaMemcpyDeviceToHost, h->stream);
-  cudaMemcpyAsync(hp.data(), dp, sizeof(uint32_t) * slots, cudaMemcpyDeviceToHost, h->stream);
-  if (mw) cudaMemcpyAsync(hm.data(), dm, sizeof(uint32_t) * slots, cudaMemcpyDeviceToHost, h->stream);
-  cudaError_t e = cudaStreamSynchronize(h->stream);
-  dev_free(dx);
-  dev_free(dv);
-  dev_free(dp);
-  dev_free(dm);
+  cudaError_t e = cudaMemcpyAsync(host, dev, mw ? bytes : bytes - sizeof(uint32_t) * (size_t)slots,
+                                  cudaMemcpyDeviceToHost, h->stream);
+  const cudaError_t e1 = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess) e = e1;
+  if (!keep) dev_free(dev);
   if (e != cudaSuccess) return fail(h, PIC_ECUDA, "download failed: %s", cudaGetErrorString(e));
+  const double *hx = (const double*)at(host, 0), *hv = (const double*)at(host, 1);
+  const uint32_t *hp = (const uint32_t*)at(host, 2), *hm = (const uint32_t*)at(host, 3);
   long long w = 0;
   for (long long i = 0; i < slots; ++i) {
     if (hp[i] == kPidDead) continue;
@@ -1948,16 +1970,24 @@ pic_status pic_solve(pic_handle* h, int32_t inst, const double* rho, double* phi
   cudaStream_t s = h->stream;
   const long long nu = I->solver.n;
   CK(h, ensure_phi64(I, s));
-  double *save_phi = nullptr, *drho = nullptr;
-  float *save32 = nullptr, *save_lo = nullptr;
-  CK(h, dalloc(&save_phi, g.nnode));
-  CK(h, dalloc(&drho, g.nnode));
+  // workspace: the instance's own potential, the density, and MIXED the
+  // float-float state (each part a multiple of 256 bytes)
+  auto part = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
+  const size_t b64 = part(sizeof(double) * (size_t)g.nnode), b32 = I->mixed ? part(sizeof(float) * (size_t)g.nnode) : 0;
+  const size_t blo = I->mixed ? part(sizeof(float) * (size_t)nu) : 0, bytes = 2 * b64 + b32 + blo;
+  void* ws = I->solve_ws;
+  if (!ws) CK(h, dev_malloc(&ws, bytes));
+  if (bytes <= kSolveKeep) I->solve_ws = ws;
+  struct Release {
+    void* p;
+    ~Release() { dev_free(p); }
+  } release{I->solve_ws ? nullptr : ws};
+  double *save_phi = (double*)ws, *drho = (double*)((char*)ws + b64);
+  float *save32 = (float*)((char*)ws + 2 * b64), *save_lo = (float*)((char*)ws + 2 * b64 + b32);
   // the recorded solver works on the instance's potential (and, MIXED, on its
   // float-float state): keep them meanwhile
   CK(h, cudaMemcpyAsync(save_phi, I->phi, sizeof(double) * g.nnode, cudaMemcpyDeviceToDevice, s));
   if (I->mixed) {
-    CK(h, dalloc(&save32, g.nnode));
-    CK(h, dalloc(&save_lo, nu));
     CK(h, cudaMemcpyAsync(save32, I->phi32, sizeof(float) * g.nnode, cudaMemcpyDeviceToDevice, s));
     CK(h, cudaMemcpyAsync(save_lo, I->solver.lo32, sizeof(float) * nu, cudaMemcpyDeviceToDevice, s));
   }
@@ -1984,10 +2014,6 @@ pic_status pic_solve(pic_handle* h, int32_t inst, const double* rho, double* phi
     CK(h, I->solver.invalidate(s));
   }
   cudaError_t e = cudaStreamSynchronize(s);
-  dev_free(save_lo);
-  dev_free(save32);
-  dev_free(drho);
-  dev_free(save_phi);
   if (e != cudaSuccess) return fail(h, PIC_ECUDA, "solve failed: %s", cudaGetErrorString(e));
   if (iters) *iters = r.iters;
   if (resid_rel) *resid_rel = r.resid_rel;
