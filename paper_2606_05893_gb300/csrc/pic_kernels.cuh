@@ -810,7 +810,7 @@ struct MomentsMx {
   double* part;
   unsigned int* ticket;
   float dz_in, dz_top;   // set by the launcher
-  int fe_tx, kin_blocks; // set by the launcher (kin_blocks unused: every block takes both parts)
+  int vec;  // the field energy takes float4 rows
 };
 void launch_moments_mx(const MomentsMx& a, double* out, cudaStream_t s);
 template <class S>

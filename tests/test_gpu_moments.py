@@ -130,3 +130,22 @@ def test_field_energy_of_the_vacuum_gap(pkg):
         tol = 1e-9 if p == pkg.PIC_FP64 else 27 * 2.0 ** -24
         assert abs(sim.moments()["field_energy"] - exact) <= tol * exact
         sim.close()
+
+
+@pytest.mark.parametrize("nx,ny,nz", [(5, 3, 7), (1, 1, 2), (8, 5, 3), (12, 6, 9), (4, 1, 4), (36, 20, 50)])
+def test_mixed_field_energy_over_row_shapes(pkg, nx, ny, nz):
+    """Rows of whole float4s and others, plane counts around the column length: the energy of a random
+    potential against the host's sum over its edges (a column of 16 squares in FP32 stays within 27 u)."""
+    from tests._cases import bare
+    wl = bare(nx=nx, ny=ny, nz=nz, h=5e-9, phi_c=-3.0, phi_a=40.0)
+    sim = pkg.Simulation(wl, precision=pkg.PIC_MIXED)
+    phi = np.random.default_rng(nx * ny * nz).standard_normal((nz + 1, ny, nx)) * 5.0
+    phi[0], phi[nz] = wl.phi_cathode, wl.phi_anode
+    sim.set_phi(phi)
+    stored = sim.phi()
+    fg, fh = sim.moments()["field_energy"], host_field_energy(stored, wl)
+    # the stored deviation from the vacuum potential is what the differences are formed of
+    dev = np.abs(stored).max() + abs(wl.phi_anode) + abs(wl.phi_cathode)
+    slack = 0.5 * W.EPS0 * wl.h * 3 * stored.size * (2 * 2 * dev * (8 * 2.0 ** -24 * dev))
+    assert abs(fg - fh) <= mixed_fe_rounding_bound(stored, wl) + slack
+    sim.close()
