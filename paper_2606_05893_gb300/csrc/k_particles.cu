@@ -17,8 +17,6 @@
 
 namespace pic {
 
-constexpr int kPushBlock = 256;
-constexpr int kPushWarps = kPushBlock / 32;
 constexpr int kIlp = 2;  // particles per thread and round
 
 // ---------------------------------------------------------------------------
@@ -313,7 +311,9 @@ __global__ void k_inject(InjectArgs<S> a) {
 // atomics (summing doubles across lanes would load the narrow FP64 pipe).
 // Every lane of the warp calls it.
 // Shared memory of a push block (one for whichever species the block pushes).
+template <class S>
 struct PushShared {
+  static constexpr int kPushBlock = PTraits<S>::kBlock, kPushWarps = kPushBlock / 32;
   unsigned int wcnt[kPushWarps];
   unsigned long long base;
   // per-thread tallies, each touched by its own thread only (no atomics, no
@@ -326,7 +326,8 @@ struct PushShared {
   float w[kPushWarps][8 * 32];  // a warp's deposit weights, [corner][lane] (conflict-free rows of 32 words)
 };
 template <bool CHARGED, bool NEUTRAL>
-__device__ __forceinline__ void next_deposit(const PushArgs<StoreMx>& a, const ParticleMx& p, bool stored, PushShared& sh) {
+__device__ __forceinline__ void next_deposit(const PushArgs<StoreMx>& a, const ParticleMx& p, bool stored,
+                                             PushShared<StoreMx>& sh) {
   const int lane = threadIdx.x & 31;
   // a lane without a particle gets a key of its own (negative: never a cell)
   const int key = stored ? p.cell : -1 - lane;
@@ -369,7 +370,8 @@ __device__ __forceinline__ void next_deposit(const PushArgs<StoreMx>& a, const P
   }
 }
 template <bool CHARGED, bool NEUTRAL>
-__device__ __forceinline__ void next_deposit(const PushArgs<Store64>& a, const Particle64& p, bool stored, PushShared&) {
+__device__ __forceinline__ void next_deposit(const PushArgs<Store64>& a, const Particle64& p, bool stored,
+                                             PushShared<Store64>&) {
   if (!stored) return;
   if (CHARGED) deposit_one(a.g, p, nullptr, a.nd.rho64, a.nd.qw_h3[a.species]);
   if (NEUTRAL) atomicAdd(&a.nd.ncount[a.species][cell_now(a.g, p)], (int)p.mw);
@@ -392,7 +394,8 @@ __device__ __noinline__ void log_cathode_hit(const HitLog& h, uint32_t pid, int 
 }
 
 template <class S, bool CHARGED, bool MCC, bool NEUTRAL>
-__device__ __forceinline__ void push_block(const PushArgs<S>& a, PushShared& sh) {
+__device__ __forceinline__ void push_block(const PushArgs<S>& a, PushShared<S>& sh) {
+  constexpr int kPushBlock = PTraits<S>::kBlock, kPushWarps = kPushBlock / 32;
   // Each thread advances kIlp particles per round (their loads are issued
   // together, so the memory latency of one hides behind the others). Output
   // slots are reserved once per block and round (one global atomic per
@@ -606,8 +609,8 @@ __device__ __forceinline__ void push_block(const PushArgs<S>& a, PushShared& sh)
 }
 
 template <class S, bool CHARGED, bool MCC, bool NEUTRAL>
-__global__ void __launch_bounds__(kPushBlock, PTraits<S>::kMinBlocks) k_push(const __grid_constant__ PushArgs<S> a) {
-  __shared__ PushShared sh;
+__global__ void __launch_bounds__(PTraits<S>::kBlock, PTraits<S>::kMinBlocks) k_push(const __grid_constant__ PushArgs<S> a) {
+  __shared__ PushShared<S> sh;
   push_block<S, CHARGED, MCC, NEUTRAL>(a, sh);
 }
 
@@ -615,9 +618,9 @@ __global__ void __launch_bounds__(kPushBlock, PTraits<S>::kMinBlocks) k_push(con
 // writes, their sums are atomics either way, and a species that fills only part
 // of the GPU, or ends in a nearly empty wave, leaves the rest to the other.
 template <class S, bool MCC0, bool MCC1>
-__global__ void __launch_bounds__(kPushBlock, PTraits<S>::kMinBlocks)
+__global__ void __launch_bounds__(PTraits<S>::kBlock, PTraits<S>::kMinBlocks)
     k_push_pair(const __grid_constant__ PushArgs<S> a0, const __grid_constant__ PushArgs<S> a1) {
-  __shared__ PushShared sh;
+  __shared__ PushShared<S> sh;
   if (blockIdx.y == 0) push_block<S, true, MCC0, false>(a0, sh);
   else push_block<S, true, MCC1, false>(a1, sh);
 }
@@ -942,21 +945,21 @@ void launch_inject(const InjectArgs<S>& a, int grid, cudaStream_t st) {
 template <class S>
 void launch_push(const PushArgs<S>& a, int role, bool mcc, int grid, cudaStream_t st) {
   if (role == ROLE_NEUTRAL)
-    PIC_LAUNCH(grid, 256, 0, st, k_push<S, false, false, true>)(a);
+    PIC_LAUNCH(grid, PTraits<S>::kBlock, 0, st, k_push<S, false, false, true>)(a);
   else if (mcc)
-    PIC_LAUNCH(grid, 256, 0, st, k_push<S, true, true, false>)(a);
+    PIC_LAUNCH(grid, PTraits<S>::kBlock, 0, st, k_push<S, true, true, false>)(a);
   else
-    PIC_LAUNCH(grid, 256, 0, st, k_push<S, true, false, false>)(a);
+    PIC_LAUNCH(grid, PTraits<S>::kBlock, 0, st, k_push<S, true, false, false>)(a);
 }
 
 
 template <class S>
 void launch_push_pair(const PushArgs<S>& a0, bool mcc0, const PushArgs<S>& a1, bool mcc1, int grid, cudaStream_t st) {
   const dim3 g(grid, 2);
-  if (mcc0 && mcc1) PIC_LAUNCH(g, 256, 0, st, k_push_pair<S, true, true>)(a0, a1);
-  else if (mcc0) PIC_LAUNCH(g, 256, 0, st, k_push_pair<S, true, false>)(a0, a1);
-  else if (mcc1) PIC_LAUNCH(g, 256, 0, st, k_push_pair<S, false, true>)(a0, a1);
-  else PIC_LAUNCH(g, 256, 0, st, k_push_pair<S, false, false>)(a0, a1);
+  if (mcc0 && mcc1) PIC_LAUNCH(g, PTraits<S>::kBlock, 0, st, k_push_pair<S, true, true>)(a0, a1);
+  else if (mcc0) PIC_LAUNCH(g, PTraits<S>::kBlock, 0, st, k_push_pair<S, true, false>)(a0, a1);
+  else if (mcc1) PIC_LAUNCH(g, PTraits<S>::kBlock, 0, st, k_push_pair<S, false, true>)(a0, a1);
+  else PIC_LAUNCH(g, PTraits<S>::kBlock, 0, st, k_push_pair<S, false, false>)(a0, a1);
 }
 
 void launch_resolve_rank(const ResolveArgs& a, int grid, cudaStream_t st) {

@@ -369,11 +369,16 @@ struct PTraits;
 template <>
 struct PTraits<Store64> {
   using P = Particle64;
-  static constexpr int kMinBlocks = 2;  // resident 256-thread push blocks per SM
+  // push blocks: 512 threads per SM either way (128 registers), and a block's
+  // compaction waits for its own four warps alone (64x64x128, per step with 8 warps
+  // 431 us, with 4 422; the mixed store's larger populations lose 1-2 % that way)
+  static constexpr int kBlock = 128;
+  static constexpr int kMinBlocks = 4;  // resident per SM
 };
 template <>
 struct PTraits<StoreMx> {
   using P = ParticleMx;
+  static constexpr int kBlock = 256;
   static constexpr int kMinBlocks = 4;
 };
 
