@@ -130,14 +130,22 @@ __device__ __forceinline__ void dft_odd(float2 (&v)[R], const float2* w, int ste
   }
 }
 
-// One pass over the tile: butterflies of radix R on blocks of L points.
+// One pass over the tiles (one after the other in memory): butterflies of radix R
+// on blocks of L points.
 template <int R, bool INV, int LP>
-__device__ __forceinline__ void fft_pass(float2* Z, const float2* tw, int n, int L, const FastDiv& dM) {
+__device__ __forceinline__ void fft_pass(float2* Z, const float2* tw, int n, int L, const FastDiv& dM, int tiles) {
   const int M = dM.d, nb = n / R, step = n / L, st = M * LP;
-  for (int t = threadIdx.x; t < nb * kDirLines; t += blockDim.x) {
-    const int l = t & (kDirLines - 1), b = t / kDirLines;
+  for (int t = threadIdx.x; t < tiles * nb * kDirLines; t += blockDim.x) {
+    const int l = t & (kDirLines - 1);
+    int b = t / kDirLines;
+    float2* z = Z;
+    if (tiles > 1) {
+      const int tile = (int)((unsigned)b / (unsigned)nb);
+      b -= tile * nb;
+      z += tile * n * LP;
+    }
     const int s = fdiv(b, dM), j = b - s * M;
-    float2* z = Z + (s * L + j) * LP + l;
+    z += (s * L + j) * LP + l;
     const int jw = j * step;
     float2 v[R];
 #pragma unroll
@@ -183,24 +191,24 @@ __device__ void fft_pass_any(const float2* Z, float2* Z2, const float2* tw, int 
 // All passes of an axis on the tile in Z (forward: natural in, digit reversed
 // out; inverse: the reverse). Returns the buffer that holds the result.
 template <bool INV, int LP, bool POW2>
-__device__ __forceinline__ float2* fft_tile(float2* Z, float2* Z2, const float2* tw, const AxisPlan& A) {
+__device__ __forceinline__ float2* fft_tile(float2* Z, float2* Z2, const float2* tw, const AxisPlan& A, int tiles = 1) {
   for (int p = 0; p < A.npass; ++p) {
     const int q = INV ? A.npass - 1 - p : p;
     const int R = A.R[q], L = A.L[q];
     const FastDiv dM = A.dM[q];
     switch (R) {
-      case 2: fft_pass<2, INV, LP>(Z, tw, A.n, L, dM); break;
-      case 4: fft_pass<4, INV, LP>(Z, tw, A.n, L, dM); break;
-      case 8: fft_pass<8, INV, LP>(Z, tw, A.n, L, dM); break;
-      case 16: fft_pass<16, INV, LP>(Z, tw, A.n, L, dM); break;
+      case 2: fft_pass<2, INV, LP>(Z, tw, A.n, L, dM, tiles); break;
+      case 4: fft_pass<4, INV, LP>(Z, tw, A.n, L, dM, tiles); break;
+      case 8: fft_pass<8, INV, LP>(Z, tw, A.n, L, dM, tiles); break;
+      case 16: fft_pass<16, INV, LP>(Z, tw, A.n, L, dM, tiles); break;
       default:
         if constexpr (!POW2) {
           switch (R) {
-            case 3: fft_pass<3, INV, LP>(Z, tw, A.n, L, dM); break;
-            case 5: fft_pass<5, INV, LP>(Z, tw, A.n, L, dM); break;
-            case 7: fft_pass<7, INV, LP>(Z, tw, A.n, L, dM); break;
-            case 11: fft_pass<11, INV, LP>(Z, tw, A.n, L, dM); break;
-            case 13: fft_pass<13, INV, LP>(Z, tw, A.n, L, dM); break;
+            case 3: fft_pass<3, INV, LP>(Z, tw, A.n, L, dM, tiles); break;
+            case 5: fft_pass<5, INV, LP>(Z, tw, A.n, L, dM, tiles); break;
+            case 7: fft_pass<7, INV, LP>(Z, tw, A.n, L, dM, tiles); break;
+            case 11: fft_pass<11, INV, LP>(Z, tw, A.n, L, dM, tiles); break;
+            case 13: fft_pass<13, INV, LP>(Z, tw, A.n, L, dM, tiles); break;
             default: {
               fft_pass_any<INV, LP>(Z, Z2, tw, A.n, R, L, dM);
               float2* t = Z;
@@ -236,6 +244,33 @@ __device__ __forceinline__ float scaled(T v, double scale) {
   else return v;
 }
 
+// The spectra A, B of the two rows packed in line l of a tile, at column c:
+// A = (Z_f + conj Z_-f) / 2, B = (Z_f - conj Z_-f) / 2i; column 0 holds the mean and,
+// for an even n, the Nyquist coefficient. And back: Z_f = A + i B, Z_-f = conj A + i conj B.
+__device__ __forceinline__ void rows_from_line(const DirectArgs& a, const float2* Z, int l, int c, float2& A, float2& B) {
+  const int2 at = __ldg(a.col + c);
+  if (c == 0) {
+    const float2 z0 = Z[l];
+    const float2 zh = a.packed ? Z[at.y * kLpX + l] : make_float2(0.f, 0.f);
+    A = make_float2(z0.x, zh.x);
+    B = make_float2(z0.y, zh.y);
+  } else {
+    const float2 p = Z[at.x * kLpX + l], m = Z[at.y * kLpX + l];
+    A = make_float2(0.5f * (p.x + m.x), 0.5f * (p.y - m.y));
+    B = make_float2(0.5f * (p.y + m.y), 0.5f * (m.x - p.x));
+  }
+}
+__device__ __forceinline__ void line_from_rows(const DirectArgs& a, float2* Z, int l, int c, float2 A, float2 B) {
+  const int2 at = __ldg(a.col + c);
+  if (c == 0) {
+    Z[l] = make_float2(A.x, B.x);
+    if (a.packed) Z[at.y * kLpX + l] = make_float2(A.y, B.y);
+  } else {
+    Z[at.x * kLpX + l] = make_float2(A.x - B.y, A.y + B.x);
+    Z[at.y * kLpX + l] = make_float2(A.x + B.y, B.x - A.y);
+  }
+}
+
 template <class T, bool POW2>
 __global__ void __launch_bounds__(kFftThreads, 3) k_dir_xf(DirectArgs a, const T* __restrict__ in, const SolveCtl* c) {
   pdl_enter();
@@ -268,25 +303,14 @@ __global__ void __launch_bounds__(kFftThreads, 3) k_dir_xf(DirectArgs a, const T
   if constexpr (sizeof(T) == 4) copy_async_wait();
   __syncthreads();
   Z = fft_tile<false, kLpX, POW2>(Z, Z + n * kLpX, tw, a.x);
-  // the two rows' spectra from their packed line: A = (Z_f + conj Z_-f) / 2, B = (Z_f - conj Z_-f) / 2i
   float2* out = reinterpret_cast<float2*>(a.spec);
   for (int l = w; l < kDirLines; l += (int)blockDim.x / 32) {
     const long long r = row0 + 2 * l;
     if (r >= a.rows) break;
     const bool vb = r + 1 < a.rows;
     for (int f = lane; f < a.C; f += 32) {
-      const int2 at = __ldg(a.col + f);
       float2 A, B;
-      if (f == 0) {
-        const float2 z0 = Z[l];
-        const float2 zh = a.packed ? Z[at.y * kLpX + l] : make_float2(0.f, 0.f);
-        A = make_float2(z0.x, zh.x);
-        B = make_float2(z0.y, zh.y);
-      } else {
-        const float2 p = Z[at.x * kLpX + l], m = Z[at.y * kLpX + l];
-        A = make_float2(0.5f * (p.x + m.x), 0.5f * (p.y - m.y));
-        B = make_float2(0.5f * (p.y + m.y), 0.5f * (m.x - p.x));
-      }
+      rows_from_line(a, Z, l, f, A, B);
       out[r * a.C + f] = A;
       if (vb) out[(r + 1) * a.C + f] = B;
     }
@@ -377,6 +401,31 @@ struct Add64 {
   __device__ __forceinline__ void zero(long long u, int) const { x[u] = 0.0; }
 };
 
+// Rows r and r + 1 (if vb) of the potential plus line l of a transformed tile.
+template <class Add>
+__device__ __forceinline__ void add_rows(const Add& add, const float2* Z, int l, long long r, bool vb, int n, int lane,
+                                         float norm, double inv_scale) {
+  constexpr int B = 4;  // points of both rows a thread loads before it stores any
+  for (int i0 = lane; i0 < n; i0 += 32 * B) {
+    typename Add::Val xa[B] = {}, xb[B] = {};
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+      const int i = i0 + 32 * q;
+      if (i >= n) break;
+      xa[q] = add.load(r * n + i);
+      if (vb) xb[q] = add.load((r + 1) * n + i);
+    }
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+      const int i = i0 + 32 * q;
+      if (i >= n) break;
+      const float2 d = Z[i * kLpX + l];
+      add.store(r * n + i, xa[q], d.x * norm, inv_scale);
+      if (vb) add.store((r + 1) * n + i, xb[q], d.y * norm, inv_scale);
+    }
+  }
+}
+
 template <class Add, bool POW2>
 __global__ void __launch_bounds__(kFftThreads, 3) k_dir_xi(DirectArgs a, Add add, const SolveCtl* c) {
   pdl_enter();
@@ -401,14 +450,7 @@ __global__ void __launch_bounds__(kFftThreads, 3) k_dir_xi(DirectArgs a, Add add
     for (int f = lane; f < a.C; f += 32) {
       const float2 A = va ? spec[r * a.C + f] : make_float2(0.f, 0.f);
       const float2 B = vb ? spec[(r + 1) * a.C + f] : make_float2(0.f, 0.f);
-      const int2 at = __ldg(a.col + f);
-      if (f == 0) {
-        Z[l] = make_float2(A.x, B.x);
-        if (a.packed) Z[at.y * kLpX + l] = make_float2(A.y, B.y);
-      } else {  // Z_f = A + i B, Z_-f = conj A + i conj B
-        Z[at.x * kLpX + l] = make_float2(A.x - B.y, A.y + B.x);
-        Z[at.y * kLpX + l] = make_float2(A.x + B.y, B.x - A.y);
-      }
+      line_from_rows(a, Z, l, f, A, B);
     }
   }
   __syncthreads();
@@ -418,26 +460,95 @@ __global__ void __launch_bounds__(kFftThreads, 3) k_dir_xi(DirectArgs a, Add add
     const long long r = row0 + 2 * l;
     const bool va = r < a.rows, vb = r + 1 < a.rows;
     if (!va) break;
-    constexpr int B = 4;  // points of both rows a thread loads before it stores any
-    for (int i0 = lane; i0 < n; i0 += 32 * B) {
-      typename Add::Val xa[B] = {}, xb[B] = {};
-#pragma unroll
-      for (int q = 0; q < B; ++q) {
-        const int i = i0 + 32 * q;
-        if (i >= n) break;
-        xa[q] = add.load(r * n + i);
-        if (vb) xb[q] = add.load((r + 1) * n + i);
-      }
-#pragma unroll
-      for (int q = 0; q < B; ++q) {
-        const int i = i0 + 32 * q;
-        if (i >= n) break;
-        const float2 d = Z[i * kLpX + l];
-        add.store(r * n + i, xa[q], d.x * a.norm, inv_scale);
-        if (vb) add.store((r + 1) * n + i, xb[q], d.y * a.norm, inv_scale);
-      }
-    }
+    add_rows(add, Z, l, r, vb, n, lane, a.norm, inv_scale);
   }
+}
+
+// Whole planes in one block, x and y transforms after one another in shared
+// memory: two launches fewer per pass where a plane is small (measured with
+// separate launches and fused, a whole pass of steps at 32x32x64: 3025 and 2948 us
+// mixed, 4270 and 4053 FP64). Rows pair up within a plane, so ny is even.
+template <class T, bool POW2>
+__global__ void __launch_bounds__(kFftThreads, 3) k_dir_xyf(DirectArgs a, const T* __restrict__ in, const SolveCtl* c) {
+  pdl_enter();
+  if (c->stopped) return;
+  extern __shared__ __align__(16) float2 sm[];
+  const int n = a.nx, m = a.ny, pairs = m / 2, tx = (pairs + kDirLines - 1) / kDirLines;
+  const int ty = (a.C + kDirLines - 1) / kDirLines;
+  float2 *twx = sm, *twy = sm + n, *Z = twy + m, *S = Z + tx * n * kLpX;
+  load_tw(twx, a.x);
+  load_tw(twy, a.y);
+  const double scale = sizeof(T) == 8 ? c->scale : 1.0;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const T* plane = in + (long long)blockIdx.x * n * m;
+  for (int q = w; q < tx * kDirLines; q += nw) {
+    const T* pa = plane + (long long)(2 * q) * n;
+    float2* z = Z + (q / kDirLines) * n * kLpX + (q & (kDirLines - 1));
+    const bool v = q < pairs;
+#pragma unroll 4
+    for (int i = lane; i < n; i += 32) z[i * kLpX] = v ? make_float2(scaled(pa[i], scale), scaled(pa[n + i], scale)) : make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+  fft_tile<false, kLpX, POW2>(Z, nullptr, twx, a.x, tx);
+  for (int q = w; q < pairs; q += nw)
+    for (int f = lane; f < ty * kDirLines; f += 32) {
+      float2 A = make_float2(0.f, 0.f), B = A;
+      if (f < a.C) rows_from_line(a, Z + (q / kDirLines) * n * kLpX, q & (kDirLines - 1), f, A, B);
+      float2* o = S + ((f / kDirLines) * m + 2 * q) * kLpY + (f & (kDirLines - 1));
+      o[0] = A;
+      o[kLpY] = B;
+    }
+  __syncthreads();
+  fft_tile<false, kLpY, POW2>(S, nullptr, twy, a.y, ty);
+  if (a.packed) {
+    split_packed<false>(S, a.y);
+    __syncthreads();
+  }
+  float2* out = reinterpret_cast<float2*>(a.spec) + (long long)blockIdx.x * m * a.C;
+  for (int u = threadIdx.x; u < m * a.C; u += blockDim.x) {
+    const int y = (int)((unsigned)u / (unsigned)a.C), f = u - y * a.C;
+    out[u] = S[((f / kDirLines) * m + y) * kLpY + (f & (kDirLines - 1))];
+  }
+}
+
+template <class Add, bool POW2>
+__global__ void __launch_bounds__(kFftThreads, 3) k_dir_xyi(DirectArgs a, Add add, const SolveCtl* c) {
+  pdl_enter();
+  const int n = a.nx, m = a.ny, pairs = m / 2, tx = (pairs + kDirLines - 1) / kDirLines;
+  const int ty = (a.C + kDirLines - 1) / kDirLines;
+  if (c->stopped) {
+    if (c->bb != 0.0) return;
+    for (int u = threadIdx.x; u < n * m; u += blockDim.x) add.zero((long long)blockIdx.x * n * m + u, blockIdx.x);  // b = 0: x = 0
+    return;
+  }
+  extern __shared__ __align__(16) float2 sm[];
+  float2 *twx = sm, *twy = sm + n, *Z = twy + m, *S = Z + tx * n * kLpX;
+  load_tw(twx, a.x);
+  load_tw(twy, a.y);
+  const float2* spec = reinterpret_cast<const float2*>(a.spec) + (long long)blockIdx.x * m * a.C;
+#pragma unroll 4
+  for (int u = threadIdx.x; u < m * a.C; u += blockDim.x) {
+    const int y = (int)((unsigned)u / (unsigned)a.C), f = u - y * a.C;
+    S[((f / kDirLines) * m + y) * kLpY + (f & (kDirLines - 1))] = spec[u];
+  }
+  __syncthreads();
+  if (a.packed) {
+    split_packed<true>(S, a.y);
+    __syncthreads();
+  }
+  fft_tile<true, kLpY, POW2>(S, nullptr, twy, a.y, ty);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int q = w; q < pairs; q += nw)
+    for (int f = lane; f < a.C; f += 32) {
+      const float2* o = S + ((f / kDirLines) * m + 2 * q) * kLpY + (f & (kDirLines - 1));
+      line_from_rows(a, Z + (q / kDirLines) * n * kLpX, q & (kDirLines - 1), f, o[0], o[kLpY]);
+    }
+  __syncthreads();
+  fft_tile<true, kLpX, POW2>(Z, nullptr, twx, a.x, tx);
+  const double inv_scale = c->inv_scale;
+  for (int q = w; q < pairs; q += nw)
+    add_rows(add, Z + (q / kDirLines) * n * kLpX, q & (kDirLines - 1), (long long)blockIdx.x * m + 2 * q, true, n, lane, a.norm,
+             inv_scale);
 }
 
 // Tridiagonal systems (2 + lambda) u_k - u_(k-1) - u_(k+1) = f_k, zero beyond
@@ -920,6 +1031,7 @@ size_t fft_smem(const AxisPlan& A, int lp) {
 }
 
 constexpr size_t kMaxSmem = 227 * 1024;
+constexpr size_t kPlaneSmem = 16 * 1024;  // planes of about 32 x 32 points (64 x 64 measured no faster, slower in ensembles)
 
 template <class K>
 cudaError_t allow_smem(K k) {
@@ -944,6 +1056,10 @@ bool DirectSolver::plan(int nx, int ny, int nz) {
   a.plane = 2 * a.C * ny;
   a.rows = (long long)ny * P;
   a.norm = (float)(1.0 / ((double)nx * ny));
+  // a whole plane in one block
+  const int tx = (ny / 2 + kDirLines - 1) / kDirLines, ty = (a.C + kDirLines - 1) / kDirLines;
+  smem_xy = sizeof(float2) * ((size_t)nx + ny + (size_t)tx * nx * kLpX + (size_t)ty * ny * kLpY);
+  planes = ny % 2 == 0 && !a.x.pingpong && !a.y.pingpong && smem_xy <= kPlaneSmem;
   zm = P <= 256 ? 16 : 32;
   zw = (P + zm - 1) / zm;
   return true;
@@ -1007,13 +1123,25 @@ void apply(const DirectSolver& D, const T* r, const Add& add, const SolveCtl* c,
   const dim3 gz((a.plane + 31) / 32);
   const int tx = a.nx > 128 ? kFftThreads : kFftThreads / 2, ty = kFftThreads / 2;
   const size_t zsm = sizeof(float) * 32 * (4 * D.zw + D.zm + 1);
+  const auto z = [&]() {
+    if (D.zm == 16) SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<16, 512, 3>)(a, c);
+    else if (D.zw <= 16) SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<32, 512, 2>)(a, c);
+    else SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<32, 1024, 1>)(a, c);
+  };
+  if (D.planes) {
+    const bool pow2 = a.x.pow2 && a.y.pow2;
+    if (pow2) SOLVER_LAUNCH(a.P, kFftThreads, D.smem_xy, s, k_dir_xyf<T, true>)(a, r, c);
+    else SOLVER_LAUNCH(a.P, kFftThreads, D.smem_xy, s, k_dir_xyf<T, false>)(a, r, c);
+    z();
+    if (pow2) SOLVER_LAUNCH(a.P, kFftThreads, D.smem_xy, s, k_dir_xyi<Add, true>)(a, add, c);
+    else SOLVER_LAUNCH(a.P, kFftThreads, D.smem_xy, s, k_dir_xyi<Add, false>)(a, add, c);
+    return;
+  }
   if (a.x.pow2) SOLVER_LAUNCH(gx, tx, D.smem_x, s, k_dir_xf<T, true>)(a, r, c);
   else SOLVER_LAUNCH(gx, tx, D.smem_x, s, k_dir_xf<T, false>)(a, r, c);
   if (a.y.pow2) SOLVER_LAUNCH(gy, ty, D.smem_y, s, k_dir_y<false, true>)(a, c);
   else SOLVER_LAUNCH(gy, ty, D.smem_y, s, k_dir_y<false, false>)(a, c);
-  if (D.zm == 16) SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<16, 512, 3>)(a, c);
-  else if (D.zw <= 16) SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<32, 512, 2>)(a, c);
-  else SOLVER_LAUNCH(gz, 32 * D.zw, zsm, s, k_dir_z<32, 1024, 1>)(a, c);
+  z();
   if (a.y.pow2) SOLVER_LAUNCH(gy, ty, D.smem_y, s, k_dir_y<true, true>)(a, c);
   else SOLVER_LAUNCH(gy, ty, D.smem_y, s, k_dir_y<true, false>)(a, c);
   if (a.x.pow2) SOLVER_LAUNCH(gx, tx, D.smem_x, s, k_dir_xi<Add, true>)(a, add, c);

@@ -54,7 +54,8 @@ struct DirectSolver {
   bool on = false;
   DirectArgs a{};
   void* tables = nullptr;
-  size_t smem_x = 0, smem_y = 0;
+  size_t smem_x = 0, smem_y = 0, smem_xy = 0;
+  bool planes = false;  // whole planes in one block (both axes in one launch each way)
   int zm = 0, zw = 0;  // planes per warp and warps of the tridiagonal kernel
   // nz - 1 unknown planes; on stays false where the sizes do not fit
   cudaError_t init(int nx, int ny, int nz);
