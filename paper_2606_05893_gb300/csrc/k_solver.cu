@@ -21,6 +21,7 @@
 // reads one decision per iteration).
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstdlib>
 #include <cstring>
 #include <type_traits>
@@ -2168,11 +2169,12 @@ cudaError_t Solver::run_host(cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t Solver::phi64_from_ff(cudaStream_t s) {
+cudaError_t Solver::phi64_from_ff(double* x, cudaStream_t s) {
   const Lv L = lv_of(plan[0]);
   const dim3 g((L.pl + 1023) / 1024, L.nz - 1);
-  if (L.pl % 4 == 0) SOLVER_LAUNCH(g, 256, 0, s, k_phi_from_ff<4>)(L, hphi32, lo32, hx, h_phi_c, h_dphi_dk);
-  else SOLVER_LAUNCH(g, 256, 0, s, k_phi_from_ff<1>)(L, hphi32, lo32, hx, h_phi_c, h_dphi_dk);
+  // double2 stores: a caller's array may start on any double
+  if (L.pl % 4 == 0 && (uintptr_t)x % 16 == 0) SOLVER_LAUNCH(g, 256, 0, s, k_phi_from_ff<4>)(L, hphi32, lo32, x, h_phi_c, h_dphi_dk);
+  else SOLVER_LAUNCH(g, 256, 0, s, k_phi_from_ff<1>)(L, hphi32, lo32, x, h_phi_c, h_dphi_dk);
   return cudaGetLastError();
 }
 

@@ -109,8 +109,8 @@ struct Solver {
   void direct_pass(const DirectLoop& d, cudaStream_t s);
   cudaError_t run_host(cudaStream_t s);
   cudaError_t invalidate(cudaStream_t s);
-  // MIXED path: FP64 phi (unknown view, hx) from (hi, lo), and back (x = nullptr: phi = 0)
-  cudaError_t phi64_from_ff(cudaStream_t s);
+  // MIXED path: FP64 phi (unknown view x) from (hi, lo), and back (x = nullptr: phi = 0)
+  cudaError_t phi64_from_ff(double* x, cudaStream_t s);
   cudaError_t ff_from_phi64(const double* x, cudaStream_t s);
   // arguments of the recorded solve (also used by the host-driven loop)
   double* hx = nullptr;
