@@ -65,6 +65,8 @@ struct unet_handle {
   int D = 0, H = 0, W = 0;
   unet::Vol vol[4];
   cudaStream_t stream = nullptr;
+  cudaStream_t side = nullptr;  // the backward pass's weight gradients
+  cudaEvent_t ready = nullptr, joined = nullptr;
   unet::Layer L[unet::kNL];
   float *wout = nullptr, *gout = nullptr, *mout = nullptr, *vout = nullptr;
   float* wbuf = nullptr;  // all master weights, then gradients, m, v (each n_store floats)
@@ -655,7 +657,7 @@ static void conv_impl(unet_handle* n, int l, bool dgrad, const Tensor& s0, const
   launch_conv3(a, st);
 }
 
-static void wgrad(unet_handle* n, int l, const Tensor& s0, const Tensor* s1, const Tensor& dz, cudaStream_t st) {
+static void wgrad_on(unet_handle* n, int l, const Tensor& s0, const Tensor* s1, const Tensor& dz, cudaStream_t st) {
   Layer& L = n->L[l];
   WgradArgs a{};
   const Vol& v = n->vol[s0.level];
@@ -685,6 +687,16 @@ static void wgrad(unet_handle* n, int l, const Tensor& s0, const Tensor* s1, con
   a.nchunks = (v.r_end - v.r_begin + a.Kc - 1) / a.Kc;
   a.err = n->err;
   launch_wgrad(a, st);
+}
+
+// Weight gradients run beside the data gradients, which they do not feed: on the
+// side stream, each after the output gradient that the main stream has written
+// by then (forward and backward at 64x32x32: 1099 us one after the other, 946 us so).
+// The backward pass joins the side stream at its end.
+static void wgrad(unet_handle* n, int l, const Tensor& s0, const Tensor* s1, const Tensor& dz, cudaStream_t st) {
+  cudaEventRecord(n->ready, st);
+  cudaStreamWaitEvent(n->side, n->ready, 0);
+  wgrad_on(n, l, s0, s1, dz, n->side);
 }
 
 static void rebuild_images(unet_handle* n, cudaStream_t st) {
@@ -778,6 +790,8 @@ static cudaError_t backward(unet_handle* n, const float* dy, const float* t, int
   wgrad(n, E0B, n->E0A, nullptr, n->GE0, st);
   conv(n, E0B, true, n->GE0, nullptr, n->GE0A, nullptr, &n->E0A, nullptr, false, st);
   wgrad(n, E0A, n->X, nullptr, n->GE0A, st);
+  if ((e = cudaEventRecord(n->joined, n->side))) return e;
+  if ((e = cudaStreamWaitEvent(st, n->joined, 0))) return e;
   return cudaGetLastError();
 }
 
@@ -1022,6 +1036,9 @@ extern "C" pic_status unet_create(int32_t D, int32_t H, int32_t W, void* cuda_st
   ns += kOutC;
   n->n_store = ns;
   n->wbuf = (float*)dev_alloc(sizeof(float) * 4 * ns);
+  ok = ok && cudaStreamCreateWithFlags(&n->side, cudaStreamNonBlocking) == cudaSuccess &&
+       cudaEventCreateWithFlags(&n->ready, cudaEventDisableTiming) == cudaSuccess &&
+       cudaEventCreateWithFlags(&n->joined, cudaEventDisableTiming) == cudaSuccess;
   n->flat = (float*)dev_alloc(sizeof(float) * num_weights());
   ok = ok && n->wbuf && n->flat;
   if (ok) {
@@ -1108,6 +1125,9 @@ extern "C" pic_status unet_destroy(unet_handle* n) {
   if (n->stream) cudaStreamSynchronize(n->stream);
   collect_times(n);
   for (cudaEvent_t e : n->ev_pool) cudaEventDestroy(e);
+  if (n->side) cudaStreamDestroy(n->side);
+  if (n->ready) cudaEventDestroy(n->ready);
+  if (n->joined) cudaEventDestroy(n->joined);
   for (void* p : n->allocs) pic::dev_free(p);
   delete n;
   pic::dev_handle_closed();
@@ -1234,7 +1254,7 @@ extern "C" pic_status unet_layer_backward(unet_handle* n, int32_t layer, const f
   ULAUNCH(grid_for(nv), 256, 0, st, k_pack_dense)(v, L.def.cout, L.def.cout / 8, dz, tdz.p);
   if (cudaMemsetAsync(L.g, 0, sizeof(float) * L.nw(), st) != cudaSuccess)
     return fail(n, PIC_ECUDA, "unet_layer_backward: memset failed");
-  wgrad(n, layer, tin, nullptr, tdz, st);
+  wgrad_on(n, layer, tin, nullptr, tdz, st);
   conv(n, layer, true, tdz, nullptr, tdx, nullptr, nullptr, nullptr, false, st);
   if (dx) ULAUNCH(grid_for(nv), 256, 0, st, k_unpack_dense)(v, L.def.cin, tdx.p, dx);
   std::vector<float> g(L.nw());
