@@ -680,7 +680,7 @@ __device__ __forceinline__ void finish_event(const ResolveArgs& a, long long e, 
   // successful charge exchanges by primary pid, then the suppressed events
   const bool cx = a.ev[e].kind == XS_CHARGE_EXCHANGE;
   a.sort_keys[e] = ((unsigned long long)(victim < 0 ? 1 : 0) << 33) | ((unsigned long long)(cx ? 1 : 0) << 32) | pid;
-  a.sort_vals[e] = (uint32_t)e;
+  if (a.sort_vals) a.sort_vals[e] = (uint32_t)e;
   if (victim >= 0) {
     atomicAdd(&a.cnt->n_success, 1u);
     if (cx) atomicAdd(&a.cnt->n_success_cx, 1u);
@@ -696,8 +696,8 @@ __global__ void __launch_bounds__(kRankWarps * 32) k_resolve_rank(ResolveArgs a)
   const unsigned int nc = min(a.cnt->n_cands, (unsigned int)a.cand_cap);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     a.cnt->ev_sort_n = ne;
-    *a.order.small = ne <= kSmallEvents ? 1 : 0;
-    if (a.order.use_graph) cudaGraphSetConditional(a.order.handle, ne > kSmallEvents ? 1u : 0u);
+    if (a.order.small) *a.order.small = ne <= kPlacedEvents ? 1 : 0;
+    if (a.order.use_graph) cudaGraphSetConditional(a.order.handle, ne > kPlacedEvents ? 1u : 0u);
   }
   if ((unsigned long long)ne * nc > kScanWork) {
     for (long long e = gtid(); e < ne; e += gstride()) {
@@ -757,6 +757,70 @@ __global__ void __launch_bounds__(kRankWarps * 32) k_resolve_rank(ResolveArgs a)
   }
 }
 
+// Places of events first .. first + m - 1 among all ne events of the step, by key
+// (ties by event): sorted in shared memory (bitonic, padded to a power of two with
+// keys above all), then every key of the step is counted at the first of them that
+// lies above it, and the running sum of those counts is the place. sk: key << 24 |
+// event, ascending; place: of sk[j]. Every block reads all keys (from L2) and no
+// block waits for another, so nothing has to be launched, or held ready in an IF
+// node (9.8 us a step, entered or not), for the few steps with so many events.
+// The work grows with the square of the events: see kPlacedEvents.
+__device__ void place_events(const unsigned long long* __restrict__ keys, unsigned ne, unsigned first, unsigned m,
+                             unsigned long long* sk, unsigned* place) {
+  unsigned P = 32;
+  while (P < m) P <<= 1;
+  for (unsigned j = threadIdx.x; j < P; j += blockDim.x) {
+    sk[j] = j < m ? keys[first + j] << 24 | (first + j) : ~0ull;
+    place[j] = 0;
+  }
+  __syncthreads();
+  for (unsigned k = 2; k <= P; k <<= 1) {
+    for (unsigned d = k >> 1; d > 0; d >>= 1) {
+      for (unsigned t = threadIdx.x; t < P / 2; t += blockDim.x) {
+        const unsigned i = 2 * t - (t & (d - 1));
+        const unsigned long long x = sk[i], y = sk[i + d];
+        if ((x > y) == ((i & k) == 0)) {
+          sk[i] = y;
+          sk[i + d] = x;
+        }
+      }
+      __syncthreads();
+    }
+  }
+  for (unsigned t0 = threadIdx.x; t0 < ne; t0 += 4 * blockDim.x) {
+    unsigned long long kk[4];
+    unsigned lo[4] = {};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const unsigned t = t0 + q * blockDim.x;
+      kk[q] = t < ne ? keys[t] << 24 | t : ~0ull;
+    }
+    for (unsigned d = P >> 1; d > 0; d >>= 1) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) lo[q] += sk[lo[q] + d - 1] <= kk[q] ? d : 0u;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (sk[lo[q]] > kk[q]) atomicAdd(&place[lo[q]], 1u);  // none above the largest
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    unsigned run = 0;
+    for (unsigned b = 0; b < P; b += 32) {
+      unsigned v = place[b + threadIdx.x];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned u = __shfl_up_sync(0xffffffffu, v, o);
+        if ((int)threadIdx.x >= o) v += u;
+      }
+      place[b + threadIdx.x] = run + v;
+      run += __shfl_sync(0xffffffffu, v, 31);
+    }
+  }
+  __syncthreads();
+}
+
 // Counters of the resolved step: outcomes, the stores' new lengths, pids.
 __device__ void resolve_commit(DevCounters* cnt, const ResolveCommit& c) {
   const unsigned int ne = min(cnt->n_events, (unsigned int)c.ev_cap);
@@ -804,112 +868,130 @@ __global__ void k_resolve_apply(ApplyArgs<S> a) {
   const unsigned long long nn_out = a.cnt->n[a.n_out][a.n_species];
   const uint32_t pid0 = a.cnt->next_pid;
   const unsigned int ne = min(a.cnt->n_events, (unsigned int)a.commit.ev_cap);
-  // few events: each thread takes one and finds its place r among the successful
-  // ones (the keys are unique and put those first); more: in the sorted order
-  const bool few = ne <= kSmallEvents;
-  // event q on block q mod G (as for injection: each event's FP64 kinematics
-  // then run on their own SM's FP64 pipe instead of queueing on one)
-  for (long long q = blockIdx.x + (long long)gridDim.x * threadIdx.x; q < (few ? ne : ns);
-       q += (long long)gridDim.x * blockDim.x) {
-    long long r = q;
-    uint32_t e = (uint32_t)q;
-    if (few) {
-      if (a.ev[e].victim < 0) continue;  // suppressed
-      const unsigned long long key = a.sort_keys[e];
-      r = 0;
+  // An event's place r among the successful ones (the keys are unique and put those
+  // first). Few events: event q on block q mod G (as for injection: each event's
+  // FP64 kinematics then run on their own SM's FP64 pipe instead of queueing on
+  // one), its thread counts the keys below its own. More: runs of events on a
+  // block, placed at once. Beyond those: as the few, in the order of the radix passes.
+  __shared__ unsigned long long sk[kOrderRun];
+  __shared__ unsigned place[kOrderRun];
+  const bool few = ne <= kCountEvents, flat = few || ne > kPlacedEvents;
+  const unsigned G = gridDim.x, total = flat && !few ? ns : ne;
+  const unsigned over = min(G, kOrderBlocks), run = min(max((ne + over - 1) / over, 32u), kOrderRun);
+  for (long long c0 = flat ? 0 : (long long)blockIdx.x * run; c0 < total; c0 += flat ? total : (long long)G * run) {
+    const unsigned m = flat ? (total + G - 1 - min(blockIdx.x, total)) / G : min(run, ne - (unsigned)c0);
+    if (!flat) {
+      __syncthreads();  // the run before has been read
+      place_events(a.sort_keys, ne, (unsigned)c0, m, sk, place);
+    }
+    for (unsigned j = threadIdx.x; j < m; j += blockDim.x) {
+      const unsigned q = blockIdx.x + G * j;
+      long long r;
+      uint32_t e;
+      if (few) {
+        e = q;
+        if (a.ev[e].victim < 0) continue;  // suppressed
+        const unsigned long long key = a.sort_keys[e];
+        r = 0;
 #pragma unroll 8
-      for (unsigned int t = 0; t < ne; ++t) r += a.sort_keys[t] < key ? 1 : 0;
-    } else {
-      e = a.sorted_vals[q];
-    }
-    if (!PIC_BOUNDS(e < (uint32_t)a.ev_cap, a.cnt)) continue;
-    const Event ev = a.ev[e];
-    if (!PIC_BOUNDS(ev.victim >= 0 && ev.victim < a.cand_cap &&
-                        (long long)ev.slot < (ev.kind == XS_CHARGE_EXCHANGE ? a.i_cap : a.e_cap),
-                    a.cnt))
-      continue;
-    const Cand cd = a.cand[ev.victim];
-    if (!PIC_BOUNDS(cd.slot < (uint32_t)a.n_cap, a.cnt)) continue;
-    // victim neutral -> ion (position x^{n+1}, velocity and pid kept)
-    const auto vn = store_read(a.n_st, a.g, cd.slot);
-    const bool is_cx = r >= nion;
-    const uint32_t mp = a.commit.weighted ? (is_cx ? a.i_st.mw[ev.slot] : a.e_st.mw[ev.slot]) : 1u;
-    const uint32_t ms = min(mp, vn.mw);
-    auto vm = vn;  // the part that converts
-    if (ms == vn.mw) {
-      store_kill(a.n_st, cd.slot);
-      if (a.commit.weighted) atomicAdd(&a.cnt->n_kill_n, 1u);
-    } else {
-      a.n_st.mw[cd.slot] = vn.mw - ms;
-      vm.mw = ms;
-      vm.pid = pid0 + ns + 2u * (uint32_t)r;
-    }
-    const unsigned long long is = ni_out + r;
-    if (is < (unsigned long long)a.i_cap) {
-      store_write_p(a.i_st, is, vm);
-      if (a.nd.on) deposit_one(a.g, vm, a.nd.rho32, a.nd.rho64, a.nd.qw_h3[a.i_species]);
-    } else {
-      atomicOr(&a.cnt->error, ERR_CAPACITY);
-    }
-    if (a.nd.on) atomicSub(&a.nd.ncount[a.n_species][cell_now(a.g, vn)], (int)ms);
-    if (is_cx) {
-      // charge exchange: the primary ion continues as a neutral
-      auto pi = store_read(a.i_st, a.g, ev.slot);
-      if (ms == mp) {
-        store_kill(a.i_st, ev.slot);
-        if (a.commit.weighted) atomicAdd(&a.cnt->n_kill_i, 1u);
+        for (unsigned int t = 0; t < ne; ++t) r += a.sort_keys[t] < key ? 1 : 0;
+      } else if (flat) {
+        e = a.sorted_vals[q];
+        r = q;
       } else {
-        a.i_st.mw[ev.slot] = mp - ms;
-        pi.mw = ms;
-        pi.pid = pid0 + ns + 2u * (uint32_t)r + 1u;
+        e = (uint32_t)sk[j] & 0xFFFFFFu;
+        r = place[j];
+        if (r >= ns) continue;  // suppressed
       }
-      const unsigned long long os = nn_out + (r - nion);
-      if (os < (unsigned long long)a.n_cap) {
-        store_write_p(a.n_st, os, pi);
-        if (a.nd.on) {
-          deposit_one(a.g, pi, a.nd.rho32, a.nd.rho64, -a.nd.qw_h3[a.i_species]);
-          atomicAdd(&a.nd.ncount[a.n_species][cell_now(a.g, pi)], (int)ms);
-        }
+      if (!PIC_BOUNDS(e < (uint32_t)a.ev_cap, a.cnt)) continue;
+      const Event ev = a.ev[e];
+      if (!PIC_BOUNDS(ev.victim >= 0 && ev.victim < a.cand_cap &&
+                          (long long)ev.slot < (ev.kind == XS_CHARGE_EXCHANGE ? a.i_cap : a.e_cap),
+                      a.cnt))
+        continue;
+      const Cand cd = a.cand[ev.victim];
+      if (!PIC_BOUNDS(cd.slot < (uint32_t)a.n_cap, a.cnt)) continue;
+      // victim neutral -> ion (position x^{n+1}, velocity and pid kept)
+      const auto vn = store_read(a.n_st, a.g, cd.slot);
+      const bool is_cx = r >= nion;
+      const uint32_t mp = a.commit.weighted ? (is_cx ? a.i_st.mw[ev.slot] : a.e_st.mw[ev.slot]) : 1u;
+      const uint32_t ms = min(mp, vn.mw);
+      auto vm = vn;  // the part that converts
+      if (ms == vn.mw) {
+        store_kill(a.n_st, cd.slot);
+        if (a.commit.weighted) atomicAdd(&a.cnt->n_kill_n, 1u);
+      } else {
+        a.n_st.mw[cd.slot] = vn.mw - ms;
+        vm.mw = ms;
+        vm.pid = pid0 + ns + 2u * (uint32_t)r;
+      }
+      const unsigned long long is = ni_out + r;
+      if (is < (unsigned long long)a.i_cap) {
+        store_write_p(a.i_st, is, vm);
+        if (a.nd.on) deposit_one(a.g, vm, a.nd.rho32, a.nd.rho64, a.nd.qw_h3[a.i_species]);
       } else {
         atomicOr(&a.cnt->error, ERR_CAPACITY);
       }
-      continue;
-    }
-    const XsDev& X = a.ch[ev.ch];
-    const uint4 g0 = draw(a.key, ev.pid, a.cnt->step, TAG_IONIZE, 0);
-    const uint4 g1 = draw(a.key, ev.pid, a.cnt->step, TAG_IONIZE, 1);
-    const double Eex = ev.E_eV - X.thr;
-    const double Us = u01_64(g0.x, g0.y);
-    const double E2 = Us * Eex;
-    const double E1 = (1.0 - Us) * Eex;
-    const double sc = sqrt(E1 / ev.E_eV);
-    // primary: direction kept, energy (1-U) (E - thr)
-    auto pr = store_read(a.e_st, a.g, ev.slot);
-    if (ms == mp || u01_64(g1.z, g1.w) < (double)ms / (double)mp) {
-      pr.scale_v(sc);
-      store_write_v(a.e_st, ev.slot, pr);
-    }
-    // secondary at the primary's new position
-    const double us = sqrt(2.0 * E2 * kQe / a.e_mass);
-    const double ct = 2.0 * u01_64(g0.z, g0.w) - 1.0;
-    const double st = sqrt(fmax(0.0, 1.0 - ct * ct));
-    const double ph = 2.0 * kPi * u01_64(g1.x, g1.y);
-    const uint32_t spid = pid0 + (uint32_t)r;
-    auto sec = pr;
-    sec.set_v(us * st * cos(ph), us * st * sin(ph), us * ct);
-    sec.pid = spid;
-    sec.mw = ms;
-    const unsigned long long es = ne_out + r;
-    if (es < (unsigned long long)a.e_cap) {
-      store_write_p(a.e_st, es, sec);
-      if (a.nd.on) deposit_one(a.g, sec, a.nd.rho32, a.nd.rho64, a.nd.qw_h3[a.e_species]);
-    } else {
-      atomicOr(&a.cnt->error, ERR_CAPACITY);
-    }
-    if (a.log) {
-      a.log[3 * r] = ev.pid;
-      a.log[3 * r + 1] = vn.pid;
-      a.log[3 * r + 2] = spid;
+      if (a.nd.on) atomicSub(&a.nd.ncount[a.n_species][cell_now(a.g, vn)], (int)ms);
+      if (is_cx) {
+        // charge exchange: the primary ion continues as a neutral
+        auto pi = store_read(a.i_st, a.g, ev.slot);
+        if (ms == mp) {
+          store_kill(a.i_st, ev.slot);
+          if (a.commit.weighted) atomicAdd(&a.cnt->n_kill_i, 1u);
+        } else {
+          a.i_st.mw[ev.slot] = mp - ms;
+          pi.mw = ms;
+          pi.pid = pid0 + ns + 2u * (uint32_t)r + 1u;
+        }
+        const unsigned long long os = nn_out + (r - nion);
+        if (os < (unsigned long long)a.n_cap) {
+          store_write_p(a.n_st, os, pi);
+          if (a.nd.on) {
+            deposit_one(a.g, pi, a.nd.rho32, a.nd.rho64, -a.nd.qw_h3[a.i_species]);
+            atomicAdd(&a.nd.ncount[a.n_species][cell_now(a.g, pi)], (int)ms);
+          }
+        } else {
+          atomicOr(&a.cnt->error, ERR_CAPACITY);
+        }
+        continue;
+      }
+      const XsDev& X = a.ch[ev.ch];
+      const uint4 g0 = draw(a.key, ev.pid, a.cnt->step, TAG_IONIZE, 0);
+      const uint4 g1 = draw(a.key, ev.pid, a.cnt->step, TAG_IONIZE, 1);
+      const double Eex = ev.E_eV - X.thr;
+      const double Us = u01_64(g0.x, g0.y);
+      const double E2 = Us * Eex;
+      const double E1 = (1.0 - Us) * Eex;
+      const double sc = sqrt(E1 / ev.E_eV);
+      // primary: direction kept, energy (1-U) (E - thr)
+      auto pr = store_read(a.e_st, a.g, ev.slot);
+      if (ms == mp || u01_64(g1.z, g1.w) < (double)ms / (double)mp) {
+        pr.scale_v(sc);
+        store_write_v(a.e_st, ev.slot, pr);
+      }
+      // secondary at the primary's new position
+      const double us = sqrt(2.0 * E2 * kQe / a.e_mass);
+      const double ct = 2.0 * u01_64(g0.z, g0.w) - 1.0;
+      const double st = sqrt(fmax(0.0, 1.0 - ct * ct));
+      const double ph = 2.0 * kPi * u01_64(g1.x, g1.y);
+      const uint32_t spid = pid0 + (uint32_t)r;
+      auto sec = pr;
+      sec.set_v(us * st * cos(ph), us * st * sin(ph), us * ct);
+      sec.pid = spid;
+      sec.mw = ms;
+      const unsigned long long es = ne_out + r;
+      if (es < (unsigned long long)a.e_cap) {
+        store_write_p(a.e_st, es, sec);
+        if (a.nd.on) deposit_one(a.g, sec, a.nd.rho32, a.nd.rho64, a.nd.qw_h3[a.e_species]);
+      } else {
+        atomicOr(&a.cnt->error, ERR_CAPACITY);
+      }
+      if (a.log) {
+        a.log[3 * r] = ev.pid;
+        a.log[3 * r + 1] = vn.pid;
+        a.log[3 * r + 2] = spid;
+      }
     }
   }
   // the per-cell list heads of this step's events (and so of its candidates) go

@@ -129,13 +129,9 @@ __global__ void __launch_bounds__(kSortBlock) k_radix_scatter(const unsigned lon
   }
 }
 
-// Small inputs (n <= kSmallSort, the usual ionization event count): one block
-// ranks every pair against all others (ties by input position, so the order is
-// the stable one), writes it at its rank in the buffers the radix passes would
-// end in, and sets *done so that those passes return at once.
 // ---------------------------------------------------------------------------
-// Order of a step's events. Up to kSmallEvents the resolve's apply kernel ranks
-// each event against all others itself; larger lists take the radix passes. Which
+// Order of a step's events. Up to kPlacedEvents the resolve's apply kernel finds
+// each event's place itself; larger lists take the radix passes. Which
 // of the two is known on the device only: the rank kernel sets `order.small`, so
 // that the passes return at once, or, in a step being recorded, the condition of
 // the IF node they sit in, so that they are not launched at all.

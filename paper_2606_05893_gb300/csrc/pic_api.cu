@@ -713,7 +713,11 @@ pic_status create_instance(pic_handle* h, const pic_instance_cfg& c, Instance** 
     CK(h, cudaMemset(I->ev_head, 0xFF, sizeof(int32_t) * g.ncell));
     CK(h, cudaMemset(I->cand_head, 0xFF, sizeof(int32_t) * g.ncell));
     CK(h, dalloc(&I->ion_log, 3 * (size_t)I->ev_cap));
-    if (alloc_sort(I->evsort, I->ev_cap)) return fail(h, PIC_ENOMEM, "event sort buffers");
+    if (I->ev_cap > (int)kPlacedEvents) {
+      if (alloc_sort(I->evsort, I->ev_cap)) return fail(h, PIC_ENOMEM, "event sort buffers");
+    } else {
+      CK(h, dalloc(&I->evsort.ka, I->ev_cap));  // the keys alone
+    }
   }
   if (alloc_sort(I->csort, maxcap)) return fail(h, PIC_ENOMEM, "sort buffers");
   CK(h, dalloc(&I->cell_count, g.ncell));
@@ -1061,9 +1065,10 @@ pic_status step_instance(pic_handle* h, Instance* I) {
     r.sort_keys = I->evsort.ka;
     r.sort_vals = I->evsort.va;
     const int rb = std::min(blocks, (I->ev_cap + 255) / 256);
-    r.order = event_order_begin(I->evsort, st);
+    const bool radix = I->evsort.kb != nullptr;
+    if (radix) r.order = event_order_begin(I->evsort, st);
     launch_resolve_rank(r, rb, st);
-    const int where = event_order_end(I->evsort, r.order, &I->cnt->ev_sort_n, 40, st);
+    const int where = radix ? event_order_end(I->evsort, r.order, &I->cnt->ev_sort_n, 40, st) : 0;
     ApplyArgs<S> ap{};
     ap.g = g;
     ap.cnt = I->cnt;

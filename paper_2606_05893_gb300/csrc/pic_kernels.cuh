@@ -617,10 +617,20 @@ struct PushArgs {
   HitLog hits;
 };
 
+// How the apply kernel orders a step's events: up to kCountEvents by counting, up to
+// kPlacedEvents by runs, more by radix passes, which only an instance that can have
+// more of them keeps ready. Resolve of a step of 16x8x8 cells with 128 / 256 / 512 /
+// 2048 events: 25 / 28 / 37 / 86 us by counting, 25 / 25 / 27 / 37 us by runs; with
+// 2049 / 8192 / 32768 / 131072: 121 / 203 / 1200 / 35000 us by radix passes, 37 /
+// 100 / 1100 / 35000 us by runs (the search for victims takes over; the runs' work
+// grows with the square of the events, so the line is not drawn further out). A
+// recorded step without the passes' IF node is 8 us shorter.
+constexpr unsigned kCountEvents = 128, kPlacedEvents = 1u << 17;
+// events of a run at most; runs at least, as long as they hold 32 or more
+constexpr unsigned kOrderRun = 1024, kOrderBlocks = 152;
 // How the rank kernel tells the radix passes of the events whether they run.
-constexpr unsigned kSmallEvents = 2048;  // events that the apply kernel ranks itself
 struct EventOrder {
-  int* small;     // set to 1 for at most kSmallEvents events, else 0
+  int* small;     // set to 1 for at most kPlacedEvents events, else 0 (nullptr: no radix passes)
   int use_graph;  // a recorded step: the IF node's condition instead
   cudaGraphConditionalHandle handle;
 };
@@ -659,7 +669,7 @@ struct ApplyArgs {
   int ev_cap;
   const Cand* cand;
   int cand_cap;
-  const uint32_t* sorted_vals;           // events in apply order (more than kSmallEvents)
+  const uint32_t* sorted_vals;           // events in apply order (more than kPlacedEvents)
   const unsigned long long* sort_keys;  // of every event
   XsDev ch[kMaxXsec];
   uint2 key;
