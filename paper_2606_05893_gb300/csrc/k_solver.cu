@@ -1560,18 +1560,20 @@ __global__ void __launch_bounds__(256) k_update_ff(Lv L, float* __restrict__ hi,
 }
 
 // A float as a double by its bits: conversions run on the narrow FP64 pipe, where
-// the kernel below would queue two of them and two additions a node. Zeros,
-// denormals, infinities and NaN take the instruction.
+// the kernel below would queue two of them and two additions a node. Denormals,
+// infinities and NaN take the instruction, in a function of its own: inline it was
+// issued for every node, its lanes switched off.
+__device__ __noinline__ double widen_rare(float v) { return (double)v; }
 __device__ __forceinline__ double widen(float v) {
   const unsigned u = __float_as_uint(v), m = u & 0x7FFFFFFFu;
-  if (m - 0x00800000u >= 0x7F000000u) return (double)v;
-  return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+  if (m != 0u && m - 0x00800000u >= 0x7F000000u) return widen_rare(v);
+  return __hiloint2double((int)((u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), (int)(u << 29));
 }
 
 // phi (FP64, unknown view) = vac + hi + lo; a block takes 1024 points of one plane,
-// whole float4s where V = 4
-// (256x256x512, 33 million points: 270 us by rows of one point a thread or with the
-// conversion instruction, either alone no faster)
+// whole float4s where V = 4. Bound by the two FP64 additions a node (82 % of that
+// pipe; 16 B a node take 79 us): 256x256x512, 33 million points, 284 us with the
+// conversions, 162 us without. 32-byte stores were no faster.
 template <int V>
 __global__ void __launch_bounds__(256) k_phi_from_ff(Lv L, const float* __restrict__ hi, const float* __restrict__ lo,
                                                      double* __restrict__ x, double phi_c, double dphi_dk) {
