@@ -705,17 +705,17 @@ __device__ __forceinline__ bool grid_total2(V v0, V v1, double* part, unsigned* 
 }
 
 // The refinement's decision from r.r: another pass or stop; the power of two
-// that brings r to unit size for the FP32 pass of an FP64 residual.
+// that brings r to unit size for the FP32 pass of an FP64 residual, from the
+// exponents alone, and no relative residual (the host forms it): two square roots
+// and two divisions by one thread were on every solve's critical path (1.1 us a residual).
 __device__ __forceinline__ void fin_pass(const DirectLoop& d, SolveCtl* c, double rr, long long n) {
   c->rr_true = rr;
-  c->resid_rel = c->bb > 0.0 ? sqrt(rr / c->bb) : 0.0;
   const bool small = c->bb == 0.0 || rr <= c->tol2;
   const bool done = small || !(rr == rr) || c->it_total >= d.maxit || c->outer >= d.max_outer;
   c->converged = small ? 1 : 0;
   c->more = done ? 0 : 1;
   c->stopped = done ? 1 : 0;
-  const double rms = sqrt(rr / (double)n);
-  const int ex = rms > 0.0 && rms < 1e300 ? max(-900, min(900, -ilogb(rms))) : 0;
+  const int ex = rr > 0.0 && rr < INFINITY ? max(-900, min(900, (ilogb((double)n) - ilogb(rr)) >> 1)) : 0;
   c->scale = scalbn(1.0, ex);
   c->inv_scale = scalbn(1.0, -ex);
   if (d.use_graph) cudaGraphSetConditional(d.handle, done ? 0u : 1u);

@@ -2204,7 +2204,8 @@ cudaError_t Solver::result_async(cudaStream_t s) {
 SolveResult Solver::result_read() const {
   SolveResult r;
   r.iters = host_ctl->it_total;
-  r.resid_rel = host_ctl->resid_rel;
+  if (direct.on) r.resid_rel = host_ctl->bb > 0.0 ? std::sqrt(host_ctl->rr_true / host_ctl->bb) : 0.0;
+  else r.resid_rel = host_ctl->resid_rel;
   r.converged = host_ctl->converged != 0;
   r.timeout = host_ctl->spec_timeout != 0;
   return r;
