@@ -5,9 +5,10 @@
 // discrete Fourier modes of x and y decouple it into one tridiagonal system per
 // mode, (2 + lx + ly) u_k - u_(k-1) - u_(k+1) = f_k. Five launches:
 //   k_dir_xf  real FFT of every row (two rows packed as one complex line)
-//   k_dir_yf  complex FFT of every column of a plane
+//   k_dir_y   complex FFT of every column of a plane
 //   k_dir_z   tridiagonal solve of every mode, the planes split over warps
-//   k_dir_yi, k_dir_xi  the inverse transforms; the last adds d to the potential
+//   k_dir_y, k_dir_xi  the inverse transforms; the last adds d to the potential
+// (planes of about 32 x 32 points: three, k_dir_xyf and k_dir_xyi transform both axes)
 // The solve is one pass of iterative refinement: the caller forms r = b - A x in
 // float-float (mixed) or FP64, and repeats until the residual meets its tolerance.
 // FP32 rounding leaves 1e-6 to 1e-3 of the residual per pass (the most for modes
@@ -21,9 +22,11 @@
 // 128-byte row whatever the radix (rows of 17 float2 in x, where the loads
 // transpose). What is left is latency: a tile is loaded by asynchronous copies,
 // all in flight at once, and the last kernel loads what it adds to in batches
-// before it stores (256x256x512: k_dir_xi 281 -> 170 us, k_dir_z with its pivots
-// in shared memory, two blocks an SM instead of one, 108 -> 71). Spectra stay in the order the passes leave them in (digit
-// reversed): the tridiagonal kernel only needs each column's eigenvalue.
+// before it stores (256x256x512: k_dir_xi 281 -> 170 us, with wider blocks 148, with
+// the columns ordered by their place in the tile 123; k_dir_z with its pivots in
+// shared memory, two blocks an SM instead of one, 108 -> 71). Spectra stay in the
+// order the passes leave them in (digit reversed): the tridiagonal kernel only
+// needs each column's eigenvalue.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
