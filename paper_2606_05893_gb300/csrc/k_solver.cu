@@ -1559,21 +1559,35 @@ __global__ void __launch_bounds__(256) k_update_ff(Lv L, float* __restrict__ hi,
   }
 }
 
-// A float as a double by its bits: conversions run on the narrow FP64 pipe, where
-// the kernel below would queue two of them and two additions a node. Denormals,
-// infinities and NaN take the instruction, in a function of its own: inline it was
-// issued for every node, its lanes switched off.
-__device__ __noinline__ double widen_rare(float v) { return (double)v; }
-__device__ __forceinline__ double widen(float v) {
-  const unsigned u = __float_as_uint(v), m = u & 0x7FFFFFFFu;
-  if (m != 0u && m - 0x00800000u >= 0x7F000000u) return widen_rare(v);
-  return __hiloint2double((int)((u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), (int)(u << 29));
+// hi + lo as the FP64 addition rounds it, by integers: conversions and additions run
+// on the narrow FP64 pipe, where the kernel below would queue four of them a node.
+// lo lies below the last bit of a normalised hi, so in units of hi's last FP64 bit it
+// is an integer below 2^29, rounded to nearest even where its own bits reach further
+// down, and the sum stays in hi's binade. What does not fit (a lo that is not small
+// against hi, zero or denormal hi, denormal lo, infinities, NaN, a power of two
+// lessened) takes the instructions, in a function of its own: inline they were issued
+// for every node with their lanes switched off.
+__device__ __noinline__ double sum_rare(float hi, float lo) { return (double)hi + (double)lo; }
+__device__ __forceinline__ double sum64(float hi, float lo) {
+  const unsigned h = __float_as_uint(hi), l = __float_as_uint(lo);
+  const unsigned mh = h & 0x7FFFFFFFu, ml = l & 0x7FFFFFFFu, less = (h ^ l) >> 31;
+  const int eh = mh >> 23, el = ml >> 23, gap = eh - el;
+  if ((unsigned)(eh - 1) >= 254u || (ml != 0u && (el == 0 || gap < 24 || (less && (mh & 0x7FFFFFu) == 0u))))
+    return sum_rare(hi, lo);
+  const unsigned m = ml ? ((ml & 0x7FFFFFu) | 0x800000u) << 5 : 0u;
+  const int n = max(0, min(gap - 24, 31));
+  unsigned t = m >> n;
+  const unsigned rem = m - (t << n), half = (1u << n) >> 1;
+  t += rem > half || (rem == half && (t & 1u)) ? 1u : 0u;
+  const long long H = (long long)((unsigned long long)((h & 0x80000000u) | ((mh >> 3) + 0x38000000u)) << 32 | (h << 29));
+  return __longlong_as_double(less ? H - (long long)t : H + (long long)t);
 }
 
-// phi (FP64, unknown view) = vac + hi + lo; a block takes 1024 points of one plane,
-// whole float4s where V = 4. Bound by the two FP64 additions a node (82 % of that
-// pipe; 16 B a node take 79 us): 256x256x512, 33 million points, 284 us with the
-// conversions, 162 us without. 32-byte stores were no faster.
+// phi (FP64, unknown view) = vac + (hi + lo); a block takes 1024 points of one plane,
+// whole float4s where V = 4. 16 B a node take 79 us at 256x256x512 (33 million
+// points): 284 us with two conversions and two additions a node on the FP64 pipe
+// (82 % of it), 162 us without the conversions, 100 us with one addition. 32-byte
+// stores were no faster.
 template <int V>
 __global__ void __launch_bounds__(256) k_phi_from_ff(Lv L, const float* __restrict__ hi, const float* __restrict__ lo,
                                                      double* __restrict__ x, double phi_c, double dphi_dk) {
@@ -1585,12 +1599,12 @@ __global__ void __launch_bounds__(256) k_phi_from_ff(Lv L, const float* __restri
     if (r0 >= L.pl) return;
     const float4 h = *reinterpret_cast<const float4*>(hi + base + r0), l = *reinterpret_cast<const float4*>(lo + base + r0);
     double2* o = reinterpret_cast<double2*>(x + base + r0);
-    o[0] = make_double2(vac + (widen(h.x) + widen(l.x)), vac + (widen(h.y) + widen(l.y)));
-    o[1] = make_double2(vac + (widen(h.z) + widen(l.z)), vac + (widen(h.w) + widen(l.w)));
+    o[0] = make_double2(vac + sum64(h.x, l.x), vac + sum64(h.y, l.y));
+    o[1] = make_double2(vac + sum64(h.z, l.z), vac + sum64(h.w, l.w));
   } else {
     for (int q = 0; q < 4; ++q) {
       const int r = blockIdx.x * 1024 + q * 256 + threadIdx.x;
-      if (r < L.pl) x[base + r] = vac + (widen(hi[base + r]) + widen(lo[base + r]));
+      if (r < L.pl) x[base + r] = vac + sum64(hi[base + r], lo[base + r]);
     }
   }
 }

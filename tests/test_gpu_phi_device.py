@@ -43,3 +43,34 @@ def test_phi_into_device_array(pkg, nx, ny, nz, shift, mixed):
         want = sim.phi()
     assert got[0] == got[1] == np.ascontiguousarray(want).tobytes()
     sim.close()
+
+
+@pytest.mark.parametrize("nx,ny,nz", [(8, 4, 6), (5, 3, 7), (16, 12, 33)])
+@pytest.mark.parametrize("start", ["zero", "random", "charged"])
+def test_rebuild_rounds_as_fp64_additions(pkg, tmp_path, nx, ny, nz, start):
+    """phi = vac + (hi + lo) bit for bit, hi and lo as a checkpoint holds them behind the rebuilt phi."""
+    wl = bare(nx=nx, ny=ny, nz=nz, h=5e-9, phi_c=0.0, phi_a=float(nz), weight=1.0)  # vac(k) = k exactly
+    rng = np.random.default_rng(nx + ny + nz)
+    if start == "charged":
+        x = rng.random((300, 3)) * np.array([nx, ny, nz]) * wl.h
+        wl.preload = [(x, np.zeros_like(x)), (np.zeros((0, 3)),) * 2, (np.zeros((0, 3)),) * 2]
+    sim = pkg.Simulation(wl, precision=pkg.PIC_MIXED)
+    if start == "random":
+        phi = rng.standard_normal((nz + 1, ny, nx)) * 5.0
+        phi[0], phi[nz] = wl.phi_cathode, wl.phi_anode
+        sim.set_phi(phi)
+    sim.step()
+    path = str(tmp_path / "a.bin")
+    sim.save(path)
+    raw = open(path, "rb").read()
+    nnode, nu = (nz + 1) * ny * nx, (nz - 1) * ny * nx
+    lo_at = len(raw) - 4 * nu
+    hi_at = lo_at - 4 * nnode
+    got = np.frombuffer(raw[hi_at - 8 * nnode:hi_at], np.float64).reshape(nz + 1, ny, nx)
+    hi = np.frombuffer(raw[hi_at:lo_at], np.float32).reshape(nz + 1, ny, nx)
+    lo = np.frombuffer(raw[lo_at:], np.float32).reshape(nz - 1, ny, nx)
+    if start == "charged":
+        assert np.count_nonzero(lo) > nu // 2
+    want = np.arange(1, nz)[:, None, None] + (hi[1:nz].astype(np.float64) + lo.astype(np.float64))
+    assert np.array_equal(got[1:nz].view(np.int64), want.view(np.int64))
+    sim.close()
