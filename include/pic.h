@@ -439,6 +439,11 @@ uint64_t pic_launch_count(void);
  * counted once, so this is a lower bound when a solve iterates. */
 uint64_t pic_kernel_count(void);
 
+/* Steps recorded as graphs in this process so far (one instance's step or a whole
+ * ensemble's). Recording costs as much as many steps: a run that keeps its
+ * parameters records its patterns once and then only replays them. */
+uint64_t pic_record_count(void);
+
 /* ---- solve without allocating ----------------------------------------------
  * Not in the paper: an entry point for callers that cannot allocate device
  * memory while they run (programs that hand out all device memory from their

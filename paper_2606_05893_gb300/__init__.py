@@ -86,7 +86,7 @@ EXPORTED = ["pic_create", "pic_inject", "pic_inject_particles", "pic_inject_part
             "pic_last_error", "pic_get_count", "pic_get_particles", "pic_get_field", "pic_set_phi", "pic_solve",
             "pic_sort_now", "pic_get_cell_start", "pic_get_ionization_log", "pic_philox",
             "pic_set_mcc_background", "pic_version", "pic_set_profiling", "pic_get_phase_times",
-            "pic_launch_count", "pic_kernel_count", "pic_poisson_solve_static", "pic_set_sort_interval",
+            "pic_launch_count", "pic_kernel_count", "pic_record_count", "pic_poisson_solve_static", "pic_set_sort_interval",
             "pic_set_hit_log", "pic_get_hits", "pic_set_circuit", "pic_save", "pic_load",
             "pic_set_warm_unet", "pic_get_phi_device", "pic_set_launch_shape", "pic_set_allocator",
             "unet_num_weights", "unet_create", "unet_destroy", "unet_set_weights", "unet_get_weights",
@@ -156,6 +156,7 @@ def load_library(path: str = None):
         "pic_get_phase_times": ([P, C.c_int32, d, i64], st),
         "pic_launch_count": ([], C.c_uint64),
         "pic_kernel_count": ([], C.c_uint64),
+        "pic_record_count": ([], C.c_uint64),
         "pic_poisson_solve_static": ([C.c_int32, C.c_int32, C.c_int32, C.c_double, C.c_double, C.c_double, P, P,
                                       C.c_double, C.c_int32, P, C.POINTER(C.c_int32), d], st),
         "pic_set_warm_unet": ([P, C.c_int32, P], st),
@@ -442,6 +443,10 @@ def pic_launch_count():
 
 def pic_kernel_count():
     return int(load_library().pic_kernel_count())
+
+
+def pic_record_count():
+    return int(load_library().pic_record_count())
 
 
 PIC_STATIC_MAX_UNKNOWNS = 1 << 18

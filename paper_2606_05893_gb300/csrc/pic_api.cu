@@ -78,6 +78,7 @@ static bool set_device_allocator(pic_alloc_fn alloc, pic_free_fn free_fn, void* 
 }
 unsigned long long g_launches = 0;
 unsigned long long g_kernels = 0;
+unsigned long long g_records = 0;  // step graphs recorded (all handles)
 void set_static_error(const char* msg);
 int sm_count() {
   static int n = 0;
@@ -301,6 +302,8 @@ struct EnsembleGraph {
   std::vector<uint32_t> key;
   cudaGraphExec_t exec = nullptr;
   unsigned long long kernels = 0;
+  unsigned long long used = 0;  // pic_handle::ens_tick of its last use
+  bool sorts = false;           // an instance sorts in this step
 };
 
 struct pic_handle {
@@ -310,7 +313,9 @@ struct pic_handle {
   std::string err;
   bool dead = false;
   int sticky = 0;  // sticky non-fatal status bits (ENOCONV)
-  std::vector<EnsembleGraph> ens;  // recorded ensemble steps (a few parity patterns)
+  std::vector<EnsembleGraph> ens;  // recorded ensemble steps, by pattern of parities and sorts
+  unsigned long long ens_tick = 0;  // ensemble steps looked up so far
+  std::vector<uint64_t> ens_seen;   // hashes of patterns met once: some instances sort, others do not
   bool ens_ok = true;              // false once recording an ensemble step failed
   cudaStream_t ens_cap = nullptr;  // origin stream of the ensemble recording
   cudaEvent_t ens_fork = nullptr;  // the recording's fork into the instance streams
@@ -1302,6 +1307,7 @@ pic_status run_step(pic_handle* h, Instance* I) {
   }
   I->step_exec[key] = exec;
   I->step_kernels[key] = kernels;
+  ++g_records;
   count_graph(kernels);
   CK(h, cudaGraphLaunch(exec, I->stream));
   return PIC_OK;
@@ -1311,11 +1317,24 @@ pic_status run_step(pic_handle* h, Instance* I) {
 // the handle's stream: each instance's step is a branch between a common fork
 // and join, so the instances run concurrently as they do on their own streams,
 // with one launch per ensemble step instead of one per instance. Used when
-// every instance's step qualifies for recording (no sort, no phase timing, no
-// deposit from scratch); the graph is recorded the first time a pattern of
-// parities appears (a handful of patterns: each step flips every parity).
-// Returns false, with nothing enqueued and every host state unchanged, when the
-// step cannot be recorded; the caller then steps the instances one by one.
+// every instance's step qualifies for recording (no phase timing, no deposit from
+// scratch). A pattern is the parities of every instance and whether it sorts:
+// with one sort interval 6 recur, with two that divide each other 12, with 5, 10,
+// 20 and 40 together 48, with others up to some hundred, and recording one costs
+// as much as many steps. So
+//  - a pattern in which some instances sort and others do not is recorded when it
+//    comes a second time;
+//  - a full list gives up a graph only if it has not run for kEnsStale steps, or
+//    for a pattern without a sort (they recur most) one with a sort.
+// The list thus settles, and what it does not hold runs from the instances' own
+// recorded steps, of which each needs eight. Eight small boxes (config_small,
+// mixed), us per ensemble step against a list of 8, oldest out first, which went on
+// recording: one interval of 20 198 and 199, intervals 20/40 214 and 275, 5/10 263
+// and 828, 5/10/20/40 359 and 669.
+constexpr unsigned long long kEnsStale = 4096;
+// graphs a handle holds: 64 for a few instances, 8 from 64 on (a graph grows with them)
+size_t ens_capacity(const pic_handle* h) { return std::max<size_t>(8, std::min<size_t>(64, 512 / h->inst.size())); }
+
 bool ensemble_recordable(const pic_handle* h) {
   if (h->inst.size() < 2 || !h->ens_ok) return false;
   for (const auto* I : h->inst)
@@ -1323,12 +1342,69 @@ bool ensemble_recordable(const pic_handle* h) {
   return true;
 }
 
-bool run_ensemble_step(pic_handle* h) {
+// What to do with the next ensemble step: run the recorded graph `at` (>= 0),
+// record it, or step the instances one by one.
+struct EnsemblePlan {
+  enum { kReplay, kRecord, kSingly } what = kSingly;
+  size_t at = 0;
+  bool sorts = false;
   std::vector<uint32_t> key;
-  key.reserve(h->inst.size());
-  for (const auto* I : h->inst) key.push_back(graph_key(I) | (I->graph_epoch << 3));
-  for (auto& g : h->ens) {
-    if (g.key != key) continue;
+};
+EnsemblePlan plan_ensemble_step(pic_handle* h) {
+  EnsemblePlan p;
+  if (!ensemble_recordable(h)) return p;
+  ++h->ens_tick;
+  p.key.reserve(h->inst.size());
+  size_t nsort = 0;
+  uint64_t hash = 0xCBF29CE484222325ull;  // FNV-1a
+  for (const auto* I : h->inst) {
+    p.key.push_back(graph_key(I) | (I->graph_epoch << 3));
+    nsort += sort_due(I) ? 1 : 0;
+    hash = (hash ^ p.key.back()) * 0x100000001B3ull;
+  }
+  p.sorts = nsort != 0;
+  for (p.at = 0; p.at < h->ens.size(); ++p.at) {
+    if (h->ens[p.at].key != p.key) continue;
+    h->ens[p.at].used = h->ens_tick;
+    p.what = EnsemblePlan::kReplay;
+    return p;
+  }
+  if (nsort != 0 && nsort != h->inst.size() &&
+      std::find(h->ens_seen.begin(), h->ens_seen.end(), hash) == h->ens_seen.end()) {
+    if (h->ens_seen.size() >= 256) h->ens_seen.erase(h->ens_seen.begin());
+    h->ens_seen.push_back(hash);
+    return p;
+  }
+  auto drop = [&](size_t q) {
+    cudaGraphExecDestroy(h->ens[q].exec);
+    h->ens.erase(h->ens.begin() + q);
+  };
+  // graphs with steps that were dropped since match nothing any more
+  for (size_t q = h->ens.size(); q-- > 0;)
+    for (size_t i = 0; i < h->inst.size(); ++i)
+      if ((h->ens[q].key[i] ^ p.key[i]) >> 3) {
+        drop(q);
+        break;
+      }
+  if (h->ens.size() >= ens_capacity(h)) {
+    size_t out = h->ens.size();
+    for (size_t q = 0; q < h->ens.size(); ++q) {
+      const EnsembleGraph& g = h->ens[q];
+      if (h->ens_tick - g.used < kEnsStale && !(g.sorts && !p.sorts)) continue;
+      if (out == h->ens.size() || g.used < h->ens[out].used) out = q;
+    }
+    if (out == h->ens.size()) return p;
+    drop(out);
+  }
+  p.what = EnsemblePlan::kRecord;
+  return p;
+}
+
+// Returns false, with nothing enqueued and every host state unchanged, when the
+// step cannot be recorded or launched; the caller then steps the instances one by one.
+bool run_ensemble_step(pic_handle* h, const EnsemblePlan& plan) {
+  if (plan.what == EnsemblePlan::kReplay) {
+    const EnsembleGraph& g = h->ens[plan.at];
     count_graph(g.kernels);
     if (cudaGraphLaunch(g.exec, h->stream) != cudaSuccess) {
       cudaGetLastError();
@@ -1393,14 +1469,13 @@ bool run_ensemble_step(pic_handle* h) {
     h->ens_ok = false;
     return false;
   }
-  if (h->ens.size() >= 8) {  // a few patterns recur; drop the oldest beyond that
-    cudaGraphExecDestroy(h->ens.front().exec);
-    h->ens.erase(h->ens.begin());
-  }
   EnsembleGraph eg;
-  eg.key = key;
+  eg.key = plan.key;
   eg.exec = exec;
   eg.kernels = kernels;
+  eg.used = h->ens_tick;
+  eg.sorts = plan.sorts;
+  ++g_records;
   h->ens.push_back(eg);
   count_graph(kernels);
   if (cudaGraphLaunch(exec, h->stream) != cudaSuccess) {
@@ -1708,11 +1783,14 @@ pic_status pic_step(pic_handle* h, int32_t nsteps) {
   };
   pic_status step_status = PIC_OK;
   for (int n = 0; n < nsteps && step_status == PIC_OK; ++n) {
-    if (multi && ensemble_recordable(h)) {
-      if (pending && (step_status = join_instances()) != PIC_OK) break;
-      if (run_ensemble_step(h)) {
-        forked = false;
-        continue;
+    if (multi) {
+      const EnsemblePlan plan = plan_ensemble_step(h);
+      if (plan.what != EnsemblePlan::kSingly) {
+        if (pending && (step_status = join_instances()) != PIC_OK) break;
+        if (run_ensemble_step(h, plan)) {
+          forked = false;
+          continue;
+        }
       }
     }
     if (multi && !forked && (step_status = fork_instances()) != PIC_OK) break;
@@ -2132,6 +2210,8 @@ pic_status pic_get_phase_times(pic_handle* h, int32_t inst, double* ms, int64_t*
 
 uint64_t pic_launch_count(void) { return (uint64_t)pic::g_launches; }
 uint64_t pic_kernel_count(void) { return (uint64_t)pic::g_kernels; }
+
+uint64_t pic_record_count(void) { return g_records; }
 
 pic_status pic_set_sort_interval(pic_handle* h, int32_t inst, int32_t interval) {
   pic_status st = check(h, inst);
