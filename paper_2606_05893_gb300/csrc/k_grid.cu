@@ -4,6 +4,7 @@
 
 #include "pic_internal.cuh"
 #include "pic_kernels.cuh"
+#include "solver_dev.cuh"
 
 namespace pic {
 
@@ -681,87 +682,17 @@ void launch_field_energy(const Grid& g, const double* phi, double* out, cudaStre
 // FP32 remainder). The vacuum part cancels in x and y and is one constant per
 // z edge (dz_in inside, dz_top for the last edge). A difference of two exact
 // FP32 values is rounded relative to the difference itself, so every edge
-// difference comes out within ~1e-7 of its size; the squares are summed in
-// FP32 over runs of 8 nodes and those sums in FP64.
-__global__ void k_field_energy_ff(Grid g, const float* __restrict__ hi, const float* __restrict__ lo, float dz_in,
-                                  float dz_top, double* out) {
-  // threads (x over a row, y over kFeRows rows): a block keeps that many rows'
-  // loads in flight at once
-  const long long pl = g.nplane;
-  const long long rows = (long long)g.ny * (g.nz + 1);
-  double acc = 0.0;
-  float part = 0.f;
-  int run = 0;
-  for (long long r = (long long)blockIdx.x * blockDim.y + threadIdx.y; r < rows; r += (long long)gridDim.x * blockDim.y) {
-    const int k = (int)(r / g.ny);
-    const int j = (int)(r - (long long)k * g.ny);
-    const long long c0 = (long long)j * g.nx;                               // row j in a plane
-    const long long cn = (long long)(j + 1 == g.ny ? 0 : j + 1) * g.nx;     // row j + 1
-    const float* H = hi + (long long)k * pl;                                 // plane k (node view)
-    const float* L = lo + (long long)(k - 1) * pl;                           // plane k (unknown view)
-    const bool interior = k > 0 && k < g.nz;
-    for (int i = threadIdx.x; i < g.nx; i += blockDim.x) {
-      const int ip = i + 1 == g.nx ? 0 : i + 1;
-      float h0 = 0.f, hx = 0.f, hy = 0.f, l0 = 0.f, lx = 0.f, ly = 0.f;
-      if (k > 0) {
-        h0 = H[c0 + i];
-        hx = H[c0 + ip];
-        hy = H[cn + i];
-      }
-      if (interior) {
-        l0 = L[c0 + i];
-        lx = L[c0 + ip];
-        ly = L[cn + i];
-      }
-      const float dx = (hx - h0) + (lx - l0);
-      const float dy = (hy - h0) + (ly - l0);
-      float sq = fmaf(dx, dx, dy * dy);
-      if (k < g.nz) {
-        const float h1 = H[pl + c0 + i];
-        const float l1 = k + 1 < g.nz ? L[pl + c0 + i] : 0.f;
-        const float dz = (k + 1 == g.nz ? dz_top : dz_in) + ((h1 - h0) + (l1 - l0));
-        sq = fmaf(dz, dz, sq);
-      }
-      part += sq;
-      if (++run == 8) {
-        acc += (double)part;
-        part = 0.f;
-        run = 0;
-      }
-    }
-  }
-  acc += (double)part;
-  // block sum over the linear thread index (two-dimensional block)
-  __shared__ double sm[32];
-  const int t = threadIdx.y * blockDim.x + threadIdx.x, nw = (blockDim.x * blockDim.y) >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if ((t & 31) == 0) sm[t >> 5] = acc;
-  __syncthreads();
-  if (t < 32) {
-    acc = t < nw ? sm[t] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if (t == 0) atomicAdd(out, acc);
-  }
-}
-void launch_field_energy_ff(const Grid& g, const float* phi32, const float* lo32, double* out, cudaStream_t s) {
-  const double dphi_dk = (g.phi_a - g.phi_c) / (double)g.nz;
-  const float dz_in = (float)dphi_dk;
-  const float dz_top = (float)(g.phi_a - (g.phi_c + dphi_dk * (double)(g.nz - 1)));
-  const long long rows = (long long)g.ny * (g.nz + 1);
-  const int tx = g.nx >= 128 ? 128 : (g.nx >= 64 ? 64 : 32);
-  const int ty = 256 / tx;
-  const int grid = (int)std::min<long long>((rows + ty - 1) / ty, 152 * 8);
-  PIC_LAUNCH(grid, dim3(tx, ty), 0, s, k_field_energy_ff)(g, phi32, lo32, dz_in, dz_top, out);
-}
-
+// difference comes out within ~1e-7 of its size.
 // This thread's share of the squared edge differences: columns of V neighbouring
 // points of a row through kFePlanes planes. A plane is loaded once, as the upper
 // neighbour, and kept as the next centre, so a point costs its own plane's load and
 // its y neighbour's (a point at a time with two index divisions and ten loads: 210 us
-// at 256x256x512 with 8.5 million particles, now 118).
-// Summed in FP32 over a column, in FP64 over columns.
+// at 256x256x512 with 8.5 million particles, 118 so).
+// The squares of two neighbouring nodes are summed in FP32, pairs in float-float
+// over a column, columns in FP64: a column of 16 nodes in FP32 alone lost up to 3 bits
+// more, and an FP64 addition for every pair would queue on the narrow FP64 pipe
+// (pic_moments at 256x256x512 without particles 100 us with columns in FP32 alone, 103
+// us so, 112 us with every node in float-float).
 constexpr int kFePlanes = 4;
 template <int V>
 __device__ __forceinline__ double field_energy_share(const MomentsMx& a) {
@@ -799,13 +730,14 @@ __device__ __forceinline__ double field_energy_share(const MomentsMx& a) {
       hx[p] = k > 0 && k <= g.nz ? a.hi[k * pl + xat] : 0.f;
       lx[p] = k > 0 && k < g.nz ? a.lo[(k - 1) * pl + xat] : 0.f;
     }
-    float part = 0.f;
+    float part = 0.f, rest = 0.f;
 #pragma unroll
     for (int p = 0; p < kFePlanes; ++p) {
       const int k = k0 + p;
       load(k + 1, at, h1, l1);
       if (k <= g.nz) {
         const float vac = k + 1 == g.nz ? a.dz_top : a.dz_in;
+        float pair = 0.f;
 #pragma unroll
         for (int e = 0; e < V; ++e) {
           const float xh = e + 1 < V ? h0[e + 1 < V ? e + 1 : 0] : hx[p], xl = e + 1 < V ? l0[e + 1 < V ? e + 1 : 0] : lx[p];
@@ -816,7 +748,12 @@ __device__ __forceinline__ double field_energy_share(const MomentsMx& a) {
             const float dz = vac + ((h1[e] - h0[e]) + (l1[e] - l0[e]));
             sq = fmaf(dz, dz, sq);
           }
-          part += sq;
+          pair = (e & 1) != 0 ? pair + sq : sq;
+          if ((e & 1) != 0 || V == 1) {
+            float err;
+            two_sum(part, pair, part, err);
+            rest += err;
+          }
         }
       }
 #pragma unroll
@@ -825,14 +762,14 @@ __device__ __forceinline__ double field_energy_share(const MomentsMx& a) {
         l0[e] = l1[e];
       }
     }
-    acc += (double)part;
+    acc += (double)part + (double)(rest == rest ? rest : 0.f);  // (no error term of a sum that overflowed)
   }
   return acc;
 }
 
 // The moments of the mixed store in one launch: every block sums |v|^2 of its
 // share of every species (four particles per pass in FP32, the passes in FP64),
-// then its share of the field energy (edge differences as k_field_energy_ff), and
+// then its share of the field energy (edge differences of the hi / lo state), and
 // writes its totals to a.part; the last block to finish adds the blocks'
 // totals in block order (a sum that does not depend on timing) into out
 // (out[sp] per species, out[16] the field).

@@ -808,7 +808,6 @@ void launch_sort_commit(DevCounters* cnt, int c, int s, cudaStream_t st);
 template <class S>
 void launch_kinetic(S st, const unsigned long long* n_dev, long long n_max, double* out, cudaStream_t s);
 void launch_field_energy(const Grid& g, const double* phi, double* out, cudaStream_t s);
-void launch_field_energy_ff(const Grid& g, const float* phi32, const float* lo32, double* out, cudaStream_t s);
 // every species' sum of |v|^2 (out[sp]) and the field energy sum (out[16]) of the
 // mixed store in one launch (written, not added to); part holds kMomBlocks x
 // kMomSlots doubles, ticket one counter that is 0 between launches

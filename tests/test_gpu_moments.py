@@ -146,3 +146,30 @@ def test_mixed_field_energy_over_row_shapes(pkg, nx, ny, nz):
     fg, fh = sim.moments()["field_energy"], host_field_energy(stored, wl)
     assert abs(fg - fh) <= mixed_fe_rounding_bound(stored, wl)
     sim.close()
+
+
+@pytest.mark.parametrize("nx,ny,nz", [(36, 20, 50), (8, 5, 3), (6, 9, 13), (1, 1, 2), (128, 4, 33)])
+def test_mixed_field_energy_sums_its_nodes_exactly(pkg, nx, ny, nz):
+    """Whole potentials of at most 700 in size: the six squares of two nodes add up exactly in FP32 (below
+    2^24), all of them in FP64 (below 2^53), so only the final scaling rounds (three products)."""
+    from tests._cases import bare
+    wl = bare(nx=nx, ny=ny, nz=nz, h=5e-9)
+    sim = pkg.Simulation(wl, precision=pkg.PIC_MIXED)
+    phi = np.random.default_rng(nx + ny + nz).integers(-700, 701, (nz + 1, ny, nx)).astype(np.float64)
+    phi[0] = phi[nz] = 0.0
+    sim.set_phi(phi)
+    exact = host_field_energy(phi, wl)  # whole numbers below 2^53 until they are scaled
+    assert abs(sim.moments()["field_energy"] - exact) <= 6 * 2.0 ** -53 * exact
+    sim.close()
+
+
+def test_mixed_field_energy_beyond_single_range(pkg):
+    # squares that overflow FP32 make the energy infinite, not undefined
+    from tests._cases import bare
+    wl = bare(nx=8, ny=6, nz=9, h=5e-9)
+    sim = pkg.Simulation(wl, precision=pkg.PIC_MIXED)
+    phi = np.zeros((10, 6, 8))
+    phi[4, 2, 3] = 1e25
+    sim.set_phi(phi)
+    assert sim.moments()["field_energy"] == np.inf
+    sim.close()
