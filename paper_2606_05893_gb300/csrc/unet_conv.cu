@@ -31,6 +31,7 @@
 #include <cstdio>
 
 #include "tc_ptx.cuh"
+#include "tmem_share.h"
 #include "unet_internal.cuh"
 
 namespace unet {
@@ -563,18 +564,6 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_wgrad(const __grid_constant
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-constexpr int kSmemMax = 227 * 1024;
-constexpr int kSmemPerSM = 228 * 1024;
-
-// Dynamic shared memory of a CTA that holds tmem_cols TMEM columns: at least
-// enough that no more CTAs share an SM than its 512 columns hold, so a
-// tcgen05.alloc never waits for another CTA's columns.
-static size_t smem_floor(size_t need, uint32_t tmem_cols) {
-  const size_t fit = 512 / (tmem_cols ? tmem_cols : 512);
-  const size_t floor_b = kSmemPerSM / (fit + 1) + 1024;
-  return need > floor_b ? need : floor_b;
-}
-
 void launch_conv3(const ConvArgs& a, cudaStream_t s) {
   static bool attr = false;
   if (!attr) {
@@ -618,9 +607,10 @@ void launch_wgrad(const WgradArgs& a, cudaStream_t s) {
   const int gy = a.taps == 9 ? 3 : 9;
   const int gz = (a.gin + 15) / 16;
   const size_t smem = smem_floor((size_t)a.smem_main + 256, a.tmem_cols);
-  // one wave: as many CTAs as are resident at once (rounding up left two CTAs for
-  // a wave of their own)
-  const long long per_sm = std::max<long long>(1, std::min<long long>(512 / a.tmem_cols, kSmemPerSM / (smem + 1024)));
+  // one wave: as many CTAs as are resident at once with the SMs to themselves
+  // (rounding up left two CTAs for a wave of their own)
+  const long long per_sm =
+      std::max<long long>(1, std::min<long long>(kTmemColumns / a.tmem_cols, kSmemPerSM / (smem + kSmemReserved)));
   const long long gx = std::max(1ll, std::min(per_sm * sms / (gy * gz), a.nchunks));
   ++g_launches;
   k_wgrad<<<dim3((unsigned)gx, gy, gz), kConvThreads, smem, s>>>(a);
