@@ -53,3 +53,29 @@ def test_order_of_effect(pkg, n_e, capacity):
     assert np.array_equal(sim.ionization_log(), ref.ionization_log())
     sim.close()
     ref.close()
+
+
+def test_recorded_radix_passes(pkg):
+    """The radix passes as a recorded step holds them, in a node that the step opens by itself: the first
+    step (enqueued directly, 131072 events placed by runs) leaves more than 131072 electrons above the
+    threshold, and neutrals enough for them, so the recorded ones after it, one of each parity, take the passes."""
+    wl = crowded(1 << 17, 1 << 23, seed=77)
+    more = [crowded(1 << 17, 1 << 23, seed=78 + q).preload[1] for q in range(4)]
+    wl.preload[1] = tuple(np.concatenate(a) for a in zip(wl.preload[1], *more))
+    sim = pkg.Simulation(wl, precision=pkg.PIC_FP64, cg_rtol=1e-13, cg_maxit=5000)
+    ref = O.Oracle(wl, cg_rtol=1e-13)
+    events = 1 << 17
+    sim.step()
+    ref.step()
+    for _ in range(2):
+        launches = pkg.pic_launch_count()
+        sim.step()
+        assert pkg.pic_launch_count() - launches == 1
+        ref.step()
+        mg, _ = full_compare(sim, ref, wl)
+        total = mg["n_ionization"] + mg["n_suppressed"]
+        assert total - events > 1 << 17
+        events = total
+        assert np.array_equal(sim.ionization_log(), ref.ionization_log())
+    sim.close()
+    ref.close()
