@@ -274,7 +274,7 @@ void launch_planes_from_ff(const Grid& g, const float* phi32, double* phi, cudaS
 // ---------------------------------------------------------------------------
 // The kernel also readies the step's accumulators: the next step's density (set
 // to the background) and neutral counts (zero), which the particle kernels that
-// follow add to, and the counters of a step (k_step_begin's work). E.w carries the
+// follow add to, and the counters of a step (step_begin). E.w carries the
 // neutral count of the cell whose lower corner is this node (cell and node
 // indices coincide for k < nz), read by the collision filter.
 // Bound by its stores (16 or 32 B of E a node): a thread takes KC planes of its

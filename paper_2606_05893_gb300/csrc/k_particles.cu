@@ -718,8 +718,8 @@ __global__ void __launch_bounds__(kRankWarps * 32) k_resolve_rank(ResolveArgs a)
   const unsigned int nc = min(a.cnt->n_cands, (unsigned int)a.cand_cap);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     a.cnt->ev_sort_n = ne;
-    if (a.order.small) *a.order.small = ne <= kPlacedEvents ? 1 : 0;
-    if (a.order.use_graph) cudaGraphSetConditional(a.order.handle, ne > kPlacedEvents ? 1u : 0u);
+    if (a.radix.skip) *a.radix.skip = ne <= kPlacedEvents ? 1 : 0;
+    if (a.radix.use_graph) cudaGraphSetConditional(a.radix.handle, ne > kPlacedEvents ? 1u : 0u);
   }
   if ((unsigned long long)ne * nc > kScanWork) {
     for (long long e = gtid(); e < ne; e += gstride()) {

@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(kSortBlock) k_radix_scatter(const unsigned lon
 // ---------------------------------------------------------------------------
 // Order of a step's events. Up to kPlacedEvents the resolve's apply kernel finds
 // each event's place itself; larger lists take the radix passes. Which
-// of the two is known on the device only: the rank kernel sets `order.small`, so
+// of the two is known on the device only: the rank kernel sets `radix.skip`, so
 // that the passes return at once, or, in a step being recorded, the condition of
 // the IF node they sit in, so that they are not launched at all.
 // ---------------------------------------------------------------------------
@@ -144,9 +144,9 @@ bool capturing(cudaStream_t s) {
   return cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusActive;
 }
 
-EventOrder event_order_begin(const SortBuffers& b, cudaStream_t s) {
-  EventOrder o{};
-  o.small = b.small_done;
+RadixGate radix_gate(const SortBuffers& b, cudaStream_t s) {
+  RadixGate o{};
+  o.skip = b.radix_skip;
   cudaStreamCaptureStatus status;
   cudaGraph_t g;
   if (capturing(s) && cudaStreamGetCaptureInfo(s, &status, nullptr, &g, nullptr, nullptr, nullptr) == cudaSuccess &&
@@ -155,7 +155,7 @@ EventOrder event_order_begin(const SortBuffers& b, cudaStream_t s) {
   return o;
 }
 
-cudaError_t if_node(const EventOrder& o, cudaStream_t s, cudaStream_t aux, const std::function<void(cudaStream_t)>& body) {
+cudaError_t if_node(const RadixGate& o, cudaStream_t s, cudaStream_t aux, const std::function<void(cudaStream_t)>& body) {
   if (!o.use_graph) return cudaErrorIllegalState;
   cudaStreamCaptureStatus status;
   cudaGraph_t g;
@@ -185,9 +185,9 @@ void invalidate_capture(cudaStream_t s) {
   cudaGetLastError();
 }
 
-int event_order_end(const SortBuffers& b, const EventOrder& o, const unsigned long long* n_dev, int bits,
+int gated_radix_passes(const SortBuffers& b, const RadixGate& o, const unsigned long long* n_dev, int bits,
                     cudaStream_t s) {
-  if (!capturing(s)) return radix_passes(b, n_dev, 0, bits, s, b.small_done);
+  if (!capturing(s)) return radix_passes(b, n_dev, 0, bits, s, b.radix_skip);
   if (if_node(o, s, b.aux, [&](cudaStream_t t) { radix_passes(b, n_dev, 0, bits, t, nullptr); }) != cudaSuccess)
     invalidate_capture(s);
   return ((bits + 7) / 8) & 1;
@@ -351,7 +351,7 @@ void launch_seg_scatter(long long ncell, long long n_max, const unsigned long lo
 
 void launch_seg_sort(long long ncell, const long long* cell_start, const unsigned long long* n_dev,
                      const unsigned long long* vals, uint32_t* perm, int32_t* big, SegCtl* ctl, cudaStream_t s,
-                     const EventOrder& radix) {
+                     const RadixGate& radix) {
   PIC_LAUNCH(seg_grid(ncell), kSortBlock, 0, s, k_seg_sort)(ncell, cell_start, n_dev, vals, perm, big, ctl);
   PIC_LAUNCH(8 * sm_count(), kSortBlock, 0, s, k_seg_sort_mid)(ncell, cell_start, n_dev, vals, perm, big, ctl);
   PIC_LAUNCH(2 * sm_count(), kSortBlock, 0, s, k_seg_sort_big)(ncell, cell_start, n_dev, vals, perm, big, ctl,

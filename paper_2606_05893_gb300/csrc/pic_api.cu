@@ -410,7 +410,7 @@ void free_instance(Instance* I) {
   dev_free(I->evsort.vb);
   dev_free(I->evsort.hist);
   dev_free(I->evsort.digit_tot);
-  dev_free(I->evsort.small_done);
+  dev_free(I->evsort.radix_skip);
   if (I->evsort.aux) cudaStreamDestroy(I->evsort.aux);
   dev_free(I->csort.ka);
   dev_free(I->csort.kb);
@@ -418,7 +418,7 @@ void free_instance(Instance* I) {
   dev_free(I->csort.vb);
   dev_free(I->csort.hist);
   dev_free(I->csort.digit_tot);
-  dev_free(I->csort.small_done);
+  dev_free(I->csort.radix_skip);
   if (I->csort.aux) cudaStreamDestroy(I->csort.aux);
   free_hit_log(I);
   dev_free(I->cell_count);
@@ -451,7 +451,7 @@ cudaError_t alloc_sort(SortBuffers& b, long long n_max) {
   if ((e = dalloc(&b.vb, n_max))) return e;
   if ((e = dalloc(&b.hist, sort_hist_entries(n_max)))) return e;
   if ((e = dalloc(&b.digit_tot, 256))) return e;
-  if ((e = dalloc(&b.small_done, 1))) return e;
+  if ((e = dalloc(&b.radix_skip, 1))) return e;
   if ((e = cudaStreamCreateWithFlags(&b.aux, cudaStreamNonBlocking))) return e;
   return cudaSuccess;
 }
@@ -820,7 +820,7 @@ pic_status sort_instance(pic_handle* h, Instance* I) {
     exclusive_scan_i32_i64(I->cell_count, I->g.ncell, I->cell_start[s], I->scan_tmp, st);
     launch_seg_scatter(I->g.ncell, I->cap[s], ndev, I->csort.ka, I->csort.va, I->cell_start[s], I->csort.kb,
                        I->csort.vb, st);
-    const EventOrder o = event_order_begin(I->csort, st);
+    const RadixGate o = radix_gate(I->csort, st);
     launch_seg_sort(I->g.ncell, I->cell_start[s], ndev, I->csort.kb, I->csort.vb, I->seg_big, I->seg_ctl, st, o);
     const uint32_t* perm = I->csort.vb;
     // a bucket too large for one block: LSD radix sort of the key (cell, pid)
@@ -1071,9 +1071,9 @@ pic_status step_instance(pic_handle* h, Instance* I) {
     r.sort_vals = I->evsort.va;
     const int rb = std::min(blocks, (I->ev_cap + 255) / 256);
     const bool radix = I->evsort.kb != nullptr;
-    if (radix) r.order = event_order_begin(I->evsort, st);
+    if (radix) r.radix = radix_gate(I->evsort, st);
     launch_resolve_rank(r, rb, st);
-    const int where = radix ? event_order_end(I->evsort, r.order, &I->cnt->ev_sort_n, 40, st) : 0;
+    const int where = radix ? gated_radix_passes(I->evsort, r.radix, &I->cnt->ev_sort_n, 40, st) : 0;
     ApplyArgs<S> ap{};
     ap.g = g;
     ap.cnt = I->cnt;

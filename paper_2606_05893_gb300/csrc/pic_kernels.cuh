@@ -628,9 +628,10 @@ struct PushArgs {
 constexpr unsigned kCountEvents = 128, kPlacedEvents = 1u << 17;
 // events of a run at most; runs at least, as long as they hold 32 or more
 constexpr unsigned kOrderRun = 1024, kOrderBlocks = 152;
-// How the rank kernel tells the radix passes of the events whether they run.
-struct EventOrder {
-  int* small;     // set to 1 for at most kPlacedEvents events, else 0 (nullptr: no radix passes)
+// How a kernel tells the radix passes that follow it whether they run: the rank
+// kernel those of the events, the bucket sort those of the cell sort.
+struct RadixGate {
+  int* skip;      // set to 1 where the passes are not needed, else 0 (nullptr: there are none)
   int use_graph;  // a recorded step: the IF node's condition instead
   cudaGraphConditionalHandle handle;
 };
@@ -646,7 +647,7 @@ struct ResolveArgs {
   int32_t* cand_head;
   unsigned long long* sort_keys;
   uint32_t* sort_vals;
-  EventOrder order;
+  RadixGate radix;
 };
 
 // Buffers and capacities the resolve commit updates (species < 0: absent).
@@ -773,27 +774,27 @@ void launch_seg_scatter(long long ncell, long long n_max, const unsigned long lo
                         unsigned long long* out, uint32_t* perm, cudaStream_t s);
 void launch_seg_sort(long long ncell, const long long* cell_start, const unsigned long long* n_dev,
                      const unsigned long long* vals, uint32_t* perm, int32_t* big, SegCtl* ctl, cudaStream_t s,
-                     const EventOrder& radix);
+                     const RadixGate& radix);
 
 struct SortBuffers {
   unsigned long long *ka, *kb;
   uint32_t *va, *vb;
   uint32_t* hist;      // 256 * nblocks(n_max)
   uint32_t* digit_tot; // 256
-  int* small_done;     // set when the radix passes are not needed (EventOrder)
+  int* radix_skip;     // set when the radix passes are not needed (RadixGate::skip)
   long long n_max;
-  cudaStream_t aux;    // capture stream of the radix passes inside a recorded step (small path)
+  cudaStream_t aux;    // capture stream of the radix passes inside a recorded step
 };
 long long sort_hist_entries(long long n_max);
 bool capturing(cudaStream_t s);
 // An IF node on o's handle at the capture position of s, its body captured on aux.
-cudaError_t if_node(const EventOrder& o, cudaStream_t s, cudaStream_t aux, const std::function<void(cudaStream_t)>& body);
+cudaError_t if_node(const RadixGate& o, cudaStream_t s, cudaStream_t aux, const std::function<void(cudaStream_t)>& body);
 // A half-built node must not be replayed: synchronising a capturing stream is
 // illegal and invalidates the capture, so the recording fails and the instance
 // steps directly from then on.
 void invalidate_capture(cudaStream_t s);
-EventOrder event_order_begin(const SortBuffers& b, cudaStream_t s);
-int event_order_end(const SortBuffers& b, const EventOrder& o, const unsigned long long* n_dev, int bits, cudaStream_t s);
+RadixGate radix_gate(const SortBuffers& b, cudaStream_t s);
+int gated_radix_passes(const SortBuffers& b, const RadixGate& o, const unsigned long long* n_dev, int bits, cudaStream_t s);
 int radix_sort_pairs(const SortBuffers& b, const unsigned long long* n_dev, int bit0, int bit1, cudaStream_t s);
 // exclusive scan of int32 counts[n] into int64 out[n+1] (out[n] = total)
 size_t scan_temp_bytes(long long n);

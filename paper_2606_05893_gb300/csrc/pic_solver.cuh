@@ -1,5 +1,6 @@
-// pic_solver.cuh -- multigrid-preconditioned CG for the scaled 7-point operator,
-// recorded once per instance as a CUDA graph with device-side stopping.
+// pic_solver.cuh -- the Poisson solve of an instance: refinement passes of the direct
+// solver (pic_direct.cuh) or, beyond its sizes, multigrid-preconditioned CG for the
+// scaled 7-point operator, recorded once as a CUDA graph with device-side stopping.
 #pragma once
 
 #include <vector>
