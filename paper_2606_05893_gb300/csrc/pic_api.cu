@@ -799,19 +799,33 @@ McArgs mc_args(Instance* I, int proj) {
   return m;
 }
 
-// a2: sort every species by (cell, pid). Nothing is read back: whether a bucket is
-// too large for one block (the species then takes the radix sort of its whole key)
-// is known on the device, and the radix passes sit in an IF node of a recorded
-// step; a step that is not recorded reads it once per species instead.
+// a2: sort every species by (cell, pid). A recorded step reads nothing back: whether
+// a bucket is too large for one block (the species then takes the radix sort of its
+// whole key) is known on the device, and the radix passes sit in an IF node. A sort
+// that is not recorded (pic_sort_now, timed steps, the first step) reads the counters
+// and, per species, that outcome: empty species are skipped and the radix passes
+// cover only the bits that pids have reached (without the counters 0.20 ms instead of
+// 0.17 for 25 000 particles of two species out of three, 0.59 instead of 0.49 with an overfull cell).
 template <class S>
 pic_status sort_instance(pic_handle* h, Instance* I) {
   cudaStream_t st = I->stream;
   const bool rec = capturing(st);
+  if (!rec) {
+    CK(h, cudaMemcpyAsync(I->host_cnt, I->cnt, sizeof(DevCounters), cudaMemcpyDeviceToHost, st));
+    CK(h, cudaStreamSynchronize(st));
+  }
+  const int pid_bits = rec ? 32 : std::max(1, bits_for(I->host_cnt->next_pid));
   const int cell_bits = bits_for((unsigned long long)I->g.ncell);
-  const int key_bits = std::min(64, cell_bits + 32);
+  const int key_bits = std::min(64, cell_bits + pid_bits);
   for (int s = 0; s < I->nsp; ++s) {
     const int c = I->cur[s];
     unsigned long long* ndev = &I->cnt->n[c][s];
+    if (!rec && I->host_cnt->n[c][s] == 0) {  // nothing to move: offsets all zero; buffers flip as for every species
+      CK(h, cudaMemsetAsync(I->cell_start[s], 0, sizeof(long long) * (I->g.ncell + 1), st));
+      launch_sort_commit(I->cnt, c, s, st);
+      I->cur[s] = c ^ 1;
+      continue;
+    }
     // bucket path: slots, offsets, scatter, per-bucket sort by (pid, index)
     CK(h, cudaMemsetAsync(I->cell_count, 0, sizeof(int32_t) * I->g.ncell, st));
     CK(h, cudaMemsetAsync(I->seg_ctl, 0, sizeof(SegCtl), st));
@@ -827,7 +841,7 @@ pic_status sort_instance(pic_handle* h, Instance* I) {
     SortBuffers b = I->csort;
     b.n_max = I->cap[s];
     auto radix = [&](cudaStream_t t) -> int {
-      launch_cell_keys<S>(I->g, store_of<S>(I, s, c), I->cap[s], ndev, 32, I->csort.ka, I->csort.va, nullptr, t);
+      launch_cell_keys<S>(I->g, store_of<S>(I, s, c), I->cap[s], ndev, pid_bits, I->csort.ka, I->csort.va, nullptr, t);
       return radix_sort_pairs(b, ndev, 0, ((key_bits + 7) / 8) * 8, t);
     };
     if (rec) {
