@@ -468,7 +468,8 @@ uint64_t pic_record_count(void);
  *           electrode planes hold their potentials. Caller-owned.
  *  Iterates until the residual (of the passes the true one b - A phi, of CG the
  *  recursive one) reaches rtol ||b|| or maxit iterations have run (passes: at
- *  most 40); the status follows the true residual, which CG recomputes at the end
+ *  most 40, and one beyond rtol where the residual is still above a tenth of it
+ *  and that tolerance is clear of rounding); the status follows the true residual, which CG recomputes at the end
  *  and which at very tight rtol can sit just above its recursive one. The true
  *  relative residual is reported in *resid_rel and the passes or CG iterations
  *  in *iters (either may be NULL). rho = 0 with both electrodes
@@ -483,7 +484,8 @@ uint64_t pic_record_count(void);
  * vector before reading it); calls that overlap on the GPU -- on different
  * streams or from different host threads on the same device -- race on it.
  * Work runs on cuda_stream; the call reads the outcome back and synchronises
- * that stream after the second and every later pass, or once per CG iteration. */
+ * that stream after the second (rtol below 1e-10: third) and every later pass, or once
+ * per CG iteration. */
 #define PIC_STATIC_MAX_UNKNOWNS (1 << 18)
 pic_status pic_poisson_solve_static(int32_t nx, int32_t ny, int32_t nz, double h, double phi_cathode_V,
                                     double phi_anode_V, const double* rho_dev, double* phi_dev, double rtol,

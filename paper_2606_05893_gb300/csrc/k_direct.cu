@@ -714,7 +714,12 @@ __device__ __forceinline__ bool grid_total2(V v0, V v1, double* part, unsigned* 
 __device__ __forceinline__ void fin_pass(const DirectLoop& d, SolveCtl* c, double rr, long long n) {
   c->rr_true = rr;
   const bool small = c->bb == 0.0 || rr <= c->tol2;
-  const bool done = small || !(rr == rr) || c->it_total >= d.maxit || c->outer >= d.max_outer;
+  bool enough = small;
+  if (d.margin2 < 1.0 && small && c->it_total > 0 && !c->margin_used && rr > d.margin2 * c->tol2 && c->tol2 > c->floor2) {
+    c->margin_used = 1;
+    enough = false;
+  }
+  const bool done = enough || !(rr == rr) || c->it_total >= d.maxit || c->outer >= d.max_outer;
   c->converged = small ? 1 : 0;
   c->more = done ? 0 : 1;
   c->stopped = done ? 1 : 0;

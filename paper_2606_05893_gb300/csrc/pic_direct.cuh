@@ -47,6 +47,8 @@ struct DirectLoop {
   double rtol;
   int maxit, max_outer, use_graph;
   cudaGraphConditionalHandle handle;
+  double margin2 = 1.0;  // below 1: a residual that meets the tolerance (squared) but not margin2 of it takes one
+                         // more pass, unless the tolerance is within SolveCtl::floor2
 };
 constexpr int kDirParts = 1 << 15;  // blocks of a residual launch (two partial sums each)
 

@@ -25,6 +25,8 @@ struct SolveCtl {
   int ax_valid;     // Solver::ax holds A x for the current x
   int stopped;      // the last residual ended the outer loop
   double scale, inv_scale;  // direct solver: brings the FP64 residual to unit size for its FP32 pass
+  double floor2;    // direct solver with a margin: square of what rounding can leave of a residual
+  int margin_used;  // its one more pass has been granted
   int spec_timeout; // a copy of the exact coarse solve did not arrive in time (sticky until reported)
 };
 

@@ -12,7 +12,7 @@
 // planes that solver does not take, by conjugate gradients (right-hand side,
 // residual, search direction, operator image). Measured on 64 x 64 x 63 unknowns
 // to 1e-12: 318 CG iterations of five launches and one wait each, 43.3 ms;
-// direct, 3 passes and two waits, 0.22 ms.
+// direct, 3 passes and one wait, 0.22 ms.
 //
 // The array is a fixed PIC_STATIC_MAX_UNKNOWNS-sized allocation that every GPU
 // loading this library holds until the process exits (4 vectors of 2^18
@@ -28,12 +28,22 @@
 #include "pic_direct.cuh"
 #include "pic_internal.cuh"
 #include "pic_solver.cuh"
+#include "solver_dev.cuh"
 
 namespace pic {
 
 constexpr long long kStaticVec = PIC_STATIC_MAX_UNKNOWNS;
 constexpr int kStaticBlock = 256;
 constexpr int kStaticMaxPasses = 40;  // of the direct solver: each gains several digits, so more gain none
+// What a pass of the direct solver leaves is smooth, and so further from the solution
+// than what CG leaves at the same residual: on 33 grids and densities to 1e-12, 6 errors were
+// larger than CG's, by up to 5.5. A solve that ends above a tenth of its tolerance
+// therefore takes one more pass, unless the tolerance is so close to the rounding of the
+// residual itself (at most about 40 units of 2^-53 |x|) that the pass could
+// lose it again. All 33 errors are at most half of CG's then; 64 x 64 x 64 nodes to
+// 1e-12 take 227 us on average instead of 208.
+constexpr double kStaticMargin2 = 0.01;
+constexpr double kStaticRounding = 64 * 0x1p-53;
 constexpr int kStaticParts = 1024;  // block partials (grid size cap)
 constexpr int kStaticScalars = 32;  // CG: rr, pq, alpha, beta, bb; direct solver: its decision block
 
@@ -95,6 +105,15 @@ __global__ void k_static_rhs(StaticLv L, double h, double phi_c, double phi_a, c
     acc += v * v;
   }
   s_block_partial(acc, part);
+}
+
+// what rounding can leave of a residual, from x.x (the decisions that follow read it)
+__global__ void __launch_bounds__(kStaticBlock) k_static_floor(StaticLv L, const double* __restrict__ x, double* part,
+                                                               SolveCtl* c) {
+  double acc = 0.0, xx;
+  for (long long u = (long long)blockIdx.x * blockDim.x + threadIdx.x; u < L.nu; u += (long long)gridDim.x * blockDim.x)
+    acc += x[u] * x[u];
+  if (grid_total(acc, part, &c->ticket, &xx)) c->floor2 = kStaticRounding * kStaticRounding * xx;
 }
 
 // r = b - A x ; p = r ; part = r.r
@@ -259,17 +278,20 @@ extern "C" pic_status pic_poisson_solve_static(int32_t nx, int32_t ny, int32_t n
     const MgLevel M{nx, ny, nz, nu};
     SolveCtl* ctl = reinterpret_cast<SolveCtl*>(sc);
     double* dpart = q + kStaticVec / 2;
-    const DirectLoop d{rtol, maxit, kStaticMaxPasses, 0, 0};
+    const DirectLoop d{rtol, maxit, kStaticMaxPasses, 0, 0, kStaticMargin2};
     SolveCtl now;
     if ((e = cudaMemsetAsync(ctl, 0, sizeof(SolveCtl), s)) != cudaSuccess) return fail("decision block", e);
     if ((e = D.place(q, p, s)) != cudaSuccess) return fail("tables", e);
     PIC_LAUNCH(G, kStaticBlock, 0, s, k_static_rhs)(L, h, phi_cathode_V, phi_anode_V, rho_dev, phi_dev, b, part);
     D.residual_fp64(true, M, x, b, r, dpart, ctl, d, s);
-    // two passes before the first look at the outcome (passes after the decision to stop return at once)
-    for (int n = 0;; ++n) {
+    // the passes that a solve usually takes before the first look at the outcome (passes after the decision to
+    // stop return at once; to 1e-12, 64 x 64 x 64 nodes, with two and a third after the look 238 us)
+    const int ahead = rtol < 1e-10 ? 3 : 2;
+    for (int n = 1;; ++n) {
       D.apply_fp64(r, x, ctl, s);
+      if (n == 1) PIC_LAUNCH(G, kStaticBlock, 0, s, k_static_floor)(L, x, part, ctl);  // x to 6 digits
       D.residual_fp64(false, M, x, b, r, dpart, ctl, d, s);
-      if (n == 0) continue;
+      if (n < ahead) continue;
       if ((e = cudaGetLastError()) != cudaSuccess) return fail("refinement pass", e);
       if ((e = cudaMemcpyAsync(&now, ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
           (e = cudaStreamSynchronize(s)) != cudaSuccess)

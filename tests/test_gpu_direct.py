@@ -111,3 +111,45 @@ def test_static_solve_on_caller_memory(nx, ny, nz, offset):
     bound = rtol * np.linalg.norm(b) + 12 * np.abs(exact).max() * math.sqrt(b.size) * 2.0 ** -52
     assert np.linalg.norm(phi[1:nz] - exact) <= bound / (4 * math.sin(math.pi / (2 * nz)) ** 2)
     assert np.all(phi[0] == -2.0) and np.all(phi[nz] == phi_a)
+
+
+@pytest.mark.parametrize("nx,ny,nz", [(13, 15, 118), (22, 49, 103), (39, 13, 98), (16, 40, 72), (64, 64, 64), (8, 8, 9)])
+def test_static_solve_keeps_a_margin(nx, ny, nz):
+    """A residual of the direct solver is smooth: it may lie twice as far from the solution as its tolerance
+    says, where CG stayed below. So a solve whose tolerance is clear of rounding ends at a tenth of it, and a
+    guess that already meets the tolerance is kept as it is."""
+    import torch
+    import paper_2606_05893_gb300 as pkg
+    h, rtol = 2.5e-9, 1e-12
+    phi_a = 9.375e9 * nz * h
+    rng = np.random.default_rng(nx * ny * nz)
+    z, y, x = np.meshgrid(np.arange(nz + 1) / nz, np.arange(ny) / ny - 0.5, np.arange(nx) / nx - 0.5, indexing="ij")
+    shape = np.exp(-(x * x + y * y) / 0.08) * (0.3 + np.exp(-4 * z))
+    for _ in range(6):
+        rho = 0.2 * 9.375e9 * EPS0 / (nz * h) * shape * (0.5 + rng.random() + 0.7 * rng.standard_normal(shape.shape))
+        rho_dev, phi_dev = torch.from_numpy(rho).cuda(), torch.zeros(rho.shape, dtype=torch.float64, device="cuda")
+        args = (nx, ny, nz, h, -2.0, phi_a, rho_dev.data_ptr(), phi_dev.data_ptr())
+        st, iters, rel = pkg.pic_poisson_solve_static(*args, rtol, 100000)
+        assert st == pkg.PIC_OK and rel <= 0.1 * rtol
+        phi = phi_dev.clone()
+        st, iters, again = pkg.pic_poisson_solve_static(*args, rtol, 100000)
+        assert st == pkg.PIC_OK and iters == 0 and again == rel and torch.equal(phi, phi_dev)
+        phi_dev.zero_()
+        st, iters, _ = pkg.pic_poisson_solve_static(*args, rtol, 1)
+        assert iters == 1
+
+
+def test_static_solve_near_rounding():
+    """A smooth density between grounded electrodes: |x| is 1500 |b|, so the residual's rounding comes up to
+    common tolerances. Whatever is reached is reported, and a looser tolerance is never missed."""
+    import torch
+    import paper_2606_05893_gb300 as pkg
+    nx, ny, nz = 12, 10, 120
+    rho = torch.full((nz + 1, ny, nx), 2e6, dtype=torch.float64, device="cuda")
+    reached = []
+    for rtol in 10.0 ** -np.arange(6.0, 14.0, 0.25):
+        phi = torch.zeros_like(rho)
+        st, iters, rel = pkg.pic_poisson_solve_static(nx, ny, nz, 2.5e-9, 0.0, 0.0, rho.data_ptr(), phi.data_ptr(), rtol, 1000)
+        assert (st == pkg.PIC_OK) == (rel <= rtol) and iters <= 40
+        reached.append(st == pkg.PIC_OK)
+    assert reached == sorted(reached, reverse=True) and sum(reached) >= 20
