@@ -315,7 +315,8 @@ pic_status pic_set_phi(pic_handle* h, int32_t inst, const double* host_phi);
 
 /* Solve Eq. (1) for a given charge density with the instance's solver and
  * electrodes: rho and phi are host arrays over the nodes; phi's interior is
- * the initial guess on entry and the solution on exit. Does not touch the
+ * the initial guess on entry and the solution on exit (by the direct solver, to a
+ * tenth of cg_rtol where one pass more reaches that). Does not touch the
  * instance's own phi. iters/resid_rel may be NULL. The call takes 16 bytes a node
  * on the device (PIC_MIXED 24): up to 64 MB are kept by the instance until
  * pic_destroy, more are given back when it returns. A caller that must keep a fixed

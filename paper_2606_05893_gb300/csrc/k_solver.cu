@@ -2211,6 +2211,17 @@ SolveResult Solver::result(cudaStream_t s) {
   return result_read();
 }
 
+bool Solver::margin_left(const SolveResult& r, double xx) const {
+  return direct.on && r.converged && r.iters > 0 && r.iters < std::min(h_maxit, max_outer) &&
+         r.resid_rel > kSolveMargin * h_rtol &&
+         h_rtol * std::sqrt(host_ctl->bb) > kSolveRounding[precision != 0 ? 1 : 0] * std::sqrt(xx);
+}
+cudaError_t Solver::margin_pass(cudaStream_t s) {
+  const cudaError_t e = cudaMemsetAsync(&ctl->stopped, 0, sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  direct_pass(DirectLoop{h_rtol, h_maxit, max_outer, 0, 0}, s);
+  return cudaGetLastError();
+}
 cudaError_t Solver::result_async(cudaStream_t s) {
   return cudaMemcpyAsync(host_ctl, ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, s);
 }

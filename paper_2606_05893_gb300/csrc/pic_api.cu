@@ -2127,9 +2127,20 @@ pic_status pic_solve(pic_handle* h, int32_t inst, const double* rho, double* phi
     launch_rhs(g, I->cnt, drho, nullptr, I->solver.b, s);
   }
   CK(h, I->solver.launch(s));
-  if (I->mixed) CK(h, I->solver.phi64_from_ff(I->phi + g.nplane, s));
-  CK(h, cudaMemcpyAsync(phi, I->phi, sizeof(double) * g.nnode, cudaMemcpyDeviceToHost, s));
-  SolveResult r = I->solver.result(s);
+  SolveResult r;
+  for (bool more = false;;) {
+    if (I->mixed) CK(h, I->solver.phi64_from_ff(I->phi + g.nplane, s));
+    CK(h, cudaMemcpyAsync(phi, I->phi, sizeof(double) * g.nnode, cudaMemcpyDeviceToHost, s));
+    r = I->solver.result(s);
+    // a residual close to the tolerance: one more pass (at 1e-12, 3 of 27 solves were further from the 64-bit
+    // solution than MG-PCG's, by up to 3.9; at 1e-8 and 1e-13 none ends there)
+    if (more || !I->solver.margin_left(r, 0.0)) break;
+    double xx = (double)nu * std::max(g.phi_c * g.phi_c, g.phi_a * g.phi_a);
+    for (long long n = g.nplane; n < g.nplane + nu; ++n) xx += phi[n] * phi[n];
+    if (!I->solver.margin_left(r, xx)) break;
+    CK(h, I->solver.margin_pass(s));
+    more = true;
+  }
   CK(h, cudaMemcpyAsync(I->phi, save_phi, sizeof(double) * g.nnode, cudaMemcpyDeviceToDevice, s));
   if (I->mixed) {
     CK(h, cudaMemcpyAsync(I->phi32, save32, sizeof(float) * g.nnode, cudaMemcpyDeviceToDevice, s));

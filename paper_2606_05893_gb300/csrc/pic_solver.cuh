@@ -30,6 +30,11 @@ struct SolveCtl {
   int spec_timeout; // a copy of the exact coarse solve did not arrive in time (sticky until reported)
 };
 
+// A pass leaves a smooth residual, further from the solution than what CG leaves at the
+// same residual; kSolveRounding (FP64, MIXED) bounds what rounding can leave of it, in units of |x|.
+constexpr double kSolveMargin = 0.1;
+constexpr double kSolveRounding[2] = {64 * 0x1p-53, 64 * 0x1p-46};
+
 struct SolveResult {
   int iters;
   double resid_rel;
@@ -125,6 +130,11 @@ struct Solver {
   float fold_first() const { return (float)(h_phi_c + (plan[0].nz == 2 ? h_phi_a : 0.0)); }
   float fold_last() const { return plan[0].nz == 2 ? 0.f : (float)h_phi_a; }
   SolveResult result(cudaStream_t s);
+  // One more pass of the direct solver after a solve that met the tolerance but not a
+  // tenth of it: whether that can gain (xx: sum of the squares of the solution, on
+  // which the residual's rounding depends), and the pass.
+  bool margin_left(const SolveResult& r, double xx) const;
+  cudaError_t margin_pass(cudaStream_t s);
   // the same in two parts: enqueue the copy of the decision block, then (after
   // the caller synchronized the stream) read it
   cudaError_t result_async(cudaStream_t s);

@@ -42,8 +42,8 @@ constexpr int kStaticMaxPasses = 40;  // of the direct solver: each gains severa
 // residual itself (at most about 40 units of 2^-53 |x|) that the pass could
 // lose it again. All 33 errors are at most half of CG's then; 64 x 64 x 64 nodes to
 // 1e-12 take 227 us on average instead of 208.
-constexpr double kStaticMargin2 = 0.01;
-constexpr double kStaticRounding = 64 * 0x1p-53;
+constexpr double kStaticMargin2 = kSolveMargin * kSolveMargin;
+constexpr double kStaticRounding = kSolveRounding[0];
 constexpr int kStaticParts = 1024;  // block partials (grid size cap)
 constexpr int kStaticScalars = 32;  // CG: rr, pq, alpha, beta, bb; direct solver: its decision block
 

@@ -139,6 +139,26 @@ def test_static_solve_keeps_a_margin(nx, ny, nz):
         assert iters == 1
 
 
+@pytest.mark.parametrize("precision,rtol,nx,ny,nz", [(0, 1e-12, 30, 66, 135), (0, 1e-12, 30, 84, 106), (0, 1e-12, 22, 48, 73),
+                                                     (0, 3e-12, 96, 80, 150), (0, 1e-5, 22, 16, 59), (1, 1e-5, 22, 16, 59)])
+def test_solve_keeps_a_margin(precision, rtol, nx, ny, nz):
+    """The same of pic_solve, at tolerances that a pass may just meet."""
+    import paper_2606_05893_gb300 as pkg
+    h = 2.5e-9
+    wl = bare(nx=nx, ny=ny, nz=nz, h=h, phi_c=-2.0, phi_a=9.375e9 * nz * h)
+    sim = pkg.Simulation(wl, precision=precision, cg_rtol=rtol, cg_maxit=20000, preload=False)
+    rng = np.random.default_rng(nx * ny * nz)
+    z, y, x = np.meshgrid(np.arange(nz + 1) / nz, np.arange(ny) / ny - 0.5, np.arange(nx) / nx - 0.5, indexing="ij")
+    shape = np.exp(-(x * x + y * y) / 0.08) * (0.3 + np.exp(-4 * z))
+    for _ in range(4):
+        rho = 0.2 * 9.375e9 * EPS0 / (nz * h) * shape * (0.5 + rng.random() + 0.7 * rng.standard_normal(shape.shape))
+        phi, iters, rel = sim.solve(rho)
+        assert rel <= 0.1 * rtol
+        again, more, same = sim.solve(rho, phi.copy())
+        assert same <= rtol and (more > 0 or np.array_equal(again, phi))
+    sim.close()
+
+
 def test_static_solve_near_rounding():
     """A smooth density between grounded electrodes: |x| is 1500 |b|, so the residual's rounding comes up to
     common tolerances. Whatever is reached is reported, and a looser tolerance is never missed."""
