@@ -448,7 +448,10 @@ uint64_t pic_kernel_count(void);
 
 /* Steps recorded as graphs in this process so far (one instance's step or a whole
  * ensemble's). Recording costs as much as many steps: a run that keeps its
- * parameters records its patterns once and then only replays them. */
+ * parameters records its patterns once and then only replays them. The driver keeps
+ * about 0.3 MB of device memory for an instance's step in a recorded pattern: up to 8
+ * patterns an instance, and for several instances up to 64 of a handle (8 from 64
+ * instances on). */
 uint64_t pic_record_count(void);
 
 /* ---- solve without allocating ----------------------------------------------

@@ -1346,7 +1346,8 @@ pic_status run_step(pic_handle* h, Instance* I) {
 // recording: one interval of 20 198 and 199, intervals 20/40 214 and 275, 5/10 263
 // and 828, 5/10/20/40 359 and 669.
 constexpr unsigned long long kEnsStale = 4096;
-// graphs a handle holds: 64 for a few instances, 8 from 64 on (a graph grows with them)
+// graphs a handle holds: 64 for a few instances, 8 from 64 on (a graph takes about 0.3 MB
+// of device memory per instance: 130 MB for 48 patterns of 8 instances)
 size_t ens_capacity(const pic_handle* h) { return std::max<size_t>(8, std::min<size_t>(64, 512 / h->inst.size())); }
 
 bool ensemble_recordable(const pic_handle* h) {

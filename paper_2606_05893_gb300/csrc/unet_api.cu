@@ -691,7 +691,7 @@ static void wgrad_on(unet_handle* n, int l, const Tensor& s0, const Tensor* s1, 
 
 // Weight gradients run beside the data gradients, which they do not feed: on the
 // side stream, each after the output gradient that the main stream has written
-// by then (forward and backward at 64x32x32: 1099 us one after the other, 946 us so).
+// by then (forward and backward at 64x32x32: 1099 us one after the other, 940 us so).
 // The backward pass joins the side stream at its end.
 static void wgrad(unet_handle* n, int l, const Tensor& s0, const Tensor* s1, const Tensor& dz, cudaStream_t st) {
   cudaEventRecord(n->ready, st);
