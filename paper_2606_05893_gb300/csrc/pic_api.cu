@@ -2165,9 +2165,12 @@ pic_status pic_sort_now(pic_handle* h, int32_t inst) {
   pic_status st = check(h, inst);
   if (st != PIC_OK) return st;
   Instance* I = h->inst[inst];
+  // an instance of several sorts on its own stream: after the uploads queued on the
+  // handle's, and done before anything that is queued there next
+  if (I->stream != h->stream) CK(h, cudaStreamSynchronize(h->stream));
   st = I->mixed ? sort_instance<StoreMx>(h, I) : sort_instance<Store64>(h, I);
   if (st != PIC_OK) return st;
-  CK(h, cudaStreamSynchronize(h->stream));
+  CK(h, cudaStreamSynchronize(I->stream));
   return PIC_OK;
 }
 
